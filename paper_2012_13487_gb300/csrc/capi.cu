@@ -16,6 +16,7 @@
 #include "host_setup.h"
 #include "krylov.h"
 #include "stage_dispatch.h"
+#include "transfer.h"
 
 namespace {
 // NVTX range over one library call (shown by Nsight timelines; a no-op when no
@@ -121,79 +122,6 @@ __global__ void equilibrium_kernel(double* out, const double* vel64, const int32
   }
 }
 
-// canonical FP64 or FP32 [K][Np][Q] -> internal storage [K][Np][Qp], canonical
-// velocity c at internal index iperm[c], the padding velocities zero (one CTA
-// per element; the deviation forms compute their scale and codes in FP64)
-template <class ST, typename TIn>
-__global__ void encode_kernel(const TIn* in, void* out, float* scale, const double* vel64, const int32_t* iperm,
-                              int Np, int Q, int Qp) {
-  using S = typename ST::S;
-  const int64_t k = blockIdx.x;
-  const TIn* src = in + k * Np * Q;
-  S* dst = static_cast<S*>(out) + k * Np * Qp;
-  const double* w = vel64 + 2 * Qp;
-  if constexpr (ST::dev) {
-    __shared__ float red[32];
-    float m = 0.f;
-    for (int j = threadIdx.x; j < Np * Q; j += blockDim.x) {
-      const int i = iperm[j % Q];
-      if (w[i] > 0) m = fmaxf(m, float(fabs((double(src[j]) - w[i]) / w[i])));
-    }
-    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float mm = 0.f;
-      for (int j = 0; j < int(blockDim.x + 31) / 32; ++j) mm = fmaxf(mm, red[j]);
-      float sc = 1.0f;
-      if (mm > 0.f) {
-        int e2;
-        frexpf(mm, &e2);
-        sc = ldexpf(1.0f, e2 - ST::qmax_log2);
-      }
-      red[0] = sc;
-      scale[k] = sc;
-    }
-    __syncthreads();
-    const double inv_s = 1.0 / double(red[0]);
-    for (int j = threadIdx.x; j < Np * Q; j += blockDim.x) {
-      const int n = j / Q, i = iperm[j % Q];
-      float q = 0.f;
-      if (w[i] > 0) q = float((double(src[j]) - w[i]) / w[i] * inv_s);
-      dst[n * Qp + i] = ST::from_r(q);
-    }
-  } else {
-    (void)scale;
-    (void)w;
-    for (int j = threadIdx.x; j < Np * Q; j += blockDim.x) dst[(j / Q) * Qp + iperm[j % Q]] = S(double(src[j]));
-  }
-  for (int j = threadIdx.x; j < Np * (Qp - Q); j += blockDim.x)
-    dst[(j / (Qp - Q)) * Qp + Q + j % (Qp - Q)] = S(0.0f);
-}
-
-template <class ST>
-__device__ __forceinline__ double decode64(const typename ST::S v, double w, double s) {
-  if constexpr (ST::dev) return w + w * s * double(ST::to_r(v));
-  else return double(v);
-}
-
-// internal state -> canonical FP64 (canonical velocity c from internal index iperm[c])
-template <class ST>
-__global__ void decode_kernel(const void* in, const float* scale, double* out, const double* vel64,
-                              const int32_t* iperm, int64_t K, int Np, int Q, int Qp) {
-  using S = typename ST::S;
-  const int64_t n = K * Np * Q;
-  const double* w = vel64 + 2 * Qp;
-  for (int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; idx < n;
-       idx += int64_t(gridDim.x) * blockDim.x) {
-    const int i = iperm[int(idx % Q)];
-    const int64_t kn = idx / Q;
-    const int64_t k = kn / Np;
-    const double s = ST::dev ? double(scale[k]) : 0.0;
-    out[idx] = decode64<ST>(static_cast<const S*>(in)[kn * Qp + i], w[i], s);
-  }
-}
-
 template <typename R>
 __global__ void decode_residual_kernel(const R* in, const int32_t* iperm, double* out, int64_t K, int Np, int Q,
                                        int Qp) {
@@ -203,76 +131,6 @@ __global__ void decode_residual_kernel(const R* in, const int32_t* iperm, double
     const int i = iperm[int(idx % Q)];
     const int64_t kn = idx / Q;
     out[idx] = double(in[kn * Qp + i]);
-  }
-}
-
-// One value of a node row in the state's compute precision R (FP64 state:
-// double; FP32 and 16-bit states: float, f = w + (w s) q for the latter).
-template <class ST>
-__device__ __forceinline__ typename ST::R decode_r(const typename ST::S v, typename ST::R w, typename ST::R ws) {
-  if constexpr (ST::dev) return fmaf(ws, ST::to_r(v), w);
-  else return typename ST::R(v);
-}
-
-// Sums over one node row: one warp per node, lanes on consecutive velocities
-// (coalesced), partial sums and the warp reduction in the state's compute
-// precision R (FP64 for the FP64 state), returned as FP64.
-template <class ST>
-__device__ __forceinline__ void node_sums(const typename ST::S* row, const typename ST::R* vel, int Qp,
-                                          typename ST::R s, int lane, typename ST::R& d0, typename ST::R& d1,
-                                          typename ST::R& d2) {
-  using R = typename ST::R;
-  using S = typename ST::S;
-  constexpr int V = 16 / sizeof(S);  // values per 16-byte load (Qp is a multiple of 8)
-  R m0 = 0, m1 = 0, m2 = 0;
-  // 16-byte loads, several in flight per lane: one 128-byte load per warp at a
-  // time leaves HBM latency-bound
-#pragma unroll 4
-  for (int i = lane * V; i < Qp; i += 32 * V) {
-    __align__(16) S q[V];
-    *reinterpret_cast<uint4*>(q) = *reinterpret_cast<const uint4*>(row + i);
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-      const R w = vel[kVelW * Qp + i + j];
-      const R f = decode_r<ST>(q[j], w, w * s);
-      m0 += f;
-      m1 = fma(vel[kVelEx * Qp + i + j], f, m1);
-      m2 = fma(vel[kVelEy * Qp + i + j], f, m2);
-    }
-  }
-  // the warp reduction in R as well (FP64 throughput is low on this part; for
-  // the FP32 and 16-bit states the lane sums are FP32 already)
-  for (int off = 16; off > 0; off >>= 1) {
-    m0 += __shfl_xor_sync(0xffffffffu, m0, off);
-    m1 += __shfl_xor_sync(0xffffffffu, m1, off);
-    m2 += __shfl_xor_sync(0xffffffffu, m2, off);
-  }
-  d0 = m0;
-  d1 = m1;
-  d2 = m2;
-}
-
-// node moments rho, u_x, u_y (FP64 outputs), one warp per node
-template <class ST>
-__global__ void moments_kernel(const void* in, const float* scale, const typename ST::R* vel, int64_t K, int Np,
-                               int Qp, double* rho, double* ux, double* uy) {
-  using S = typename ST::S;
-  using R = typename ST::R;
-  const int lane = threadIdx.x & 31;
-  const int64_t nodes = K * Np;
-  const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
-  for (int64_t kn = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5; kn < nodes; kn += nw) {
-    const S* row = static_cast<const S*>(in) + kn * Qp;
-    const R s = ST::dev ? R(scale[kn / Np]) : R(0);
-    R m0, m1, m2;
-    node_sums<ST>(row, vel, Qp, s, lane, m0, m1, m2);
-    if (lane == 0) {
-      // the quotients in R too: FP64 division is slow here, and the FP32 and
-      // 16-bit states carry FP32 precision
-      rho[kn] = double(m0);
-      ux[kn] = double(m1 / m0);
-      uy[kn] = double(m2 / m0);
-    }
   }
 }
 
@@ -1221,6 +1079,26 @@ int timeout_status(int word) {
               : FEDBM_OK;
 }
 
+// What the transfer kernels need to know of case c's slice of its group.
+transfer::Shape layout_of(const Batch& b, const Group& g, const Case& cs) {
+  transfer::Shape t;
+  t.store = g.store;
+  t.K = cs.K;
+  t.Np = g.Np;
+  t.Q = g.Q;
+  t.Qp = g.Qp;
+  t.vel64 = g.vel64;
+  t.iperm = g.iperm;
+  t.device = b.device;
+  return t;
+}
+const void* state_of(const Group& g, int cur, const Case& cs) {
+  return static_cast<const unsigned char*>(g.f[cur]) + size_t(cs.k_off) * g.Np * g.Qp * store_bytes(g.store);
+}
+const float* scale_of(const Group& g, int cur, const Case& cs) {
+  return g.scale[cur] ? g.scale[cur] + cs.k_off : nullptr;
+}
+
 // canonical FP64 (device) -> internal state of case c
 template <typename TIn>
 int encode_case(Batch& b, int c, const TIn* src) {
@@ -1228,14 +1106,8 @@ int encode_case(Batch& b, int c, const TIn* src) {
   const Group& g = b.groups[cs.group];
   const size_t off = size_t(cs.k_off) * g.Np * g.Qp;
   float* sc = g.scale[b.cur] ? g.scale[b.cur] + cs.k_off : nullptr;
-  const int blk = 256;
-  switch (g.store) {
-    case kStoreF64: encode_kernel<StoreF64, TIn><<<int(cs.K), blk, 0, b.stream>>>(src, static_cast<double*>(g.f[b.cur]) + off, nullptr, g.vel64, g.iperm, g.Np, g.Q, g.Qp); break;
-    case kStoreF32: encode_kernel<StoreF32, TIn><<<int(cs.K), blk, 0, b.stream>>>(src, static_cast<float*>(g.f[b.cur]) + off, nullptr, g.vel64, g.iperm, g.Np, g.Q, g.Qp); break;
-    case kStoreBF16: encode_kernel<StoreBF16, TIn><<<int(cs.K), blk, 0, b.stream>>>(src, static_cast<__nv_bfloat16*>(g.f[b.cur]) + off, sc, g.vel64, g.iperm, g.Np, g.Q, g.Qp); break;
-    default: encode_kernel<StoreF16, TIn><<<int(cs.K), blk, 0, b.stream>>>(src, static_cast<__half*>(g.f[b.cur]) + off, sc, g.vel64, g.iperm, g.Np, g.Q, g.Qp); break;
-  }
-  FEDBM_CK(cudaGetLastError());
+  void* dst = static_cast<unsigned char*>(g.f[b.cur]) + off * store_bytes(g.store);
+  FEDBM_CK(transfer::encode(layout_of(b, g, cs), src, dst, sc, b.stream));
   // a new state starts with a clear stage-kernel timeout word (and the
   // stochastic-rounding draws from step 0)
   FEDBM_CK(cudaMemsetAsync(g.flag + 1, 0, sizeof(int), b.stream));
@@ -1278,15 +1150,6 @@ int set_equilibrium(Batch& b, int c, double rho0, double ux0, double uy0, double
   return encode_case(b, c, static_cast<const double*>(b.staging));
 }
 
-template <class ST>
-void launch_decode(const Group& g, int cur, const Case& cs, double* dst, cudaStream_t st) {
-  using S = typename ST::S;
-  const int64_t n = cs.K * g.Np * g.Q;
-  const S* in = static_cast<const S*>(g.f[cur]) + size_t(cs.k_off) * g.Np * g.Qp;
-  const float* sc = g.scale[cur] ? g.scale[cur] + cs.k_off : nullptr;
-  decode_kernel<ST><<<grid_for(n, 256), 256, 0, st>>>(in, sc, dst, g.vel64, g.iperm, cs.K, g.Np, g.Q, g.Qp);
-}
-
 int get_state(Batch& b, int c, double* f, int on_device) {
   NvtxRange nvtx("fedbm get_state");
   if (!f) return fail(FEDBM_EINVAL, "null output");
@@ -1299,13 +1162,7 @@ int get_state(Batch& b, int c, double* f, int on_device) {
     if (rc) return rc;
     dst = b.staging;
   }
-  switch (g.store) {
-    case kStoreF64: launch_decode<StoreF64>(g, b.cur, cs, dst, b.stream); break;
-    case kStoreF32: launch_decode<StoreF32>(g, b.cur, cs, dst, b.stream); break;
-    case kStoreBF16: launch_decode<StoreBF16>(g, b.cur, cs, dst, b.stream); break;
-    default: launch_decode<StoreF16>(g, b.cur, cs, dst, b.stream); break;
-  }
-  FEDBM_CK(cudaGetLastError());
+  FEDBM_CK(transfer::decode(layout_of(b, g, cs), state_of(g, b.cur, cs), scale_of(g, b.cur, cs), dst, b.stream));
   if (!on_device) {
     int word = 0;
     FEDBM_CK(cudaMemcpyAsync(f, dst, n * sizeof(double), cudaMemcpyDeviceToHost, b.stream));
@@ -1341,17 +1198,6 @@ int get_residual(Batch& b, int c, double* r, int on_device) {
   return FEDBM_OK;
 }
 
-template <class ST>
-void launch_moments(const Group& g, int cur, const Case& cs, double* r, double* x, double* y, cudaStream_t st) {
-  using S = typename ST::S;
-  const int64_t nodes = cs.K * g.Np;
-  const S* in = static_cast<const S*>(g.f[cur]) + size_t(cs.k_off) * g.Np * g.Qp;
-  const float* sc = g.scale[cur] ? g.scale[cur] + cs.k_off : nullptr;
-  using R = typename ST::R;
-  moments_kernel<ST><<<grid_for(nodes * 32, 256), 256, 0, st>>>(in, sc, static_cast<const R*>(g.vel), cs.K, g.Np,
-                                                                  g.Qp, r, x, y);
-}
-
 int get_moments(Batch& b, int c, double* rho, double* ux, double* uy, int on_device) {
   NvtxRange nvtx("fedbm get_moments");
   const Case& cs = b.cases[c];
@@ -1372,13 +1218,8 @@ int get_moments(Batch& b, int c, double* rho, double* ux, double* uy, int on_dev
   } else if (!rho || !ux || !uy) {
     return fail(FEDBM_EINVAL, "device moments need three output pointers");
   }
-  switch (g.store) {
-    case kStoreF64: launch_moments<StoreF64>(g, b.cur, cs, dr, dx, dy, b.stream); break;
-    case kStoreF32: launch_moments<StoreF32>(g, b.cur, cs, dr, dx, dy, b.stream); break;
-    case kStoreBF16: launch_moments<StoreBF16>(g, b.cur, cs, dr, dx, dy, b.stream); break;
-    default: launch_moments<StoreF16>(g, b.cur, cs, dr, dx, dy, b.stream); break;
-  }
-  FEDBM_CK(cudaGetLastError());
+  FEDBM_CK(transfer::moments(layout_of(b, g, cs), state_of(g, b.cur, cs), scale_of(g, b.cur, cs), g.vel, dr, dx, dy,
+                             b.stream));
   if (!on_device) {
     const size_t bytes = size_t(nodes) * sizeof(double);
     if (rho) FEDBM_CK(cudaMemcpyAsync(rho, dr, bytes, cudaMemcpyDeviceToHost, b.stream));

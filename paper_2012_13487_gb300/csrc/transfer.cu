@@ -1,0 +1,505 @@
+// Encode, decode and node-moment kernels (see transfer.h).
+#include "transfer.h"
+
+#include <algorithm>
+#include <type_traits>
+
+#include "device_common.cuh"
+
+namespace fedbm {
+namespace transfer {
+namespace {
+
+constexpr int kThreads = 256;
+constexpr size_t kSmemCap = 227 * 1024 - 64;  // dynamic; the encode kernel has 32 bytes of its own
+// Rows of an element are staged through at most about this much shared memory
+// per CTA, so that several CTAs share an SM and one's loads overlap another's
+// stores.
+constexpr size_t kStageBytes = 48 * 1024;
+
+// FP32 -> FP64 with integer operations for zeros and normal numbers: the
+// conversion instruction to FP64 runs at the part's low FP64 rate (two lanes
+// per clock and SM), which bounded the FP32 decode at 31M values (90 us
+// against 56 us for its bytes).
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), e = u & 0x7f800000u, m = u & 0x7fffffffu;
+  if (m != 0u && (e == 0u || e == 0x7f800000u)) return double(x);  // denormal, infinity, NaN
+  const uint32_t hi = (u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
+  return __hiloint2double(int(hi), int(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// Work split shared by encode and decode: a group of G threads (a warp where
+// an element has at most kWarpValues values, else the whole CTA) handles one
+// element at a time, kRows rows of it per pass through shared memory.
+constexpr int kWarpValues = 1536;
+
+struct Split {
+  bool warp;       // groups are warps
+  int rows;        // rows of an element staged at once
+  size_t tables;   // bytes of the velocity tables in front of the buffers
+  size_t smem;
+  int grid;
+};
+
+inline size_t up16(size_t b) { return (b + 15) / 16 * 16; }
+
+Split split_for(const Shape& sh, size_t table_bytes_per_q, size_t value_bytes) {
+  Split s;
+  s.warp = sh.Np * sh.Qp <= kWarpValues;
+  s.tables = up16(table_bytes_per_q * size_t(sh.Q) + 4 * size_t(sh.Qp));
+  const size_t row = size_t(sh.Qp) * value_bytes;
+  const int groups = s.warp ? kThreads / 32 : 1;
+  s.rows = s.warp ? sh.Np : std::max(1, std::min(sh.Np, int(kStageBytes / row)));
+  s.smem = s.tables + size_t(groups) * s.rows * row;
+  int nsm = 152, smem_sm = 228 * 1024;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, sh.device);
+  cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, sh.device);
+  const int per_sm = std::max(1, std::min(8, int(size_t(smem_sm) / (s.smem + 1024))));
+  const int64_t tiles = s.warp ? (sh.K + groups - 1) / groups : sh.K;
+  s.grid = int(std::max<int64_t>(1, std::min<int64_t>(tiles, int64_t(nsm) * per_sm)));
+  return s;
+}
+
+template <bool kWarp>
+__device__ __forceinline__ void group_sync() {
+  if constexpr (kWarp) __syncwarp();
+  else __syncthreads();
+}
+
+// Canonical positions j = row * Q + c of one group in steps of G, with the
+// row and velocity kept without a division per value.
+struct Walk {
+  int c, row, dc, drow, Q;
+  __device__ Walk(int start, int G, int Q_) : Q(Q_) {
+    row = start / Q;
+    c = start - row * Q;
+    drow = G / Q;
+    dc = G - drow * Q;
+  }
+  __device__ void next() {
+    row += drow;
+    c += dc;
+    if (c >= Q) {
+      c -= Q;
+      ++row;
+    }
+  }
+};
+
+// f - w relative to w, in FP32 with w = wh + wl: x - wh is exact where x is
+// within a factor of two of w, so the difference keeps FP32's relative
+// precision however small the deviation, without FP64 arithmetic per value.
+// An FP64 x that FP32 holds exactly takes the same path, so that an FP32 value
+// and the same value given in FP64 give the same bits; any other is subtracted
+// in FP64.  Weights below FP32's normal range take the FP64 quotient.
+struct DevTable {
+  const float *wh, *wl, *iw;  // canonical order; iw < 0: tiny weight, 0: weight 0
+};
+__device__ __forceinline__ float difference(float x, const DevTable& t, int c) {
+  return (x - t.wh[c]) - t.wl[c];
+}
+template <typename TIn>
+__device__ __forceinline__ float deviation(TIn x, const DevTable& t, int c, const double* w64, const int* perm) {
+  const float iw = t.iw[c];
+  if (iw <= 0.f) {
+    if (iw == 0.f) return 0.f;
+    const double w = w64[perm[c]];
+    return float((double(x) - w) / w);
+  }
+  if constexpr (sizeof(TIn) == 8) {
+    const float xh = float(x);
+    if (__double_as_longlong(widen(xh)) != __double_as_longlong(x)) return float(x - w64[perm[c]]) * iw;
+    return difference(xh, t, c) * iw;
+  } else {
+    return difference(x, t, c) * iw;
+  }
+}
+
+// Encode: the caller's rows are read along the canonical order (consecutive
+// lanes, consecutive addresses), scattered into shared memory by the internal
+// velocity order, and written from there as 16-byte vectors of the internal
+// row.  Deviation forms keep (f - w)/w of the whole element in shared memory
+// between finding the element's largest deviation and writing the codes, so
+// the input is read once and only one quotient is formed per value.  Before,
+// with two FP64 divisions per value, scattered 2- and 4-byte stores and an
+// integer division per value (GB300, ncu): BF16 from FP32 input 15.3 ms at 335M
+// values (1,024 velocities), 1.45 ms at 31M (256) and 2.44 ms at 44M (16), FP32
+// from FP32 71 us at 31M; now 1.18 ms, 79 us, 122 us and 43 us.
+template <class ST, typename TIn, bool kWarp>
+__global__ void __launch_bounds__(kThreads) encode_kernel(const TIn* __restrict__ in, void* out, float* scale,
+                                                          const double* __restrict__ vel64,
+                                                          const int32_t* __restrict__ iperm, int64_t K, int Np,
+                                                          int Q, int Qp, int rows, int table_bytes) {
+  using S = typename ST::S;
+  using T = std::conditional_t<ST::dev, float, S>;  // staged values
+  constexpr int V = 16 / int(sizeof(S));
+  extern __shared__ __align__(16) unsigned char smem[];
+  int* perm = reinterpret_cast<int*>(smem);
+  float* tab = reinterpret_cast<float*>(perm + Qp);
+  DevTable dt{tab, tab + Q, tab + 2 * Q};
+  const double* w64 = vel64 + 2 * Qp;
+  for (int c = threadIdx.x; c < Q; c += kThreads) {
+    const int i = iperm[c];
+    perm[c] = i;
+    if constexpr (ST::dev) {
+      const double w = w64[i];
+      const float wh = float(w);
+      tab[c] = wh;
+      tab[Q + c] = float(w - double(wh));
+      tab[2 * Q + c] = !(w > 0) ? 0.f : w < 1e-30 ? -1.f : float(1.0 / w);
+    }
+  }
+  const int G = kWarp ? 32 : kThreads;
+  const int grp = kWarp ? threadIdx.x / 32 : 0, lane = kWarp ? threadIdx.x % 32 : threadIdx.x;
+  const int ngroups = kWarp ? kThreads / 32 : 1;
+  T* buf = reinterpret_cast<T*>(smem + table_bytes) + size_t(grp) * rows * Qp;
+  for (int v = lane; v < rows * Qp; v += G) buf[v] = T(0);  // the padding velocities stay zero
+  __shared__ float red[kThreads / 32];
+  __syncthreads();
+
+  for (int64_t k = blockIdx.x * int64_t(ngroups) + grp; k < K; k += int64_t(gridDim.x) * ngroups) {
+    const TIn* src = in + k * Np * Q;
+    S* dst = static_cast<S*>(out) + k * Np * Qp;
+    float inv_s = 1.f, sc = 1.f;
+    // largest deviation of the element into its scale, over all threads of the group
+    auto set_scale = [&](float m) {
+      for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+      if constexpr (!kWarp) {
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+        __syncthreads();
+        m = red[0];
+        for (int j = 1; j < kThreads / 32; ++j) m = fmaxf(m, red[j]);
+      }
+      if constexpr (ST::dev) {
+        sc = 1.f;
+        if (m > 0.f) {
+          int e2;
+          frexpf(m, &e2);
+          sc = ldexpf(1.0f, e2 - ST::qmax_log2);
+        }
+        inv_s = 1.0f / sc;
+        if (lane == 0) scale[k] = sc;
+      }
+    };
+    const bool whole = rows >= Np;
+    if constexpr (ST::dev) {
+      if (!whole) {  // the element does not fit: its largest deviation in a pass of its own
+        float m = 0.f;
+        Walk w(lane, G, Q);
+        for (int j = lane; j < Np * Q; j += G, w.next()) m = fmaxf(m, fabsf(deviation(src[j], dt, w.c, w64, perm)));
+        set_scale(m);
+      }
+    }
+    for (int r0 = 0; r0 < Np; r0 += rows) {
+      const int nr = min(rows, Np - r0);
+      const TIn* s0 = src + size_t(r0) * Q;
+      float m = 0.f;
+      Walk w(lane, G, Q);
+      const int n = nr * Q;
+      for (int j = lane; j < n;) {
+        // several loads in flight per thread before the first is used
+        constexpr int U = 4;
+        TIn x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (j + u * G < n) x[u] = s0[j + u * G];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (j + u * G >= n) break;
+          const int at = w.row * Qp + perm[w.c];
+          if constexpr (ST::dev) {
+            const float d = deviation(x[u], dt, w.c, w64, perm);
+            m = fmaxf(m, fabsf(d));
+            buf[at] = d;
+          } else {
+            buf[at] = T(x[u]);
+          }
+          w.next();
+        }
+        j += U * G;
+      }
+      if constexpr (ST::dev) {
+        if (whole) set_scale(m);
+      }
+      group_sync<kWarp>();
+      const int nvec = nr * Qp / V;
+      S* d0 = dst + size_t(r0) * Qp;
+      for (int v = lane; v < nvec; v += G) {
+        __align__(16) S q[V];
+        if constexpr (ST::dev) {
+          __align__(16) float d[V];
+#pragma unroll
+          for (int j = 0; j < V / 4; ++j)
+            reinterpret_cast<uint4*>(d)[j] = reinterpret_cast<const uint4*>(buf + size_t(v) * V)[j];
+#pragma unroll
+          for (int j = 0; j < V; ++j) {
+            // the scale is a power of two; where its inverse leaves FP32's range, divide in FP64
+            q[j] = sc >= 1e-30f ? ST::from_r(d[j] * inv_s) : ST::from_r(float(double(d[j]) / double(sc)));
+          }
+          reinterpret_cast<uint4*>(d0)[v] = *reinterpret_cast<const uint4*>(q);
+        } else {
+          reinterpret_cast<uint4*>(d0)[v] = reinterpret_cast<const uint4*>(buf)[v];
+        }
+      }
+      group_sync<kWarp>();  // the buffer is free for the next rows (and red[] for the next element)
+    }
+  }
+}
+
+// Decode: the mirror image.  The internal row is read as 16-byte vectors and
+// scattered into shared memory by the canonical order; the caller's rows are
+// written along the canonical order.  Deviation forms stage s q (exact in
+// FP32: s is a power of two) and form w + w (s q) with one FP64 FMA per value.
+// Before (gathered 2- and 4-byte loads, three FP64-rate operations and two
+// integer divisions per value): 2.44 ms at 335M BF16 values, 90 us at 31M FP32
+// values; now 1.34 ms and 73 us (56 us for the latter's bytes).
+template <class ST, bool kWarp>
+__global__ void __launch_bounds__(kThreads) decode_kernel(const void* __restrict__ in,
+                                                          const float* __restrict__ scale, double* __restrict__ out,
+                                                          const double* __restrict__ vel64,
+                                                          const int32_t* __restrict__ iperm, int64_t K, int Np,
+                                                          int Q, int Qp, int rows, int table_bytes) {
+  using S = typename ST::S;
+  using T = std::conditional_t<ST::dev, float, S>;
+  constexpr int V = 16 / int(sizeof(S));
+  extern __shared__ __align__(16) unsigned char smem[];
+  double* wc = reinterpret_cast<double*>(smem);  // deviation forms: w in canonical order
+  int* inv = reinterpret_cast<int*>(smem + (ST::dev ? size_t(Q) * 8 : 0));  // canonical index, -1 for padding
+  const double* w64 = vel64 + 2 * Qp;
+  for (int i = threadIdx.x; i < Qp; i += kThreads) inv[i] = -1;
+  __syncthreads();
+  for (int c = threadIdx.x; c < Q; c += kThreads) {
+    const int i = iperm[c];
+    inv[i] = c;
+    if constexpr (ST::dev) wc[c] = w64[i];
+  }
+  const int G = kWarp ? 32 : kThreads;
+  const int grp = kWarp ? threadIdx.x / 32 : 0, lane = kWarp ? threadIdx.x % 32 : threadIdx.x;
+  const int ngroups = kWarp ? kThreads / 32 : 1;
+  T* buf = reinterpret_cast<T*>(smem + table_bytes) + size_t(grp) * rows * Qp;
+  __syncthreads();
+
+  const int vrow = Qp / V;  // vectors per row
+  for (int64_t k = blockIdx.x * int64_t(ngroups) + grp; k < K; k += int64_t(gridDim.x) * ngroups) {
+    const S* src = static_cast<const S*>(in) + k * Np * Qp;
+    double* dst = out + k * Np * Q;
+    const float s = ST::dev ? scale[k] : 0.f;
+    for (int r0 = 0; r0 < Np; r0 += rows) {
+      const int nr = min(rows, Np - r0);
+      const uint4* s0 = reinterpret_cast<const uint4*>(src + size_t(r0) * Qp);
+      const int nvec = nr * vrow;
+      Walk w(lane, G, vrow);
+      for (int v = lane; v < nvec;) {
+        constexpr int U = 2;
+        uint4 x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (v + u * G < nvec) x[u] = s0[v + u * G];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (v + u * G >= nvec) break;
+          const S* q = reinterpret_cast<const S*>(&x[u]);
+          T* row = buf + size_t(w.row) * Q;
+#pragma unroll
+          for (int j = 0; j < V; ++j) {
+            const int c = inv[w.c * V + j];
+            if (c >= 0) {
+              if constexpr (ST::dev) row[c] = s * ST::to_r(q[j]);
+              else row[c] = q[j];
+            }
+          }
+          w.next();
+        }
+        v += U * G;
+      }
+      group_sync<kWarp>();
+      double* d0 = dst + size_t(r0) * Q;
+      const int n = nr * Q;
+      if constexpr (ST::dev) {
+        Walk c(lane, G, Q);
+        for (int j = lane; j < n; j += G, c.next()) d0[j] = fma(wc[c.c], widen(buf[j]), wc[c.c]);
+      } else {
+        for (int j = lane; j < n; j += G) d0[j] = widen(buf[j]);
+      }
+      group_sync<kWarp>();
+    }
+  }
+}
+
+// Node moments.  G lanes share a node (as many as its row has 16-byte chunks,
+// at most a warp) and a group takes kNodes consecutive nodes at once, so that
+// each chunk's e_x, e_y (and w) are loaded once for kNodes nodes and the row
+// loads of all of them are in flight together.  Sums and quotients in the
+// state's compute precision R: FP64 arithmetic is slow here, and the FP32 and
+// 16-bit states carry FP32 precision.  Before, one warp per node whatever the
+// row's length, with the tables read again for every node: 480 us for 44M FP32
+// values at 16 velocities (4 of 32 lanes busy; 26 us for the bytes) and 851 us
+// for 335M BF16 values at 1,024 velocities (96 bytes of table per 16 of state);
+// now 51 us and 192 us.
+template <class ST>
+__global__ void __launch_bounds__(kThreads) moments_kernel(const void* __restrict__ in,
+                                                           const float* __restrict__ scale,
+                                                           const typename ST::R* __restrict__ vel, int64_t nodes,
+                                                           int Np, int Qp, int G, double* rho, double* ux,
+                                                           double* uy) {
+  using R = typename ST::R;
+  using S = typename ST::S;
+  constexpr int V = 16 / int(sizeof(S));
+  constexpr int kNodes = 4;
+  const int lane = threadIdx.x % G;
+  const int64_t ngroups = int64_t(gridDim.x) * (kThreads / G);
+  const R *ex = vel + kVelEx * Qp, *ey = vel + kVelEy * Qp, *wv = vel + kVelW * Qp;
+  // every lane of a warp runs the same number of iterations (the shuffles)
+  const int64_t first = (blockIdx.x * int64_t(kThreads) + threadIdx.x) / G;
+  const int64_t warp_first = (blockIdx.x * int64_t(kThreads) + threadIdx.x) / 32 * (32 / G);
+  for (int64_t it = 0; (warp_first + it * ngroups) * kNodes < nodes; ++it) {
+    const int64_t n0 = (first + it * ngroups) * kNodes;
+    R m0[kNodes] = {}, m1[kNodes] = {}, m2[kNodes] = {}, s[kNodes] = {};
+    const S* row[kNodes];
+#pragma unroll
+    for (int a = 0; a < kNodes; ++a) {
+      const int64_t kn = n0 + a < nodes ? n0 + a : nodes - 1;  // past the end: read the last node again
+      row[a] = static_cast<const S*>(in) + kn * Qp;
+      if constexpr (ST::dev) s[a] = R(scale[kn / Np]);
+    }
+#pragma unroll 2
+    for (int i = lane * V; i < Qp; i += G * V) {
+      uint4 x[kNodes];
+#pragma unroll
+      for (int a = 0; a < kNodes; ++a) x[a] = *reinterpret_cast<const uint4*>(row[a] + i);
+      __align__(16) R tx[V], ty[V], tw[V];
+#pragma unroll
+      for (int j = 0; j < V * int(sizeof(R)) / 16; ++j) {
+        reinterpret_cast<uint4*>(tx)[j] = __ldg(reinterpret_cast<const uint4*>(ex + i) + j);
+        reinterpret_cast<uint4*>(ty)[j] = __ldg(reinterpret_cast<const uint4*>(ey + i) + j);
+        if constexpr (ST::dev) reinterpret_cast<uint4*>(tw)[j] = __ldg(reinterpret_cast<const uint4*>(wv + i) + j);
+      }
+#pragma unroll
+      for (int a = 0; a < kNodes; ++a) {
+        const S* q = reinterpret_cast<const S*>(&x[a]);
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+          R f;
+          if constexpr (ST::dev) f = fmaf(tw[j] * s[a], ST::to_r(q[j]), tw[j]);
+          else f = R(q[j]);
+          m0[a] += f;
+          m1[a] = fma(tx[j], f, m1[a]);
+          m2[a] = fma(ty[j], f, m2[a]);
+        }
+      }
+    }
+    for (int off = G >> 1; off > 0; off >>= 1) {
+#pragma unroll
+      for (int a = 0; a < kNodes; ++a) {
+        m0[a] += __shfl_xor_sync(0xffffffffu, m0[a], off);
+        m1[a] += __shfl_xor_sync(0xffffffffu, m1[a], off);
+        m2[a] += __shfl_xor_sync(0xffffffffu, m2[a], off);
+      }
+    }
+    // every lane holds the sums: lane a of the group writes node a, so that the
+    // quotients of its nodes run side by side (fewer than kNodes lanes take turns)
+    for (int a0 = 0; a0 < kNodes; a0 += (G < kNodes ? G : kNodes)) {
+      const int a = a0 + lane;
+      R r0 = m0[0], r1 = m1[0], r2 = m2[0];
+#pragma unroll
+      for (int b = 1; b < kNodes; ++b)
+        if (a == b) {
+          r0 = m0[b];
+          r1 = m1[b];
+          r2 = m2[b];
+        }
+      if (a < kNodes && n0 + a < nodes) {
+        rho[n0 + a] = double(r0);
+        ux[n0 + a] = double(r1 / r0);
+        uy[n0 + a] = double(r2 / r0);
+      }
+    }
+  }
+}
+
+template <class F>
+cudaError_t allow_smem(F kernel, size_t smem) {
+  if (smem <= 48 * 1024) return cudaSuccess;
+  if (smem > kSmemCap) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemCap));
+}
+
+template <class ST, typename TIn>
+cudaError_t encode_as(const Shape& sh, const TIn* in, void* out, float* scale, cudaStream_t st) {
+  const Split s = split_for(sh, ST::dev ? 12 : 0, ST::dev ? 4 : sizeof(typename ST::S));
+  auto kernel = s.warp ? encode_kernel<ST, TIn, true> : encode_kernel<ST, TIn, false>;
+  cudaError_t e = allow_smem(kernel, s.smem);
+  if (e != cudaSuccess) return e;
+  kernel<<<s.grid, kThreads, s.smem, st>>>(in, out, scale, sh.vel64, sh.iperm, sh.K, sh.Np, sh.Q, sh.Qp, s.rows,
+                                           int(s.tables));
+  return cudaGetLastError();
+}
+
+template <class ST>
+cudaError_t decode_as(const Shape& sh, const void* in, const float* scale, double* out, cudaStream_t st) {
+  const Split s = split_for(sh, ST::dev ? 8 : 0, ST::dev ? 4 : sizeof(typename ST::S));
+  auto kernel = s.warp ? decode_kernel<ST, true> : decode_kernel<ST, false>;
+  cudaError_t e = allow_smem(kernel, s.smem);
+  if (e != cudaSuccess) return e;
+  kernel<<<s.grid, kThreads, s.smem, st>>>(in, scale, out, sh.vel64, sh.iperm, sh.K, sh.Np, sh.Q, sh.Qp, s.rows,
+                                           int(s.tables));
+  return cudaGetLastError();
+}
+
+template <class ST>
+cudaError_t moments_as(const Shape& sh, const void* in, const float* scale, const void* vel, double* rho, double* ux,
+                       double* uy, cudaStream_t st) {
+  const int chunks = sh.Qp * int(sizeof(typename ST::S)) / 16;
+  int G = 1;
+  while (G < 32 && G < chunks) G *= 2;
+  const int64_t nodes = sh.K * sh.Np;
+  int nsm = 152;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, sh.device);
+  const int64_t per_block = 4 * (kThreads / G);
+  const int grid = int(std::max<int64_t>(1, std::min<int64_t>((nodes + per_block - 1) / per_block, int64_t(nsm) * 32)));
+  moments_kernel<ST><<<grid, kThreads, 0, st>>>(in, scale, static_cast<const typename ST::R*>(vel), nodes, sh.Np,
+                                                sh.Qp, G, rho, ux, uy);
+  return cudaGetLastError();
+}
+
+template <typename TIn>
+cudaError_t encode_any(const Shape& sh, const TIn* in, void* out, float* scale, cudaStream_t st) {
+  switch (sh.store) {
+    case kStoreF64: return encode_as<StoreF64, TIn>(sh, in, out, scale, st);
+    case kStoreF32: return encode_as<StoreF32, TIn>(sh, in, out, scale, st);
+    case kStoreBF16: return encode_as<StoreBF16, TIn>(sh, in, out, scale, st);
+    default: return encode_as<StoreF16, TIn>(sh, in, out, scale, st);
+  }
+}
+
+}  // namespace
+
+cudaError_t encode(const Shape& sh, const double* in, void* out, float* scale, cudaStream_t st) {
+  return encode_any(sh, in, out, scale, st);
+}
+cudaError_t encode(const Shape& sh, const float* in, void* out, float* scale, cudaStream_t st) {
+  return encode_any(sh, in, out, scale, st);
+}
+
+cudaError_t decode(const Shape& sh, const void* in, const float* scale, double* out, cudaStream_t st) {
+  switch (sh.store) {
+    case kStoreF64: return decode_as<StoreF64>(sh, in, scale, out, st);
+    case kStoreF32: return decode_as<StoreF32>(sh, in, scale, out, st);
+    case kStoreBF16: return decode_as<StoreBF16>(sh, in, scale, out, st);
+    default: return decode_as<StoreF16>(sh, in, scale, out, st);
+  }
+}
+
+cudaError_t moments(const Shape& sh, const void* in, const float* scale, const void* vel, double* rho, double* ux,
+                    double* uy, cudaStream_t st) {
+  switch (sh.store) {
+    case kStoreF64: return moments_as<StoreF64>(sh, in, scale, vel, rho, ux, uy, st);
+    case kStoreF32: return moments_as<StoreF32>(sh, in, scale, vel, rho, ux, uy, st);
+    case kStoreBF16: return moments_as<StoreBF16>(sh, in, scale, vel, rho, ux, uy, st);
+    default: return moments_as<StoreF16>(sh, in, scale, vel, rho, ux, uy, st);
+  }
+}
+
+}  // namespace transfer
+}  // namespace fedbm
