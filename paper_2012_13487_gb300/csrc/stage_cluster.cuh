@@ -337,17 +337,10 @@ __global__ void __launch_bounds__(kThreads, cl_min_blocks<ST>()) stage_kernel_cl
         }
         R invw = R(0);
         if constexpr (ST::dev) invw = a.vel[kVelInvW * Qp + ig] / R(s_scale[e]);
-#pragma unroll
-        for (int n = 0; n < NP; ++n) {
-          R dr = 0, ds = 0, lf = 0;
-#pragma unroll
-          for (int m = 0; m < NP; ++m) {
-            dr = fma(opv<R, kImm>(OFF_DR + n * NP + m), fr[m], dr);
-            ds = fma(opv<R, kImm>(OFF_DS + n * NP + m), fr[m], ds);
-          }
-#pragma unroll
-          for (int q = 0; q < NF; ++q) lf = fma(opv<R, kImm>(OFF_LIFT + n * NF + q), flux[q], lf);
-          R rhs = fma(-ar, dr, fma(-as, ds, lf));
+        using M = EoScalar<R, kImm>;
+        R le[NE], lo[at_least_1(NO)];
+        eo_lift<M>(flux, true, true, le, lo);
+        eo_volume<M>(fr, R(-0.5) * (ar + as), R(0.5) * (ar - as), le, lo, [&](int n, R rhs) {
           rhs += collision<R>(s_mom + (size_t(e) * NP + n) * 8, ex, ey, w, fr[n], inv_tau, third);
           R r = dt * rhs;
           if (read_res) r = fma(rkA, rrow[n * Qc], r);
@@ -364,7 +357,7 @@ __global__ void __launch_bounds__(kThreads, cl_min_blocks<ST>()) stage_kernel_cl
           } else {
             frow[n * Qc] = S(fnew);
           }
-        }
+        });
       }
       if constexpr (ST::dev)
         for (int e = tid; e < ne; e += nth)

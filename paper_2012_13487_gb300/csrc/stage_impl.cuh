@@ -21,28 +21,24 @@
 //   3. wall numerators sum_{e.n>0} (e.n) f^- of eq. FullBC per wall node;
 //   4. residual and update, one thread per (element, velocity) item, with
 //      Dr, Ds, LIFT as instruction immediates (compile-time tables) or
-//      constant-memory operands of unrolled FMAs (the 16-bit forms up to
-//      degree 3 take two velocities per thread as packed FP32 pairs,
-//      fma.rn.f32x2);
+//      constant-memory operands of unrolled FMAs on the even and odd parts of f
+//      and of the flux (stage_eo.cuh; the 16-bit forms at degree 3 take two
+//      velocities per thread as packed FP32 pairs, fma.rn.f32x2);
 //   5. deviation forms only: per-element scale from max |f/w - 1|, encode;
 //   6. bulk-store the new state and residual tiles.
 #include "device_common.cuh"
 #include "stage_dispatch.h"
 
 #include <cstring>
+#include <type_traits>
 
-// Largest degree whose 16-bit forms take two velocities per thread (and the
-// FP32 state too when FEDBM_VPT2_FP32_STATE is 1); FEDBM_PACKED_FMA = 1 runs
-// the two velocities' contractions as packed FP32 pairs.  Measured on the BF16
-// cavities: two velocities per thread are faster at degree 3, one at degree 4.
-#ifndef FEDBM_VPT2_MAX_P
-#define FEDBM_VPT2_MAX_P 3
-#endif
-#ifndef FEDBM_VPT2_FP32_STATE
-#define FEDBM_VPT2_FP32_STATE 0
-#endif
-#ifndef FEDBM_PACKED_FMA
-#define FEDBM_PACKED_FMA 1
+// Degree at which the 16-bit forms take two velocities per thread as packed FP32
+// pairs, whose broadcast operators come from constant memory.  With the even-odd
+// contractions (GB300): BF16 cavity at 1,024 velocities, degree 3, 22.6 ms for a
+// two-step call against 24.7 ms with one velocity per thread and the operators as
+// immediates; FP16 at 256 velocities, degree 2, 640 us against 593 us.
+#ifndef FEDBM_VPT2_P
+#define FEDBM_VPT2_P 3
 #endif
 // FEDBM_FACE_SKIP = 0: the FMA kernel evaluates every face's flux and lift
 // columns also where a whole warp leaves an element through the face
@@ -66,49 +62,10 @@ constexpr int OFF_DS = NP * NP;
 constexpr int OFF_LIFT = 2 * NP * NP;
 constexpr int OPS_N = 2 * NP * NP + NP * NF;
 
-static __constant__ float c_ops32[OPS_N];
+// FP64 operators: the BF16 and TF32 pieces of the tensor-core operands are cut from them
 static __constant__ double c_ops64[OPS_N];
-// every FP32 coefficient twice, as the broadcast operand of a packed FMA
-static __constant__ unsigned long long c_ops32x2[OPS_N];
 
 #include "ops_tables.inc"
-
-// Dr, Ds, LIFT entry idx in the compute precision.  kImm: the FP32 operators
-// of this degree as a compile-time table (the operators depend only on the
-// degree, and with the node loops unrolled every entry becomes an instruction
-// immediate instead of a constant-memory load; the table holds the runtime
-// upload's values, which a CPU test checks); otherwise constant memory.
-template <typename R, bool kImm>
-__device__ __forceinline__ R opv(int idx);
-template <>
-__device__ __forceinline__ float opv<float, false>(int idx) { return c_ops32[idx]; }
-template <>
-__device__ __forceinline__ double opv<double, false>(int idx) { return c_ops64[idx]; }
-#ifdef FEDBM_OPS32_TABLE
-constexpr bool kHaveOpsTable = true;
-template <>
-__device__ __forceinline__ float opv<float, true>(int idx) {
-  constexpr float t[] = {FEDBM_OPS32_TABLE};
-  static_assert(sizeof(t) / sizeof(t[0]) == OPS_N, "operator table of another degree");
-  return t[idx];
-}
-#else
-constexpr bool kHaveOpsTable = false;
-template <>
-__device__ __forceinline__ float opv<float, true>(int idx) { return c_ops32[idx]; }
-#endif
-template <>
-__device__ __forceinline__ double opv<double, true>(int idx) { return c_ops64[idx]; }
-
-// Which FMA kernels take the operators as immediates: every FP32-arithmetic
-// kernel up to degree 4; at degree 5 (1,260 operator entries) only the
-// compile-time velocity counts of the FP32 and BF16 states, which keeps that
-// translation unit's compile time within a few minutes.
-template <class ST, int QT>
-__host__ __device__ constexpr bool ops_immediate() {
-  return kHaveOpsTable && sizeof(typename ST::R) == 4 &&
-         (P <= 4 || (QT > 0 && (ST::kind == kStoreF32 || ST::kind == kStoreBF16)));
-}
 
 // Node index of face node a on face f (rows of the reference triangle start at
 // a(P+1) - a(a-1)/2; face 0 is row 0, face 1 the row ends, face 2 the row starts).
@@ -133,6 +90,18 @@ __device__ __forceinline__ unsigned long long f2fma(unsigned long long a, unsign
   unsigned long long d;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
+}
+
+#include "stage_eo.cuh"
+
+// Which FMA kernels take the operators as immediates: every FP32-arithmetic
+// kernel up to degree 4; at degree 5 only the compile-time velocity counts of
+// the FP32 and BF16 states, which keeps that translation unit's compile time
+// within a few minutes.
+template <class ST, int QT>
+__host__ __device__ constexpr bool ops_immediate() {
+  return kHaveOpsTable && sizeof(typename ST::R) == 4 &&
+         (P <= 4 || (QT > 0 && (ST::kind == kStoreF32 || ST::kind == kStoreBF16)));
 }
 
 // ---- moment accumulators ----------------------------------------------------
@@ -437,11 +406,11 @@ __host__ __device__ constexpr bool keeps_scale() {
 }
 
 // Adjacent velocities handled by one thread in phase 4: two for the
-// specialised 16-bit-state kernels up to degree 3 (each operator constant then
-// feeds two FMAs and the per-item set-up is shared), else one.
+// specialised 16-bit-state kernels at degree FEDBM_VPT2_P (each operator constant
+// then feeds two FMAs and the per-item set-up is shared), else one.
 template <class ST, int QT>
 __host__ __device__ constexpr int items_vpt() {
-  return (QT > 0 && sizeof(typename ST::R) == 4 && (ST::dev || FEDBM_VPT2_FP32_STATE) && P <= FEDBM_VPT2_MAX_P)
+  return (QT > 0 && sizeof(typename ST::R) == 4 && ST::dev && P == FEDBM_VPT2_P)
              ? 2
              : 1;
 }
@@ -469,7 +438,7 @@ __device__ __forceinline__ void item_update(const StageArgs<typename ST::R>& a,
   const int tid = threadIdx.x, nth = blockDim.x;
   const R rkA = a.rkA, rkB = a.rkB, ab = a.ab;
   const bool third = a.eq_order == 3;
-  constexpr bool kPacked = FEDBM_PACKED_FMA && sizeof(R) == 4 && VPT == 2;
+  constexpr bool kPacked = VPT == 2;
   constexpr bool kImm = ops_immediate<ST, QT>();
   // outflow faces skipped per warp where a warp's items belong to one element
   // (one velocity per thread: with two, the packed lift accumulators measured
@@ -562,37 +531,24 @@ __device__ __forceinline__ void item_update(const StageArgs<typename ST::R>& a,
       }
     }
 
-    // kSkip: the lift contraction by faces, the faces without flux skipped
-    // (the same accumulation order as the node loop's)
-    R lfa[VPT][kSkip ? NP : 1];
-    unsigned long long lfp2[kSkip && kPacked ? NP : 1];
-    if constexpr (kSkip) {
+    using M = std::conditional_t<kPacked, EoPacked, EoScalar<R, kImm>>;
+    using T = typename M::T;
+    constexpr int NT = kPacked ? 1 : VPT;  // contractions per item
+    auto pack = [](const R* x) -> T {
+      if constexpr (kPacked) return f2pack(x[0], x[VPT - 1]);
+      else return x[0];
+    };
+    // even and odd parts of LIFT flux (the faces without flux skipped)
+    T le[NT][NE], lo[NT][at_least_1(NO)];
 #pragma unroll
-      for (int n = 0; n < NP; ++n) {
-        if constexpr (kPacked) lfp2[n] = 0ull;
+    for (int t = 0; t < NT; ++t) {
+      T fl[NF];
 #pragma unroll
-        for (int v = 0; v < VPT; ++v) lfa[v][n] = R(0);
+      for (int q = 0; q < NF; ++q) {
+        const R x[2] = {flux[t][q], flux[kPacked ? VPT - 1 : t][q]};
+        fl[q] = pack(x);
       }
-#pragma unroll
-      for (int fc = 0; fc < 3; ++fc) {
-        if (!on[fc]) continue;
-#pragma unroll
-        for (int aa = 0; aa < NFP; ++aa) {
-          const int j = fc * NFP + aa;
-          if constexpr (kPacked) {
-            const unsigned long long x = f2pack(flux[0][j], flux[1][j]);
-#pragma unroll
-            for (int n = 0; n < NP; ++n) lfp2[n] = f2fma(c_ops32x2[OFF_LIFT + n * NF + j], x, lfp2[n]);
-          } else {
-#pragma unroll
-            for (int n = 0; n < NP; ++n) {
-              const R cl = opv<R, kImm>(OFF_LIFT + n * NF + j);
-#pragma unroll
-              for (int v = 0; v < VPT; ++v) lfa[v][n] = fma(cl, flux[v][j], lfa[v][n]);
-            }
-          }
-        }
-      }
+      eo_lift<M>(fl, on[0] || on[2], on[1], le[t], lo[t]);
     }
     float dloc = 0.f;
     R invw[VPT];
@@ -601,65 +557,29 @@ __device__ __forceinline__ void item_update(const StageArgs<typename ST::R>& a,
 #pragma unroll
       for (int v = 0; v < VPT; ++v) invw[v] = iw.v[v] * (kKeep ? R(1) / R(sm.scale[e]) : R(1));
     }
-#pragma unroll
-    for (int n = 0; n < NP; ++n) {
+    // rhs, update and write-back of node n from its advection term
+    // -(e . grad) f + LIFT (flux)
+    auto finish = [&](int n, const R* adv) {
       RV rold;
       if (read_res) rold = *reinterpret_cast<const RV*>(rrow + n * Qp);
-      R dr[VPT], ds[VPT], lf[VPT];
-      if constexpr (kPacked) {
-        // two velocities per packed FMA; the same rounding as the scalar form
-        unsigned long long drp = 0ull, dsp = 0ull, lfp = 0ull;
+      // f itself from shared memory again: next to its even and odd parts the
+      // registers would not hold it without giving up a resident CTA (FP32 at
+      // degree 3, 36 velocities: 72 registers against 79, 7 CTAs against 6)
+      const SV fs = *reinterpret_cast<const SV*>(frow + n * Qp);
+      R fn[VPT];
 #pragma unroll
-        for (int m = 0; m < NP; ++m) {
-          const unsigned long long x = f2pack(fr[0][m], fr[1][m]);
-          drp = f2fma(c_ops32x2[OFF_DR + n * NP + m], x, drp);
-          dsp = f2fma(c_ops32x2[OFF_DS + n * NP + m], x, dsp);
-        }
-        if constexpr (kSkip) {
-          lfp = lfp2[n];
-        } else {
-#pragma unroll
-          for (int j = 0; j < NF; ++j)
-            lfp = f2fma(c_ops32x2[OFF_LIFT + n * NF + j], f2pack(flux[0][j], flux[1][j]), lfp);
-        }
-        f2unpack(drp, dr[0], dr[VPT - 1]);
-        f2unpack(dsp, ds[0], ds[VPT - 1]);
-        f2unpack(lfp, lf[0], lf[VPT - 1]);
-      } else {
-#pragma unroll
-        for (int v = 0; v < VPT; ++v) dr[v] = ds[v] = lf[v] = R(0);
-#pragma unroll
-        for (int m = 0; m < NP; ++m) {
-          const R cr = opv<R, kImm>(OFF_DR + n * NP + m), cs = opv<R, kImm>(OFF_DS + n * NP + m);
-#pragma unroll
-          for (int v = 0; v < VPT; ++v) {
-            dr[v] = fma(cr, fr[v][m], dr[v]);
-            ds[v] = fma(cs, fr[v][m], ds[v]);
-          }
-        }
-        if constexpr (kSkip) {
-#pragma unroll
-          for (int v = 0; v < VPT; ++v) lf[v] = lfa[v][n];
-        } else {
-#pragma unroll
-          for (int j = 0; j < NF; ++j) {
-            const R cl = opv<R, kImm>(OFF_LIFT + n * NF + j);
-#pragma unroll
-            for (int v = 0; v < VPT; ++v) lf[v] = fma(cl, flux[v][j], lf[v]);
-          }
-        }
-      }
+      for (int v = 0; v < VPT; ++v) fn[v] = decode<ST>(fs.v[v], wv.v[v], ws[v]);
       const R* mm = sm.mom + (size_t(e) * NP + n) * 8;
       RV rr;
       SV fnew_s;
 #pragma unroll
       for (int v = 0; v < VPT; ++v) {
-        R rhs = fma(-ar[v], dr[v], fma(-as[v], ds[v], lf[v]));
-        rhs += collision<R>(mm, exv.v[v], eyv.v[v], wv.v[v], fr[v][n], inv_tau, third);
+        R rhs = adv[v];
+        rhs += collision<R>(mm, exv.v[v], eyv.v[v], wv.v[v], fn[v], inv_tau, third);
         R r = dt * rhs;
         if (read_res) r = fma(rkA, rold.v[v], r);
         rr.v[v] = r;
-        const R fnew = new_f<ST>(fr[v][n], rkB, r);
+        const R fnew = new_f<ST>(fn[v], rkB, r);
         if constexpr (kTrack) {
           dloc = fmaxf(dloc, fabsf((fnew - wv.v[v]) * invw[v]));
         } else if constexpr (kKeep) {
@@ -676,7 +596,26 @@ __device__ __forceinline__ void item_update(const StageArgs<typename ST::R>& a,
       }
       *reinterpret_cast<RV*>(rrow + n * Qp) = rr;
       if constexpr (!kTrack) *reinterpret_cast<SV*>(frow + n * Qp) = fnew_s;
+    };
+    static_assert(kPacked || VPT == 1, "two velocities per thread run as packed pairs");
+    R an[2], dn[2];
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+      an[v] = R(-0.5) * (ar[v] + as[v]);
+      dn[v] = R(0.5) * (ar[v] - as[v]);
     }
+    T fp[NP];
+#pragma unroll
+    for (int m = 0; m < NP; ++m) {
+      const R x[2] = {fr[0][m], fr[VPT - 1][m]};
+      fp[m] = pack(x);
+    }
+    eo_volume<M>(fp, pack(an), pack(dn), le[0], lo[0], [&](int n, T adv) {
+      R x[2];
+      if constexpr (kPacked) f2unpack(adv, x[0], x[1]);
+      else x[0] = adv;
+      finish(n, x);
+    });
     if constexpr (kTrack) {
       if (e != emax) {
         if (emax >= 0) atomicMax(&sm.dmax[emax], __float_as_uint(dmax));
@@ -1037,25 +976,28 @@ cudaError_t set_smem(int store_kind, int Qp, size_t smem) {
 }
 
 cudaError_t upload(const double* Dr, const double* Ds, const double* LIFT) {
-  double h64[OPS_N];
-  float h32[OPS_N];
+  double h64[OPS_N], eo64[EO_N] = {};
+  float eo32[EO_N];
+  unsigned long long eo32x2[EO_N];
   for (int j = 0; j < NP * NP; ++j) {
     h64[OFF_DR + j] = Dr[j];
     h64[OFF_DS + j] = Ds[j];
   }
   for (int j = 0; j < NP * NF; ++j) h64[OFF_LIFT + j] = LIFT[j];
-  unsigned long long h32x2[OPS_N];
-  for (int j = 0; j < OPS_N; ++j) {
-    h32[j] = float(h64[j]);
+  eo_coefficients(Dr, Ds, LIFT, eo64);
+  for (int j = 0; j < EO_N; ++j) {
+    eo32[j] = float(eo64[j]);
     uint32_t bits;
-    std::memcpy(&bits, &h32[j], 4);
-    h32x2[j] = (static_cast<unsigned long long>(bits) << 32) | bits;
+    std::memcpy(&bits, &eo32[j], 4);
+    eo32x2[j] = (static_cast<unsigned long long>(bits) << 32) | bits;
   }
   cudaError_t e = cudaMemcpyToSymbol(c_ops64, h64, sizeof(h64));
   if (e != cudaSuccess) return e;
-  e = cudaMemcpyToSymbol(c_ops32x2, h32x2, sizeof(h32x2));
+  e = cudaMemcpyToSymbol(c_eo64, eo64, sizeof(eo64));
   if (e != cudaSuccess) return e;
-  return cudaMemcpyToSymbol(c_ops32, h32, sizeof(h32));
+  e = cudaMemcpyToSymbol(c_eo32x2, eo32x2, sizeof(eo32x2));
+  if (e != cudaSuccess) return e;
+  return cudaMemcpyToSymbol(c_eo32, eo32, sizeof(eo32));
 }
 
 }  // namespace

@@ -443,22 +443,21 @@ __global__ void __launch_bounds__(kWsThreads, 2) stage_kernel_ws(const StageArgs
         fout[gi] = fnew;
       }
     };
-    constexpr bool kImm = ops_immediate<ST, kWsQ>();
+    using M = EoScalar<float, ops_immediate<ST, kWsQ>()>;
+    float le[NE], lo[at_least_1(NO)];
+    eo_lift<M>(flux, on[0] || on[2], on[1], le, lo);
     if constexpr (kMma) {
       // lift on FMAs while the MMAs run, then the accumulators in groups of 8 nodes
       float lf[NP];
+      constexpr EoPairs pr = eo_pairs();
 #pragma unroll
-      for (int n = 0; n < NP; ++n) lf[n] = 0.f;
-#pragma unroll
-      for (int fc = 0; fc < 3; ++fc) {
-        if (!on[fc]) continue;
-#pragma unroll
-        for (int n = 0; n < NP; ++n)
-#pragma unroll
-          for (int aa = 0; aa < NFP; ++aa) {
-            const int q = fc * NFP + aa;
-            lf[n] = fmaf(opv<float, kImm>(OFF_LIFT + n * NF + q), flux[q], lf[n]);
-          }
+      for (int q = 0; q < NE; ++q) {
+        if (q < NO) {
+          lf[pr.a[q]] = le[q] + lo[q];
+          lf[pr.b[q]] = le[q] - lo[q];
+        } else {
+          lf[pr.a[q]] = le[q];
+        }
       }
       const float arw = ar * ws, asw = as * ws;  // Dr f = w s (Dr q)
       if (!mbar_wait_bounded(mma_bar, uint32_t(j & 1), 2000000000ull) && a.err) atomicExch(a.err, 1);
@@ -475,45 +474,8 @@ __global__ void __launch_bounds__(kWsThreads, 2) stage_kernel_ws(const StageArgs
         for (int q = 0; q < 8; ++q)
           if (8 * c + q < NP) finish(8 * c + q, fmaf(-arw, V[q], fmaf(-asw, W[q], lf[8 * c + q])));
       }
-    } else if (FEDBM_WS_SKIP) {
-      // lift by faces (the faces without flux skipped), then volume and update
-      float lf[NP];
-#pragma unroll
-      for (int n = 0; n < NP; ++n) lf[n] = 0.f;
-#pragma unroll
-      for (int fc = 0; fc < 3; ++fc) {
-        if (!on[fc]) continue;
-#pragma unroll
-        for (int n = 0; n < NP; ++n)
-#pragma unroll
-          for (int aa = 0; aa < NFP; ++aa) {
-            const int q = fc * NFP + aa;
-            lf[n] = fmaf(opv<float, kImm>(OFF_LIFT + n * NF + q), flux[q], lf[n]);
-          }
-      }
-#pragma unroll
-      for (int n = 0; n < NP; ++n) {
-        float dr = 0.f, ds = 0.f;
-#pragma unroll
-        for (int m = 0; m < NP; ++m) {
-          dr = fmaf(opv<float, kImm>(OFF_DR + n * NP + m), fr[m], dr);
-          ds = fmaf(opv<float, kImm>(OFF_DS + n * NP + m), fr[m], ds);
-        }
-        finish(n, fmaf(-ar, dr, fmaf(-as, ds, lf[n])));
-      }
     } else {
-#pragma unroll
-      for (int n = 0; n < NP; ++n) {
-        float dr = 0.f, ds = 0.f, lf = 0.f;
-#pragma unroll
-        for (int m = 0; m < NP; ++m) {
-          dr = fmaf(opv<float, kImm>(OFF_DR + n * NP + m), fr[m], dr);
-          ds = fmaf(opv<float, kImm>(OFF_DS + n * NP + m), fr[m], ds);
-        }
-#pragma unroll
-        for (int q = 0; q < NF; ++q) lf = fmaf(opv<float, kImm>(OFF_LIFT + n * NF + q), flux[q], lf);
-        finish(n, fmaf(-ar, dr, fmaf(-as, ds, lf)));
-      }
+      eo_volume<M>(fr, -0.5f * (ar + as), 0.5f * (ar - as), le, lo, finish);
     }
     if constexpr (ST::dev)
       if (tid == 0) a.scale_out[k] = sc;
