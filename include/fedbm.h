@@ -138,18 +138,20 @@ typedef struct fedbm_params {
   int32_t threads_per_cta; /* stage-kernel tile: threads per CTA, multiple of 32,
                             <= 256 (0 = auto)                                  */
   int32_t pipeline_stages; /* stage-kernel tile buffers per CTA: 1, or 2 to load
-                              the next tile while computing one (0 = auto: 3
-                              where that form measured faster, i.e. 256 padded
-                              velocities with FP32 state at degree 1-4 or BF16
-                              at degree 3-5, when the tile arguments are 0
-                              too; else 1);
+                              the next tile while computing one (0 = auto: the
+                              warp-specialised form where it measured faster,
+                              i.e. FP32 or BF16 state with 256 padded velocities
+                              at degree 1-5 or 1024 at degree 1-3, when the tile
+                              arguments are 0 too; else 1);
                               3 = the warp-specialised form: a producer warp
-                              keeps a ring of three one-element tiles filled
-                              (bulk copies) for eight consumer warps, one
-                              velocity per thread, 288 threads per CTA (tile
-                              arguments ignored); FP32 or BF16 state with 256
-                              padded velocities at degree <= 5, else EINVAL.
-                              The autotuner times it where it exists      */
+                              keeps a ring of one-element tiles filled (bulk
+                              copies) for consumer warps, two velocities per
+                              thread (tile arguments ignored); asked for by
+                              number it has two groups of four consumer warps,
+                              288 threads per CTA, and serves FP32 or BF16 state
+                              with 256 padded velocities at degree <= 5, else
+                              EINVAL.  The autotuner times the automatic
+                              choice's form where it exists              */
   int32_t tensor_cores;  /* stage-kernel form: 0 = the FMA kernel (the
                             faster form on every measured shape), with the
                             tensor-core form as one of the autotuner's

@@ -262,6 +262,7 @@ struct Group {
   int64_t K = 0;
   std::vector<int> cases;
   int epc = 0, tpb = 0, nstages = 1, grid = 0;
+  int ws_groups = 1;  // warp-specialised form: consumer groups per CTA
   size_t smem = 0;
   RefOps ops;
   VelocitySet vs;
@@ -351,7 +352,7 @@ cudaError_t launch_args(const Group& g, const void* args, cudaStream_t st, int g
   if (grid <= 0) grid = g.grid;
   if (g.ncl > 1) return e.launch_cl(g.store, args, g.grid / g.ncl, g.ncl, g.smem, st);
   if (g.tc) return e.launch_tc(g.store, args, grid, g.smem, st);
-  if (g.nstages == 3) return e.launch_ws(g.store, args, grid, g.smem, st);
+  if (g.nstages == 3) return e.launch_ws(g.store, args, g.ws_groups, grid, g.smem, st);
   return e.launch(g.store, args, grid, g.tpb, g.smem, st);
 }
 
@@ -452,37 +453,46 @@ int auto_cluster(const Group& g) {
   return best;
 }
 
-// The warp-specialised form of a group: one element per ring stage, eight
-// consumer warps (one velocity per thread) and one producer warp.
-bool ws_available(const Group& g) { return stage_entry(g.p).ws_smem(g.store, g.Qp) > 0; }
+// The warp-specialised form of a group: one element per ring stage, four or
+// eight consumer warps (two velocities per thread) and one producer warp.
+// Consumer groups per CTA of the automatic choice: one with 256 velocities (three
+// CTAs share an SM), three with 1,024 (one CTA per SM: two ring stages of each of
+// three CTAs would not fit).
+int ws_groups(const Group& g) { return g.Qp == 1024 ? 3 : 1; }
+bool ws_available(const Group& g) { return stage_entry(g.p).ws_smem(g.store, g.Qp, ws_groups(g)) > 0; }
 
-// The untuned default takes the warp-specialised form where it measured
-// faster than the FMA kernel's default tile on the 256-velocity cavities of
-// about 30M DOF: FP32 state at degree 1-4 (x1.04-1.12), BF16 at degree 3-5
-// (x1.21-1.41, the volume contractions on tensor cores).  FP32 at degree 5
-// holds one CTA per SM (three 39 KB stages) and BF16 at degree 1-2 loses to
-// the FMA kernel's two velocities per thread.
+// The untuned default takes the warp-specialised form wherever it exists from
+// degree 1 up (with 1,024 velocities up to degree 3: at degree 4 two ring stages of
+// FP32 state do not fit and BF16 spills).  One step of 20M values on the GB300, the
+// FMA kernel or the former warp-specialised one (one velocity per thread, eight
+// consumer warps) against this one, us at degree 1..5: 256 velocities FP32 484, 341,
+// 334, 349, 524 -> 361, 272, 274, 299, 399; BF16 751, 546, 433, 386, 471 -> 437, 329,
+// 322, 386, 438; 1,024 velocities FP32 736, 628, 837 -> 350, 298, 400; BF16 471, 527,
+// 636 -> 419, 306, 300.
 bool ws_default(const Group& g) {
   if (!ws_available(g)) return false;
-  return (g.store == kStoreF32 && g.p >= 1 && g.p <= 4) || (g.store == kStoreBF16 && g.p >= 3);
+  if (g.Qp == 1024) return g.p <= 3;
+  return g.p >= 1;
 }
 
-int configure_ws(Batch& b, Group& g) {
+int configure_ws(Batch& b, Group& g, int groups = 0) {
+  if (groups == 0) groups = ws_groups(g);
   const StageEntry e = stage_entry(g.p);
-  const size_t smem = e.ws_smem(g.store, g.Qp);
+  const size_t smem = e.ws_smem(g.store, g.Qp, groups);
   if (smem == 0)
     return fail(FEDBM_EINVAL, "pipeline_stages = 3 (the warp-specialised stage kernel) needs FP32 or BF16 state, "
                               "256 padded velocities and degree <= 5");
   if (smem > kMaxSmem) return fail(FEDBM_EINVAL, "warp-specialised ring does not fit in shared memory");
-  FEDBM_CK(e.set_smem_ws(g.store, kMaxSmem));
+  FEDBM_CK(e.set_smem_ws(g.store, g.Qp, groups, kMaxSmem));
   int nsm = 0;
   FEDBM_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b.device));
-  const int per_sm = e.occupancy_ws(g.store, smem);
+  const int per_sm = e.occupancy_ws(g.store, g.Qp, groups, smem);
   if (per_sm < 1) return fail(FEDBM_EINVAL, "warp-specialised stage kernel cannot be resident on an SM");
   g.tc = 0;
   g.ncl = 0;
   g.epc = 1;
-  g.tpb = 288;
+  g.tpb = e.ws_threads(g.store, g.Qp, groups);
+  g.ws_groups = groups;
   g.nstages = 3;
   g.smem = smem;
   g.grid = int(std::min<int64_t>(g.K, int64_t(per_sm) * nsm));
@@ -492,7 +502,15 @@ int configure_ws(Batch& b, Group& g) {
 
 // Tile shape, pipeline depth and persistent grid of a group's stage kernel.
 int configure_tiles(Batch& b, Group& g, int epc, int tpb, int stages) {
-  if (stages == 3) return configure_ws(b, g);  // tile and threads are the form's own
+  if (stages == 3) {
+    // tile and threads are the form's own.  Asked for by number it serves 256
+    // padded velocities, as before it had a 1,024-velocity kernel, which only
+    // the automatic choice and the autotuner take
+    if (g.Qp != 256)
+      return fail(FEDBM_EINVAL, "pipeline_stages = 3 (the warp-specialised stage kernel) needs FP32 or BF16 state, "
+                                "256 padded velocities and degree <= 5");
+    return configure_ws(b, g, 2);
+  }
   // the group is changed only once the whole configuration is valid
   int e_pc = epc > 0 ? epc : (g.Qp < 128 ? std::max(1, 128 / g.Qp) : 1);
   int t_pb = tpb > 0 ? tpb : std::min(128, std::max(32, (e_pc * g.Qp + 31) / 32 * 32));
@@ -550,6 +568,7 @@ struct TuneEntry {
 
 int apply_tune(Batch& b, Group& g, const TuneEntry& t) {
   if (t.ncl > 1) return configure_cluster(b, g, t.ncl);
+  if (t.stages == 3) return configure_ws(b, g);
   return t.tc ? configure_tc(b, g) : configure_tiles(b, g, t.epc, t.tpb, t.stages);
 }
 
@@ -661,7 +680,7 @@ int autotune(Batch& b, const char* cache_path, int trials) {
     if (ws_available(g) && configure_ws(b, g) == FEDBM_OK) {
       TuneEntry cand;
       cand.epc = 1;
-      cand.tpb = 288;
+      cand.tpb = g.tpb;
       cand.stages = 3;
       time_current(cand);
     }

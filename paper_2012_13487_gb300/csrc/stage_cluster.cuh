@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(kThreads, cl_min_blocks<ST>()) stage_kernel_cl
         using M = EoScalar<R, kImm>;
         R le[NE], lo[at_least_1(NO)];
         eo_lift<M>(flux, true, true, le, lo);
-        eo_volume<M>(fr, R(-0.5) * (ar + as), R(0.5) * (ar - as), le, lo, [&](int n, R rhs) {
+        eo_volume<M>([&](int n) { return fr[n]; }, R(-0.5) * (ar + as), R(0.5) * (ar - as), le, lo, [&](int n, R rhs) {
           rhs += collision<R>(s_mom + (size_t(e) * NP + n) * 8, ex, ey, w, fr[n], inv_tau, third);
           R r = dt * rhs;
           if (read_res) r = fma(rkA, rrow[n * Qc], r);

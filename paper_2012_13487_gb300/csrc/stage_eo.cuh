@@ -111,6 +111,20 @@ struct EoPacked {
   static __device__ __forceinline__ T fmac(int idx, T x, T z) { return f2fma(c_eo32x2[idx], x, z); }
 };
 
+// Two velocities per thread with the operators as immediates: additions and
+// scalings act on the packed pair, products with an operator on its halves (a
+// packed FMA takes no immediate, and its broadcast operand would be one more load).
+template <bool kImm>
+struct EoDual : EoPacked {
+  static __device__ __forceinline__ T fmac(int idx, T x, T z) {
+    float x0, x1, z0, z1;
+    f2unpack(x, x0, x1);
+    f2unpack(z, z0, z1);
+    const float c = eov<float, kImm>(idx);
+    return f2pack(fmaf(c, x0, z0), fmaf(c, x1, z1));
+  }
+};
+
 // Even and odd parts le, lo of LIFT flux.  on02, on1: faces 0 and 2, or face 1,
 // carry flux for some velocity of the warp; the others' columns are skipped.
 template <class M>
@@ -146,10 +160,10 @@ __device__ __forceinline__ void eo_lift(const typename M::T (&flux)[NF], bool on
   }
 }
 
-// -(ar Dr + as Ds) f + LIFT flux, handed to fin(node, value) node by node.
-// na = -(ar + as) / 2, nd = (ar - as) / 2.
-template <class M, class Fin>
-__device__ __forceinline__ void eo_volume(const typename M::T (&f)[NP], typename M::T na, typename M::T nd,
+// -(ar Dr + as Ds) f + LIFT flux of f(node), handed to fin(node, value) node by
+// node.  na = -(ar + as) / 2, nd = (ar - as) / 2.
+template <class M, class F, class Fin>
+__device__ __forceinline__ void eo_volume(F f, typename M::T na, typename M::T nd,
                                           const typename M::T (&le)[NE],
                                           const typename M::T (&lo)[at_least_1(NO)], Fin fin) {
   using T = typename M::T;
@@ -157,8 +171,14 @@ __device__ __forceinline__ void eo_volume(const typename M::T (&f)[NP], typename
   T E[NE], O[at_least_1(NO)];
 #pragma unroll
   for (int q = 0; q < NE; ++q) {
-    E[q] = q < NO ? M::add(f[pr.a[q]], f[pr.b[q]]) : f[pr.a[q]];
-    if (q < NO) O[q] = M::sub(f[pr.a[q]], f[pr.b[q]]);
+    const T fa = f(pr.a[q]);
+    if (q < NO) {
+      const T fb = f(pr.b[q]);
+      E[q] = M::add(fa, fb);
+      O[q] = M::sub(fa, fb);
+    } else {
+      E[q] = fa;
+    }
   }
 #pragma unroll
   for (int q = 0; q < NE; ++q) {

@@ -92,6 +92,12 @@ __device__ __forceinline__ unsigned long long f2fma(unsigned long long a, unsign
   return d;
 }
 
+__device__ __forceinline__ unsigned long long f2mul(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
 #include "stage_eo.cuh"
 
 // Which FMA kernels take the operators as immediates: every FP32-arithmetic
@@ -610,7 +616,7 @@ __device__ __forceinline__ void item_update(const StageArgs<typename ST::R>& a,
       const R x[2] = {fr[0][m], fr[VPT - 1][m]};
       fp[m] = pack(x);
     }
-    eo_volume<M>(fp, pack(an), pack(dn), le[0], lo[0], [&](int n, T adv) {
+    eo_volume<M>([&](int n) { return fp[n]; }, pack(an), pack(dn), le[0], lo[0], [&](int n, T adv) {
       R x[2];
       if constexpr (kPacked) f2unpack(adv, x[0], x[1]);
       else x[0] = adv;
@@ -1018,6 +1024,7 @@ StageEntry FEDBM_STAGE_ENTRY_NAME() {
   s.set_smem_cl = &set_smem_cl;
   s.occupancy_cl = &occupancy_cl;
   s.ws_smem = &ws_smem;
+  s.ws_threads = &ws_threads;
   s.launch_ws = &launch_ws;
   s.set_smem_ws = &set_smem_ws;
   s.occupancy_ws = &occupancy_ws;
