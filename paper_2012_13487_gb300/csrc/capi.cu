@@ -500,6 +500,48 @@ int configure_ws(Batch& b, Group& g, int groups = 0) {
   return FEDBM_OK;
 }
 
+// The FMA kernel's tile where the caller leaves it open: elements and threads per
+// CTA by velocity count, degree, state and the group's element count K.  FP32
+// arithmetic takes two velocities per thread, FP64 one.
+//
+// Where the elements do not fill the SMs several times over (K below 16 per SM),
+// small tiles spread them (about two CTAs per SM) and get more threads than items,
+// which the moment reduction uses; one tile per SM with idle SMs beside it was the
+// rule before.  Above that, 16 velocities run best in CTAs of one warp (no barrier
+// ever waits for another warp), with two items per thread at low degree once there
+// are enough of them.  Stage times on the GB300, us, this rule against 8 (degree <= 2:
+// 16) elements and one thread per item: FP32, 16 velocities, degree 1, 3, 5: K = 128
+// 5.6, 6.6, 8.2 against 6.3, 8.2, 11.9; K = 2,048 5.8, 7.0, 9.4 against 6.4, 8.2, 11.5;
+// K = 51,200 15.7, 38.5, 80.7 against 18.2, 39.6, 82.6; BF16 degree 1, 2, K = 204,800
+// 58.9, 96.3 against 93.9, 126.0; 36 velocities, degree 2, 4: K = 512 6.6, 8.4 against
+// 7.4, 11.1; K = 18,432 degree 2 23.5 against 27.5; FP64, 16 velocities, degree 3: K =
+// 128, 512, 2,048 20.9, 23.0, 39.0 against 28.7, 28.7, 42.7; D2Q1089 at degree 4, K =
+// 800, 256 threads instead of 128: FP32 88.6 against 102.4, BF16 108.9 against 146.7 (at
+// degree 1, 1,024 velocities, FP16, 20M values: 169 against 123, so not there).
+void auto_tile(const Group& g, int* epc, int* tpb) {
+  const bool f64 = g.store == kStoreF64;
+  const int64_t K = g.K;
+  const bool few = K < 16 * 152;
+  const int spread = int(std::min<int64_t>(4, (K + 303) / 304));  // elements per CTA, two CTAs per SM
+  if (g.Qp == 16 && f64) {
+    *epc = !few ? 8 : K <= 304 ? 1 : 2;
+    *tpb = !few ? 128 : K <= 1216 ? 64 : 32;
+  } else if (g.Qp == 16) {
+    *epc = few ? spread : K < 32768 ? 4 : g.p <= 3 ? 8 : 4;
+    if (K >= 32768 && g.p == 1 && g.store >= kStoreBF16) *epc = 16;
+    *tpb = few ? 32 * spread : 32;
+  } else if (g.Qp < 128 && !f64) {
+    *epc = std::max(1, 128 / g.Qp);
+    if (few) *epc = std::min(*epc, spread);
+    *tpb = few ? std::min(128, 64 * *epc) : g.p <= 2 && K >= 64 * 152 ? 32 : 64;
+  } else {
+    *epc = std::max(1, 128 / g.Qp);
+    const int items = *epc * g.Qp / (f64 ? 1 : 2);
+    const bool wide = !f64 && items >= 512 && (g.p >= 3 || (g.p == 2 && items > 512));
+    *tpb = wide ? 256 : std::min(128, std::max(32, (items + 31) / 32 * 32));
+  }
+}
+
 // Tile shape, pipeline depth and persistent grid of a group's stage kernel.
 int configure_tiles(Batch& b, Group& g, int epc, int tpb, int stages) {
   if (stages == 3) {
@@ -512,15 +554,12 @@ int configure_tiles(Batch& b, Group& g, int epc, int tpb, int stages) {
     return configure_ws(b, g, 2);
   }
   // the group is changed only once the whole configuration is valid
-  int e_pc = epc > 0 ? epc : (g.Qp < 128 ? std::max(1, 128 / g.Qp) : 1);
-  int t_pb = tpb > 0 ? tpb : std::min(128, std::max(32, (e_pc * g.Qp + 31) / 32 * 32));
-  if (epc == 0 && tpb == 0 && g.Qp == 16 && (g.store == kStoreF32 || g.store == kStoreBF16)) {
-    // 16 velocities: the autotuner's picks on ~20-45M-DOF Couette cases (FP32
-    // x1.4 at degree 1, x1.15 at 2; BF16 x1.9, 1.8, 1.6, 1.25, 1.04 at 1..5):
-    // 16 elements per tile up to degree 2, else 8; 64 threads for BF16 state
-    // (one item per thread where two velocities share a thread)
-    e_pc = g.p <= 2 ? 16 : 8;
-    t_pb = g.store == kStoreBF16 ? 64 : 128;
+  int e_pc = epc, t_pb = tpb;
+  if (epc <= 0 && tpb <= 0) {
+    auto_tile(g, &e_pc, &t_pb);
+  } else {
+    if (epc <= 0) e_pc = g.Qp < 128 ? std::max(1, 128 / g.Qp) : 1;
+    if (tpb <= 0) t_pb = std::min(128, std::max(32, (e_pc * g.Qp + 31) / 32 * 32));
   }
   if (t_pb % 32 || t_pb > 256) return fail(FEDBM_EINVAL, "threads_per_cta must be a multiple of 32, <= 256");
   if (stages < 0 || stages > 3) return fail(FEDBM_EINVAL, "pipeline_stages must be 0, 1, 2 or 3");

@@ -110,19 +110,21 @@ __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(
 // launch with it and the kernel carves its buffers with it.
 enum SmemPart { kSmBar, kSmF, kSmRes, kSmTr, kSmGeo, kSmNbr, kSmScale, kSmNScale, kSmDmax, kSmMom, kSmWn, kSmVel, kSmEnd };
 
+// direct: the kernel reads neighbour traces from global memory itself (their row
+// numbers stand in place of the rows) and keeps 14 floats per node record.
 __host__ __device__ inline size_t stage_smem_layout(int Np, int NF, int epc, int Qp, size_t s_bytes, size_t r_bytes,
-                                                    size_t off[kSmEnd + 1]) {
+                                                    bool direct, size_t off[kSmEnd + 1]) {
   size_t b = 0;
   off[kSmBar] = b;    b += 16;
   off[kSmF] = b;      b += align16(size_t(epc) * Np * Qp * s_bytes);   // element tile (updated in place)
   off[kSmRes] = b;    b += align16(size_t(epc) * Np * Qp * r_bytes);   // residual tile (updated in place)
-  off[kSmTr] = b;     b += align16(size_t(epc) * NF * Qp * s_bytes);   // neighbour face traces
+  off[kSmTr] = b;     b += align16(size_t(epc) * NF * (direct ? 4 : Qp * s_bytes));  // neighbour face traces or their rows
   off[kSmGeo] = b;    b += align16(size_t(epc) * kGeoStrideDev * r_bytes);
   off[kSmNbr] = b;    b += align16(size_t(epc) * 3 * 4);
   off[kSmScale] = b;  b += align16(size_t(epc) * 4);                  // element scale (deviation forms)
   off[kSmNScale] = b; b += align16(size_t(epc) * 3 * 4);              // neighbour scales, then new scale
   off[kSmDmax] = b;   b += align16(size_t(epc) * 4);
-  off[kSmMom] = b;    b += align16(size_t(epc) * Np * 8 * r_bytes);   // f^eq/tau coefficients per node
+  off[kSmMom] = b;    b += align16(size_t(epc) * Np * (direct ? 14 : 8) * r_bytes);  // f^eq/tau coefficients per node
   off[kSmWn] = b;     b += align16(size_t(epc) * NF * r_bytes);        // wall numerators
   off[kSmVel] = b;    b += align16(size_t(3) * Qp * r_bytes);          // e_x, e_y, w rows (copied once)
   off[kSmEnd] = b;
@@ -146,9 +148,9 @@ struct StageSmem {
 };
 
 template <typename R, typename S>
-__device__ inline StageSmem<R, S> carve_stage_smem(unsigned char* base, int Np, int NF, int epc, int Qp) {
+__device__ inline StageSmem<R, S> carve_stage_smem(unsigned char* base, int Np, int NF, int epc, int Qp, bool direct) {
   size_t off[kSmEnd + 1];
-  stage_smem_layout(Np, NF, epc, Qp, sizeof(S), sizeof(R), off);
+  stage_smem_layout(Np, NF, epc, Qp, sizeof(S), sizeof(R), direct, off);
   StageSmem<R, S> s;
   s.bar = reinterpret_cast<uint64_t*>(base + off[kSmBar]);
   s.f = reinterpret_cast<S*>(base + off[kSmF]);
@@ -166,16 +168,24 @@ __device__ inline StageSmem<R, S> carve_stage_smem(unsigned char* base, int Np, 
 }
 
 // Bytes between the two pipeline stages of a CTA (one stage, 128-byte aligned).
-__host__ __device__ inline size_t stage_smem_stride(int Np, int NF, int epc, int Qp, size_t s_bytes, size_t r_bytes) {
+__host__ __device__ inline size_t stage_smem_stride(int Np, int NF, int epc, int Qp, size_t s_bytes, size_t r_bytes,
+                                                    bool direct) {
   size_t off[kSmEnd + 1];
-  return (stage_smem_layout(Np, NF, epc, Qp, s_bytes, r_bytes, off) + 127) & ~size_t(127);
+  return (stage_smem_layout(Np, NF, epc, Qp, s_bytes, r_bytes, direct, off) + 127) & ~size_t(127);
+}
+
+// The FMA kernels that read neighbour traces from global memory themselves: 16
+// velocities, FP32 arithmetic, degree <= 5.
+__host__ __device__ constexpr bool stage_direct_traces(int p, int store_kind, int Qp) {
+  return Qp == 16 && p <= 5 && store_kind != kStoreF64;
 }
 
 // Dynamic shared memory of one stage CTA with `nstages` pipeline stages.
 __host__ inline size_t stage_smem_bytes(int p, int store_kind, int epc, int Qp, int nstages) {
   const size_t s_bytes = store_kind == kStoreF64 ? 8 : store_kind == kStoreF32 ? 4 : 2;
   const size_t r_bytes = store_kind == kStoreF64 ? 8 : 4;
-  return size_t(nstages) * stage_smem_stride(np_of(p), 3 * (p + 1), epc, Qp, s_bytes, r_bytes);
+  return size_t(nstages) *
+         stage_smem_stride(np_of(p), 3 * (p + 1), epc, Qp, s_bytes, r_bytes, stage_direct_traces(p, store_kind, Qp));
 }
 
 }  // namespace fedbm

@@ -22,8 +22,8 @@
 //   4. residual and update, one thread per (element, velocity) item, with
 //      Dr, Ds, LIFT as instruction immediates (compile-time tables) or
 //      constant-memory operands of unrolled FMAs on the even and odd parts of f
-//      and of the flux (stage_eo.cuh; the 16-bit forms at degree 3 take two
-//      velocities per thread as packed FP32 pairs, fma.rn.f32x2);
+//      and of the flux (stage_eo.cuh); the FP32 and 16-bit states take two
+//      velocities per thread as packed FP32 pairs;
 //   5. deviation forms only: per-element scale from max |f/w - 1|, encode;
 //   6. bulk-store the new state and residual tiles.
 #include "device_common.cuh"
@@ -32,19 +32,6 @@
 #include <cstring>
 #include <type_traits>
 
-// Degree at which the 16-bit forms take two velocities per thread as packed FP32
-// pairs, whose broadcast operators come from constant memory.  With the even-odd
-// contractions (GB300): BF16 cavity at 1,024 velocities, degree 3, 22.6 ms for a
-// two-step call against 24.7 ms with one velocity per thread and the operators as
-// immediates; FP16 at 256 velocities, degree 2, 640 us against 593 us.
-#ifndef FEDBM_VPT2_P
-#define FEDBM_VPT2_P 3
-#endif
-// FEDBM_FACE_SKIP = 0: the FMA kernel evaluates every face's flux and lift
-// columns also where a whole warp leaves an element through the face
-#ifndef FEDBM_FACE_SKIP
-#define FEDBM_FACE_SKIP 1
-#endif
 
 #ifndef FEDBM_P
 #error "FEDBM_P must be defined"
@@ -248,9 +235,52 @@ __host__ __device__ constexpr int moment_lanes(int nth, int epc, int nchunk) {
   return G;
 }
 
+// Node record: f^eq_i / tau = w_i [m0 + e_x m1 + e_y m2 + m3 (e.u)^2
+// + (e.u)(m6 (e.u)^2 - m7)] with e.u = e_x m4 + e_y m5 (eq. feq; the m6, m7 terms
+// are the third Hermite order of eq. Herm3a and vanish for eq_order 2); `it` is
+// 1/tau of the element's case.
+template <typename R>
+__device__ __forceinline__ void node_record(R rho, R jx, R jy, R it, bool third, R (&m)[8]) {
+  const R irho = R(1) / rho;
+  const R ux = jx * irho, uy = jy * irho, uu = ux * ux + uy * uy;
+  m[0] = rho * (R(1) - R(0.5) * uu) * it;
+  m[1] = jx * it;
+  m[2] = jy * it;
+  m[3] = R(0.5) * rho * it;
+  m[4] = ux;
+  m[5] = uy;
+  m[6] = third ? rho * it * R(1.0 / 6.0) : R(0);
+  m[7] = third ? R(0.5) * rho * uu * it : R(0);
+}
+
+// How a tile keeps its node records: eight values in the compute precision R; or,
+// for the kernels that take two velocities per thread, times the time step and with
+// -m7, either as eight floats or as six packed pairs (each value twice) with the
+// pairs (m6, -m7) of all nodes behind them.
+enum RecordForm { kRecPlain, kRecStep, kRecPairs };
+constexpr int kRecPairFloats = 12;
+template <RecordForm F, typename R>
+__device__ __forceinline__ void store_record(R* s_mom, int node, int nodes, R rho, R jx, R jy, const R* geo,
+                                             bool third) {
+  R m[8];
+  node_record(rho, jx, jy, F == kRecPlain ? geo[kGeoInvTau] : geo[kGeoInvTau] * geo[kGeoDt], third, m);
+  if constexpr (F == kRecPairs) {
+    float4* r = reinterpret_cast<float4*>(s_mom + size_t(node) * kRecPairFloats);
+    r[0] = make_float4(m[0], m[0], m[1], m[1]);
+    r[1] = make_float4(m[2], m[2], m[3], m[3]);
+    r[2] = make_float4(m[4], m[4], m[5], m[5]);
+    reinterpret_cast<float2*>(s_mom + size_t(nodes) * kRecPairFloats)[node] = make_float2(m[6], -m[7]);
+  } else {
+    R* mm = s_mom + size_t(node) * 8;
+#pragma unroll
+    for (int j = 0; j < 7; ++j) mm[j] = m[j];
+    mm[7] = F == kRecStep ? -m[7] : m[7];
+  }
+}
+
 // NTH > 0: a CTA of NTH threads and EPC elements per tile (the tensor-core
 // kernel), so the lane grouping and the chunk loop are compile-time.
-template <class ST, class Acc, int QT, int NTH = 0, int EPC = 1>
+template <class ST, class Acc, int QT, int NTH = 0, int EPC = 1, RecordForm F = kRecPlain>
 __device__ void tile_moments(const StageArgs<typename ST::R>& a, const typename ST::S* s_f,
                              const float* s_scale, const typename ST::R* s_geo, typename ST::R* s_mom, int ne,
                              const typename ST::R* s_vel) {
@@ -260,7 +290,14 @@ __device__ void tile_moments(const StageArgs<typename ST::R>& a, const typename 
   static_assert(NTH == 0 || QT > 0, "a compile-time CTA needs a compile-time velocity count");
   const int Qp = QT > 0 ? QT : a.Qp, tid = threadIdx.x, nth = NTH > 0 ? NTH : blockDim.x;
   const int nchunk = Qp / V;
-  const int G = NTH > 0 ? moment_lanes(NTH, EPC, (QT > 0 ? QT : 1) / V) : moment_lanes(nth, a.epc, nchunk);
+  // below 128 velocities, where the tile depends on the element count, the lanes per
+  // node do not: a case gives the same bits in a batch and on its own.  As many as the
+  // usual tiles leave per node; few in FP64, whose additions are slow.
+  constexpr bool kFew = QT == 0 && sizeof(R) == 8;
+  const int want = kFew && Qp == 16 ? (P <= 1 ? 4 : P == 2 ? 2 : 1) : P <= 1 ? 8 : P <= 3 ? 4 : 2;
+  const int short_lanes = QT == 16 ? 1 : min(pow2_floor_32(nchunk), want);
+  const int G = NTH > 0 ? moment_lanes(NTH, EPC, (QT > 0 ? QT : 1) / V)
+                        : Qp < 128 ? short_lanes : moment_lanes(nth, a.epc, nchunk);
   const int ngroups = nth / G, grp = tid / G, lane = tid % G;
   const int npair = ne * NP;
   const R* ex = s_vel + kVelEx * Qp;  // shared-memory copy of the velocity rows
@@ -270,42 +307,100 @@ __device__ void tile_moments(const StageArgs<typename ST::R>& a, const typename 
     const int pair = base + grp;
     const bool valid = pair < npair;
     Acc m0, m1, m2;
-    if (valid) {
-      const S* row = s_f + size_t(pair) * Qp;
-      auto chunk = [&](int c) {
-        __align__(16) S v[V];
-        __align__(16) R exv[V], eyv[V], wvv[V];
-        *reinterpret_cast<uint4*>(v) = *reinterpret_cast<const uint4*>(row + c * V);
+    const S* row = s_f + size_t(valid ? pair : 0) * Qp;
+    // packed sums of one chunk, added to p0, p1, p2
+    unsigned long long p0 = 0, p1 = 0, p2 = 0;
+    auto chunk_pairs = [&](int c) {
+      __align__(16) S v[V];
+      *reinterpret_cast<uint4*>(v) = *reinterpret_cast<const uint4*>(row + c * V);
 #pragma unroll
-        for (int j = 0; j < V * int(sizeof(R)) / 16; ++j) {
-          reinterpret_cast<uint4*>(exv)[j] = reinterpret_cast<const uint4*>(ex + c * V)[j];
-          reinterpret_cast<uint4*>(eyv)[j] = reinterpret_cast<const uint4*>(ey + c * V)[j];
-          if constexpr (ST::dev) reinterpret_cast<uint4*>(wvv)[j] = reinterpret_cast<const uint4*>(wv + c * V)[j];
+      for (int j = 0; j < V; j += 2) {
+        const unsigned long long x = *reinterpret_cast<const unsigned long long*>(ex + c * V + j);
+        const unsigned long long y = *reinterpret_cast<const unsigned long long*>(ey + c * V + j);
+        unsigned long long f;
+        if constexpr (ST::dev) {
+          f = f2mul(*reinterpret_cast<const unsigned long long*>(wv + c * V + j),
+                    f2pack(ST::to_r(v[j]), ST::to_r(v[j + 1])));
+        } else {
+          f = f2pack(v[j], v[j + 1]);
         }
-        // sums over the chunk in the compute precision, then one accumulator
-        // update per chunk (FP64 or compensated across chunks)
+        p0 = EoPacked::add(p0, f);
+        p1 = f2fma(x, f, p1);
+        p2 = f2fma(y, f, p2);
+      }
+    };
+    auto add_pairs = [&](Acc& a0, Acc& a1, Acc& a2) {
+      float lo, hi;
+      f2unpack(p0, lo, hi);
+      a0.add(lo + hi);
+      f2unpack(p1, lo, hi);
+      a1.add(lo + hi);
+      f2unpack(p2, lo, hi);
+      a2.add(lo + hi);
+    };
+    // sums over a chunk in the compute precision, then one accumulator update
+    auto chunk = [&](int c, Acc& a0, Acc& a1, Acc& a2) {
+      if constexpr (sizeof(R) == 4) {
+        p0 = p1 = p2 = 0ull;
+        chunk_pairs(c);
+        add_pairs(a0, a1, a2);
+      } else {
+        __align__(16) S v[V];
+        *reinterpret_cast<uint4*>(v) = *reinterpret_cast<const uint4*>(row + c * V);
         R c0 = 0, c1 = 0, c2 = 0;
 #pragma unroll
         for (int j = 0; j < V; ++j) {
-          R f;
-          if constexpr (ST::dev) f = wvv[j] * ST::to_r(v[j]);
-          else f = v[j];
-          c0 += f;
-          c1 = fma(exv[j], f, c1);
-          c2 = fma(eyv[j], f, c2);
+          c0 += v[j];
+          c1 = fma(ex[c * V + j], v[j], c1);
+          c2 = fma(ey[c * V + j], v[j], c2);
         }
-        m0.add(c0);
-        m1.add(c1);
-        m2.add(c2);
-      };
+        a0.add(c0);
+        a1.add(c1);
+        a2.add(c2);
+      }
+    };
+    // FP32 sums keep their packed pairs over the row
+    constexpr bool kPairSums = std::is_same<Acc, AccF>::value && sizeof(R) == 4;
+    auto take = [&](int c) {
+      if constexpr (kPairSums) chunk_pairs(c);
+      else chunk(c, m0, m1, m2);
+    };
+    if (valid) {
       if constexpr (NTH > 0) {
         constexpr int GC = moment_lanes(NTH > 0 ? NTH : 1, EPC, (QT > 0 ? QT : V) / V);
 #pragma unroll 8
-        for (int c = 0; c < (QT > 0 ? QT : V) / V; c += GC) chunk(c + lane);
+        for (int c = 0; c < (QT > 0 ? QT : V) / V; c += GC) take(c + lane);
+      } else if constexpr (QT == 16 && kPairSums) {
+        // one lane per node: neighbouring lanes' rows start in the same banks, so each
+        // takes its chunks from another one on; summing over distances N/2, .., 1 gives
+        // the same for every rotation
+        constexpr int N = 16 / V;
+        const int first = pair * 16 * int(sizeof(S)) / 128;
+        unsigned long long q0[N], q1[N], q2[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+          p0 = p1 = p2 = 0ull;
+          chunk_pairs((j + first) & (N - 1));
+          q0[j] = p0;
+          q1[j] = p1;
+          q2[j] = p2;
+        }
+#pragma unroll
+        for (int off = N / 2; off > 0; off >>= 1)
+#pragma unroll
+          for (int j = 0; j < off; ++j) {
+            q0[j] = EoPacked::add(q0[j], q0[j + off]);
+            q1[j] = EoPacked::add(q1[j], q1[j + off]);
+            q2[j] = EoPacked::add(q2[j], q2[j + off]);
+          }
+        p0 = q0[0];
+        p1 = q1[0];
+        p2 = q2[0];
       } else {
-        for (int c = lane; c < nchunk; c += G) chunk(c);
+        for (int c = lane; c < nchunk; c += G) take(c);
       }
     }
+    if constexpr (kPairSums) add_pairs(m0, m1, m2);
     m0.reduce(G);
     m1.reduce(G);
     m2.reduce(G);
@@ -322,22 +417,7 @@ __device__ void tile_moments(const StageArgs<typename ST::R>& a, const typename 
         jx = R(m1.value());
         jy = R(m2.value());
       }
-      // f^eq_i / tau = w_i [m0 + e_x m1 + e_y m2 + m3 (e.u)^2 + (e.u)(m6 (e.u)^2 - m7)]
-      // with e.u = e_x m4 + e_y m5 (eq. feq; the m6, m7 terms are the third
-      // Hermite order of eq. Herm3a and vanish for eq_order 2)
-      const R irho = R(1) / rho;
-      const R it = s_geo[(pair / NP) * kGeoStrideDev + kGeoInvTau];  // 1/tau of the element's case
-      const R ux = jx * irho, uy = jy * irho, uu = ux * ux + uy * uy;
-      const bool third = a.eq_order == 3;
-      R* mm = s_mom + size_t(pair) * 8;
-      mm[0] = rho * (R(1) - R(0.5) * uu) * it;
-      mm[1] = jx * it;
-      mm[2] = jy * it;
-      mm[3] = R(0.5) * rho * it;
-      mm[4] = ux;
-      mm[5] = uy;
-      mm[6] = third ? rho * it * R(1.0 / 6.0) : R(0);
-      mm[7] = third ? R(0.5) * rho * uu * it : R(0);
+      store_record<F>(s_mom, pair, a.epc * NP, rho, jx, jy, s_geo + (pair / NP) * kGeoStrideDev, a.eq_order == 3);
     }
   }
 }
@@ -350,36 +430,42 @@ __device__ void tile_wall_numerators(const StageArgs<typename ST::R>& a, const t
                                      const typename ST::R* s_vel) {
   using R = typename ST::R;
   const int Qp = QT > 0 ? QT : a.Qp, tid = threadIdx.x, nth = blockDim.x;
-  const int G = pow2_floor_32(nth / (a.epc * NF));
+  // lanes per wall node: a fixed number, so that the sum has one order whatever the tile
+  const int G = Qp < 128 ? 8 : 32;
   const int ngroups = nth / G, grp = tid / G, lane = tid % G;
-  const int ntrip = ne * NF;
   const R* ex = s_vel + kVelEx * Qp;  // shared-memory copy of the velocity rows
   const R* ey = s_vel + kVelEy * Qp;
   const R* wv = s_vel + kVelW * Qp;
-  for (int base = 0; base < ntrip; base += ngroups) {
-    const int trip = base + grp;
-    const int e = trip / NF, fc = (trip % NF) / NFP, aa = trip % NFP;
-    bool active = false;
-    if (trip < ntrip) {
-      const int code = s_nbr[e * 3 + fc];
-      active = code < 0 && __ldg(a.wall_den_inv + (-code - 1)) > R(0);
+  // most tiles have no wall: every warp looks for the tile's wall faces, 32 at a time
+  for (int f0 = 0; f0 < ne * 3; f0 += 32) {
+    const int mine = f0 + (tid & 31);
+    bool wall = false;
+    if (mine < ne * 3) {
+      const int code = s_nbr[mine];
+      wall = code < 0 && __ldg(a.wall_den_inv + (-code - 1)) > R(0);
     }
-    R acc = 0;
-    if (active) {
+    for (unsigned mask = __ballot_sync(kFull, wall); mask; mask &= mask - 1) {
+      const int face = f0 + __ffs(mask) - 1, e = face / 3, fc = face - 3 * e;
       const R nxf = s_geo[e * kGeoStrideDev + 4 + 3 * fc];
       const R nyf = s_geo[e * kGeoStrideDev + 5 + 3 * fc];
-      const int rs = aa * (P + 1) - aa * (aa - 1) / 2;
-      const int node = (fc == 0) ? aa : (fc == 1 ? rs + (P - aa) : rs);
-      const typename ST::S* row = s_f + (size_t(e) * NP + node) * Qp;
       const R sc = ST::dev ? s_scale[e] : R(0);
-      for (int i = lane; i < Qp; i += G) {
-        const R en = ex[i] * nxf + ey[i] * nyf;
-        const R w = ST::dev ? wv[i] : R(0);  // the plain forms do not use (or hold) the w row
-        if (en > 0) acc += en * decode<ST>(row[i], w, w * sc);
+      for (int base = 0; base < NFP; base += ngroups) {
+        const int aa = base + grp;
+        R acc = 0;
+        if (aa < NFP) {
+          const int rs = aa * (P + 1) - aa * (aa - 1) / 2;
+          const int node = (fc == 0) ? aa : (fc == 1 ? rs + (P - aa) : rs);
+          const typename ST::S* row = s_f + (size_t(e) * NP + node) * Qp;
+          for (int i = lane; i < Qp; i += G) {
+            const R en = ex[i] * nxf + ey[i] * nyf;
+            const R w = ST::dev ? wv[i] : R(0);  // the plain forms do not use (or hold) the w row
+            if (en > 0) acc += en * decode<ST>(row[i], w, w * sc);
+          }
+        }
+        for (int off = G >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(kFull, acc, off);
+        if (aa < NFP && lane == 0) s_wn[(e * 3 + fc) * NFP + aa] = acc;
       }
     }
-    for (int off = G >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(kFull, acc, off);
-    if (active && lane == 0) s_wn[trip] = acc;
   }
 }
 
@@ -411,216 +497,272 @@ __host__ __device__ constexpr bool keeps_scale() {
   else return false;
 }
 
-// Adjacent velocities handled by one thread in phase 4: two for the
-// specialised 16-bit-state kernels at degree FEDBM_VPT2_P (each operator constant
-// then feeds two FMAs and the per-item set-up is shared), else one.
-template <class ST, int QT>
-__host__ __device__ constexpr int items_vpt() {
-  return (QT > 0 && sizeof(typename ST::R) == 4 && ST::dev && P == FEDBM_VPT2_P)
-             ? 2
-             : 1;
+// Node of face node aa of the neighbour that face code `code` (>= 0) names: its face
+// (code >> 1) & 3, listed backwards where bit 0 is set.
+__device__ __forceinline__ int trace_node(int code, int aa) {
+  const int fn = (code >> 1) & 3;
+  const int a2 = (code & 1) ? NFP - 1 - aa : aa;
+  const int rs = a2 * (P + 1) - a2 * (a2 - 1) / 2;
+  return fn == 0 ? a2 : (fn == 1 ? rs + (P - a2) : rs);
 }
 
-template <typename T, int N>
-struct alignas(N * sizeof(T)) Vec {
-  T v[N];
-};
+// With 16 velocities a face row is 64 bytes (FP32) or 32: copied row by row into
+// shared memory, the copies' issue took 6 % of the kernel's instructions (about 90
+// per element) and their tiles 30 % of its shared memory, though a velocity uses
+// only the faces it enters through.  There the update reads its own traces from
+// global memory (L2), eight lanes to a row.
+template <class ST, int QT>
+__host__ __device__ constexpr bool direct_traces() {
+  return QT > 0 && stage_direct_traces(P, ST::kind, QT);
+}
+template <class ST, int QT>
+__host__ __device__ constexpr RecordForm record_form() {
+  return sizeof(typename ST::R) == 8 ? kRecPlain : direct_traces<ST, QT>() ? kRecPairs : kRecStep;
+}
 
-// Phase 4: residual, 2N-storage update and write-back of every (element,
-// velocity) value of the tile; each thread owns VPT adjacent velocities of one
-// element.  Plain forms and BF16 (kept element scale) update f in place in
-// shared memory; FP16 only tracks max |f/w - 1| per element (the encoding pass
-// recomputes f with the new scale).
-template <class ST, int QT, int VPT>
-__device__ __forceinline__ void item_update(const StageArgs<typename ST::R>& a,
-                                            StageSmem<typename ST::R, typename ST::S>& sm, int64_t k0, int ne,
-                                            bool read_res, float& dmax, int& emax) {
+// Phase 4, FP64 state: residual, 2N-storage update and write-back of every
+// (element, velocity) value of the tile, one velocity of one element per thread, f
+// and the residual updated in place in shared memory.
+template <class ST, int QT>
+__device__ __forceinline__ void value_update(const StageArgs<typename ST::R>& a,
+                                             StageSmem<typename ST::R, typename ST::S>& sm, int ne, bool read_res) {
   using R = typename ST::R;
-  using S = typename ST::S;
-  using SV = Vec<S, VPT>;
-  using RV = Vec<R, VPT>;
+  static_assert(sizeof(R) == 8 && !ST::dev, "the FP64 state");
   const int Qp = QT > 0 ? QT : a.Qp;
-  const int Qv = Qp / VPT;
-  const int tid = threadIdx.x, nth = blockDim.x;
   const R rkA = a.rkA, rkB = a.rkB, ab = a.ab;
   const bool third = a.eq_order == 3;
-  constexpr bool kPacked = VPT == 2;
-  constexpr bool kImm = ops_immediate<ST, QT>();
-  // outflow faces skipped per warp where a warp's items belong to one element
-  // (one velocity per thread: with two, the packed lift accumulators measured
-  // slower, 2.26e11 vs 2.37e11 on the BF16 NC 32x32 cavity)
-  constexpr bool kSkip = FEDBM_FACE_SKIP && QT >= 128 && VPT == 1;
+  for (int item = threadIdx.x; item < ne * Qp; item += blockDim.x) {
+    const int e = item / Qp, i = item - e * Qp;
+    const R ex = a.vel[kVelEx * Qp + i], ey = a.vel[kVelEy * Qp + i], w = a.vel[kVelW * Qp + i];
+    const R* g = sm.geo + e * kGeoStrideDev;
+    const R dt = g[kGeoDt], inv_tau = g[kGeoInvTau];  // per element: cases of a batch differ
+    const R ar = ex * g[0] + ey * g[2], as = ex * g[1] + ey * g[3];
+    R* frow = sm.f + size_t(e) * NP * Qp + i;
+    R* rrow = sm.res + size_t(e) * NP * Qp + i;
+    R fr[NP];
+#pragma unroll
+    for (int m = 0; m < NP; ++m) fr[m] = frow[m * Qp];
+    R flux[NF];
+#pragma unroll
+    for (int fc = 0; fc < 3; ++fc) {
+      const R en = ex * g[4 + 3 * fc] + ey * g[5 + 3 * fc];
+      const R c = R(0.5) * (en - ab * fabs(en)) * g[6 + 3 * fc];
+      const int code = sm.nbr[e * 3 + fc];
+      if (code >= 0) {
+        const R* trow = sm.tr + size_t(e * NF + fc * NFP) * Qp + i;
+#pragma unroll
+        for (int aa = 0; aa < NFP; ++aa) flux[fc * NFP + aa] = c * (fr[face_node(fc, aa)] - trow[aa * Qp]);
+      } else {
+        const int slot = -code - 1;  // wall slot: 4 * case + side
+        const R fb = a.wall_feq[slot * Qp + i];
+        const R den_inv = __ldg(a.wall_den_inv + slot);
+        const bool diffuse = den_inv > R(0);
+        // incoming velocities take the wall state; outgoing ones have no jump
+        const R scale = diffuse ? den_inv * fb : R(0);
+#pragma unroll
+        for (int aa = 0; aa < NFP; ++aa) {
+          const R fp = diffuse ? sm.wn[e * NF + fc * NFP + aa] * scale : fb;
+          flux[fc * NFP + aa] = en < R(0) ? c * (fr[face_node(fc, aa)] - fp) : R(0);
+        }
+      }
+    }
+    using M = EoScalar<R, false>;
+    R le[NE], lo[at_least_1(NO)];
+    eo_lift<M>(flux, true, true, le, lo);
+    eo_volume<M>([&](int n) { return fr[n]; }, R(-0.5) * (ar + as), R(0.5) * (ar - as), le, lo, [&](int n, R adv) {
+      // f itself from shared memory again, which keeps the registers within two
+      // resident CTAs of 256 threads
+      const R f = frow[n * Qp];
+      const R rhs = adv + collision<R>(sm.mom + (size_t(e) * NP + n) * 8, ex, ey, w, f, inv_tau, third);
+      R r = dt * rhs;
+      if (read_res) r = fma(rkA, rrow[n * Qp], r);
+      rrow[n * Qp] = r;
+      frow[n * Qp] = new_f<ST>(f, rkB, r);
+    });
+  }
+}
+
+// Two adjacent stored values as an FP32 pair, the lower velocity in the low half.
+using Pair = unsigned long long;
+__device__ __forceinline__ Pair both(float x) { return f2pack(x, x); }
+template <class ST>
+__device__ __forceinline__ Pair raw_pair(const typename ST::S* p) {
+  if constexpr (ST::kind == kStoreBF16) {
+    const uint32_t q = *reinterpret_cast<const uint32_t*>(p);  // BF16: the upper half of an FP32
+    return f2pack(__uint_as_float(q << 16), __uint_as_float(q & 0xffff0000u));
+  } else if constexpr (ST::kind == kStoreF16) {
+    const float2 x = __half22float2(*reinterpret_cast<const __half2*>(p));
+    return f2pack(x.x, x.y);
+  } else {
+    return *reinterpret_cast<const Pair*>(p);
+  }
+}
+// decoded: f, or w + (w s) q
+template <class ST>
+__device__ __forceinline__ Pair value_pair(const typename ST::S* p, Pair w, Pair ws) {
+  if constexpr (ST::dev) return f2fma(ws, raw_pair<ST>(p), w);
+  else return raw_pair<ST>(p);
+}
+
+// Phase 4, FP32 arithmetic: residual, 2N-storage update and write-back of every
+// (element, velocity) value of the tile; each thread owns two adjacent velocities
+// of one element.  Additions, collision, update, loads and stores act on packed
+// FP32 pairs, the contractions on their halves with the operators as immediates;
+// the time step is folded into the operators' factors, the flux coefficients and
+// the node records.  Plain forms and BF16 (kept element scale) update f in place
+// in shared memory; FP16 only tracks max |f/w - 1| per element (the encoding pass
+// recomputes f with the new scale).
+template <class ST, int QT>
+__device__ __forceinline__ void pair_update(const StageArgs<float>& a, StageSmem<float, typename ST::S>& sm,
+                                            int64_t k0, int ne, bool read_res, float& dmax, int& emax) {
+  using S = typename ST::S;
+  using M = EoDual<kHaveOpsTable>;
+  constexpr bool kDirect = direct_traces<ST, QT>();
   constexpr bool kKeep = keeps_scale<ST>();
   constexpr bool kTrack = ST::dev && !kKeep;
+  // outflow faces skipped per warp where a warp's items belong to one element
+  constexpr bool kSkip = QT >= 128;
+  const int Qp = QT > 0 ? QT : a.Qp, Qv = Qp / 2;
+  const Pair rkA2 = both(a.rkA), rkB2 = both(a.rkB);
+  const float ab = a.ab;
+  const bool third = a.eq_order == 3;
+  const S* fin = static_cast<const S*>(a.f_in);
   // stochastic rounding of the BF16 encode: the step counter is read once
   const bool sr = kKeep && a.sr_step != nullptr;
   const uint32_t sr_step = sr ? __ldg(a.sr_step) : 0u;
-  for (int item = tid; item < ne * Qv; item += nth) {
-    const int e = item / Qv;
-    const int i = (item - e * Qv) * VPT;
-    const RV exv = *reinterpret_cast<const RV*>(a.vel + kVelEx * Qp + i);
-    const RV eyv = *reinterpret_cast<const RV*>(a.vel + kVelEy * Qp + i);
-    const RV wv = *reinterpret_cast<const RV*>(a.vel + kVelW * Qp + i);
-    const R* g = sm.geo + e * kGeoStrideDev;
-    const R dt = g[kGeoDt], inv_tau = g[kGeoInvTau];  // per element: cases of a batch differ
-    R ar[VPT], as[VPT], ws[VPT];
-#pragma unroll
-    for (int v = 0; v < VPT; ++v) {
-      ar[v] = exv.v[v] * g[0] + eyv.v[v] * g[2];
-      as[v] = exv.v[v] * g[1] + eyv.v[v] * g[3];
-      ws[v] = ST::dev ? wv.v[v] * R(sm.scale[e]) : R(0);
-    }
-    S* frow = sm.f + size_t(e) * NP * Qp + i;
-    R* rrow = sm.res + size_t(e) * NP * Qp + i;
-
-    R fr[VPT][NP];
-#pragma unroll
-    for (int m = 0; m < NP; ++m) {
-      const SV x = *reinterpret_cast<const SV*>(frow + m * Qp);
-#pragma unroll
-      for (int v = 0; v < VPT; ++v) fr[v][m] = decode<ST>(x.v[v], wv.v[v], ws[v]);
-    }
-
-    R flux[VPT][NF];
-    // kSkip: face fc carries flux for some velocity of the lanes running this
-    // iteration together (an outflow face's upwind jump term is zero), else
-    // its traces and lift columns are skipped
-    bool on[3];
+  for (int item = threadIdx.x; item < ne * Qv; item += blockDim.x) {
+    const int e = item / Qv, i = 2 * (item - e * Qv);
+    const Pair ex = *reinterpret_cast<const Pair*>(sm.vel + kVelEx * Qp + i);
+    const Pair ey = *reinterpret_cast<const Pair*>(sm.vel + kVelEy * Qp + i);
+    const Pair w = *reinterpret_cast<const Pair*>(sm.vel + kVelW * Qp + i);
+    const float* g = sm.geo + e * kGeoStrideDev;
+    const float dt = g[kGeoDt];  // per element: cases of a batch differ
+    const int* nb = sm.nbr + e * 3;
+    // flux coefficients dt (e.n - ab |e.n|) Fscale / 2 of the three faces
+    Pair c[3];
+    bool on[3], nz[3];
 #pragma unroll
     for (int fc = 0; fc < 3; ++fc) {
-      R c[VPT], en[VPT];
-#pragma unroll
-      for (int v = 0; v < VPT; ++v) {
-        en[v] = exv.v[v] * g[4 + 3 * fc] + eyv.v[v] * g[5 + 3 * fc];
-        c[v] = R(0.5) * (en[v] - ab * fabs(en[v])) * g[6 + 3 * fc];
+      float e0, e1;
+      f2unpack(f2fma(ey, both(g[5 + 3 * fc]), f2mul(ex, both(g[4 + 3 * fc]))), e0, e1);
+      const float h = 0.5f * dt * g[6 + 3 * fc];
+      float c0 = h * fmaf(-ab, fabsf(e0), e0), c1 = h * fmaf(-ab, fabsf(e1), e1);
+      if (nb[fc] < 0) {  // incoming velocities take the wall state; outgoing ones have no jump
+        c0 = e0 < 0.f ? c0 : 0.f;
+        c1 = e1 < 0.f ? c1 : 0.f;
       }
-      const int code = sm.nbr[e * 3 + fc];
-      on[fc] = true;
+      c[fc] = f2pack(c0, c1);
+      nz[fc] = c0 != 0.f || c1 != 0.f;
+      on[fc] = kSkip ? __any_sync(__activemask(), nz[fc]) : true;
+    }
+    // 16 velocities: the traces of the faces with flux straight from global memory,
+    // all of them in flight before the first is used
+    Pair tr[kDirect ? NF : 1];
+    if constexpr (kDirect) {
+      const uint32_t* rows = reinterpret_cast<const uint32_t*>(sm.tr) + e * NF;
+#pragma unroll
+      for (int fc = 0; fc < 3; ++fc)
+#pragma unroll
+        for (int aa = 0; aa < NFP; ++aa)
+          tr[fc * NFP + aa] = nz[fc] && nb[fc] >= 0 ? raw_pair<ST>(fin + size_t(rows[fc * NFP + aa]) * QT + i) : 0ull;
+    }
+    const Pair ws = ST::dev ? f2mul(w, both(sm.scale[e])) : 0ull;
+    S* frow = sm.f + size_t(e) * NP * Qp + i;
+    float* rrow = sm.res + size_t(e) * NP * Qp + i;
+    Pair fr[NP];
+#pragma unroll
+    for (int m = 0; m < NP; ++m) fr[m] = value_pair<ST>(frow + m * Qp, w, ws);
+    Pair flux[NF];
+#pragma unroll
+    for (int fc = 0; fc < 3; ++fc) {
+      const int code = nb[fc];
       if constexpr (kSkip) {
-        bool nz = false;
 #pragma unroll
-        for (int v = 0; v < VPT; ++v) nz = nz || (c[v] != R(0) && (code >= 0 || en[v] < R(0)));
-        on[fc] = __any_sync(__activemask(), nz);
-#pragma unroll
-        for (int v = 0; v < VPT; ++v)
-#pragma unroll
-          for (int aa = 0; aa < NFP; ++aa) flux[v][fc * NFP + aa] = R(0);
+        for (int aa = 0; aa < NFP; ++aa) flux[fc * NFP + aa] = 0ull;
         if (!on[fc]) continue;
       }
       if (code >= 0) {
-        R wsn[VPT];
-#pragma unroll
-        for (int v = 0; v < VPT; ++v) wsn[v] = ST::dev ? wv.v[v] * R(sm.nscale[e * 3 + fc]) : R(0);
+        const Pair wsn = ST::dev ? f2mul(w, both(sm.nscale[e * 3 + fc])) : 0ull;
         const S* trow = sm.tr + size_t(e * NF + fc * NFP) * Qp + i;
 #pragma unroll
         for (int aa = 0; aa < NFP; ++aa) {
-          const SV x = *reinterpret_cast<const SV*>(trow + aa * Qp);
-#pragma unroll
-          for (int v = 0; v < VPT; ++v)
-            flux[v][fc * NFP + aa] = c[v] * (fr[v][face_node(fc, aa)] - decode<ST>(x.v[v], wv.v[v], wsn[v]));
+          Pair t;
+          if constexpr (kDirect) t = ST::dev ? f2fma(wsn, tr[fc * NFP + aa], w) : tr[fc * NFP + aa];
+          else t = value_pair<ST>(trow + aa * Qp, w, wsn);
+          flux[fc * NFP + aa] = f2mul(c[fc], EoPacked::sub(fr[face_node(fc, aa)], t));
         }
       } else {
         const int slot = -code - 1;  // wall slot: 4 * case + side
-        const RV fbv = *reinterpret_cast<const RV*>(a.wall_feq + slot * Qp + i);
-        const R den_inv = __ldg(a.wall_den_inv + slot);
-        const bool diffuse = den_inv > R(0);
+        const Pair fb = *reinterpret_cast<const Pair*>(a.wall_feq + size_t(slot) * Qp + i);
+        const float den_inv = __ldg(a.wall_den_inv + slot);
+        const bool diffuse = den_inv > 0.f;
+        const Pair fd = f2mul(both(den_inv), fb);
 #pragma unroll
-        for (int v = 0; v < VPT; ++v) {
-          // incoming velocities take the wall state; outgoing ones have no jump
-          const R scale = diffuse ? den_inv * fbv.v[v] : R(0);
-#pragma unroll
-          for (int aa = 0; aa < NFP; ++aa) {
-            const R fp = diffuse ? sm.wn[e * NF + fc * NFP + aa] * scale : fbv.v[v];
-            flux[v][fc * NFP + aa] = en[v] < R(0) ? c[v] * (fr[v][face_node(fc, aa)] - fp) : R(0);
-          }
+        for (int aa = 0; aa < NFP; ++aa) {
+          const Pair fp = diffuse ? f2mul(both(sm.wn[e * NF + fc * NFP + aa]), fd) : fb;
+          flux[fc * NFP + aa] = f2mul(c[fc], EoPacked::sub(fr[face_node(fc, aa)], fp));
         }
       }
     }
-
-    using M = std::conditional_t<kPacked, EoPacked, EoScalar<R, kImm>>;
-    using T = typename M::T;
-    constexpr int NT = kPacked ? 1 : VPT;  // contractions per item
-    auto pack = [](const R* x) -> T {
-      if constexpr (kPacked) return f2pack(x[0], x[VPT - 1]);
-      else return x[0];
-    };
-    // even and odd parts of LIFT flux (the faces without flux skipped)
-    T le[NT][NE], lo[NT][at_least_1(NO)];
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      T fl[NF];
-#pragma unroll
-      for (int q = 0; q < NF; ++q) {
-        const R x[2] = {flux[t][q], flux[kPacked ? VPT - 1 : t][q]};
-        fl[q] = pack(x);
-      }
-      eo_lift<M>(fl, on[0] || on[2], on[1], le[t], lo[t]);
-    }
+    Pair le[NE], lo[at_least_1(NO)];
+    eo_lift<M>(flux, on[0] || on[2], on[1], le, lo);
+    const Pair neg_k = both(-dt * g[kGeoInvTau]);
+    const Pair ar = f2fma(ey, both(g[2]), f2mul(ex, both(g[0]))), as = f2fma(ey, both(g[3]), f2mul(ex, both(g[1])));
+    const Pair na = f2mul(both(-0.5f * dt), EoPacked::add(ar, as)), nd = f2mul(both(0.5f * dt), EoPacked::sub(ar, as));
+    Pair invw = 0ull;
+    if constexpr (ST::dev)  // BF16 keeps the element's power-of-two scale: q = (f - w) / (w s)
+      invw = f2mul(*reinterpret_cast<const Pair*>(a.vel + kVelInvW * Qp + i),
+                   both(kKeep ? 1.0f / sm.scale[e] : 1.0f));
     float dloc = 0.f;
-    R invw[VPT];
-    if constexpr (ST::dev) {
-      const RV iw = *reinterpret_cast<const RV*>(a.vel + kVelInvW * Qp + i);
-#pragma unroll
-      for (int v = 0; v < VPT; ++v) invw[v] = iw.v[v] * (kKeep ? R(1) / R(sm.scale[e]) : R(1));
-    }
-    // rhs, update and write-back of node n from its advection term
+    // update and write-back of node n from dt times its advection term
     // -(e . grad) f + LIFT (flux)
-    auto finish = [&](int n, const R* adv) {
-      RV rold;
-      if (read_res) rold = *reinterpret_cast<const RV*>(rrow + n * Qp);
-      // f itself from shared memory again: next to its even and odd parts the
-      // registers would not hold it without giving up a resident CTA (FP32 at
-      // degree 3, 36 velocities: 72 registers against 79, 7 CTAs against 6)
-      const SV fs = *reinterpret_cast<const SV*>(frow + n * Qp);
-      R fn[VPT];
-#pragma unroll
-      for (int v = 0; v < VPT; ++v) fn[v] = decode<ST>(fs.v[v], wv.v[v], ws[v]);
-      const R* mm = sm.mom + (size_t(e) * NP + n) * 8;
-      RV rr;
-      SV fnew_s;
-#pragma unroll
-      for (int v = 0; v < VPT; ++v) {
-        R rhs = adv[v];
-        rhs += collision<R>(mm, exv.v[v], eyv.v[v], wv.v[v], fn[v], inv_tau, third);
-        R r = dt * rhs;
-        if (read_res) r = fma(rkA, rold.v[v], r);
-        rr.v[v] = r;
-        const R fnew = new_f<ST>(fn[v], rkB, r);
-        if constexpr (kTrack) {
-          dloc = fmaxf(dloc, fabsf((fnew - wv.v[v]) * invw[v]));
-        } else if constexpr (kKeep) {
-          const float qv = (fnew - wv.v[v]) * invw[v];
-          if (sr) {
-            const uint64_t gi = (uint64_t(k0 + e) * NP + n) * uint64_t(Qp) + uint64_t(i + v);
-            fnew_s.v[v] = bf16_round_stochastic(qv, sr_hash(gi, sr_step, uint32_t(a.sr_stage)));
-          } else {
-            fnew_s.v[v] = ST::from_r(qv);
-          }
-        } else {
-          fnew_s.v[v] = S(fnew);
-        }
+    eo_volume<M>([&](int n) { return fr[n]; }, na, nd, le, lo, [&](int n, Pair adv) {
+      Pair m0, m1, m2, m3, mx, my;
+      const int node = e * NP + n;
+      if constexpr (kDirect) {
+        const ulonglong2* mm = reinterpret_cast<const ulonglong2*>(sm.mom + size_t(node) * kRecPairFloats);
+        const ulonglong2 u = mm[0], v = mm[1], x = mm[2];
+        m0 = u.x; m1 = u.y; m2 = v.x; m3 = v.y; mx = x.x; my = x.y;
+      } else {
+        const float4* mm = reinterpret_cast<const float4*>(sm.mom + size_t(node) * 8);
+        const float4 u = mm[0], v = mm[1];
+        m0 = both(u.x); m1 = both(u.y); m2 = both(u.z); m3 = both(u.w); mx = both(v.x); my = both(v.y);
       }
-      *reinterpret_cast<RV*>(rrow + n * Qp) = rr;
-      if constexpr (!kTrack) *reinterpret_cast<SV*>(frow + n * Qp) = fnew_s;
-    };
-    static_assert(kPacked || VPT == 1, "two velocities per thread run as packed pairs");
-    R an[2], dn[2];
-#pragma unroll
-    for (int v = 0; v < VPT; ++v) {
-      an[v] = R(-0.5) * (ar[v] + as[v]);
-      dn[v] = R(0.5) * (ar[v] - as[v]);
-    }
-    T fp[NP];
-#pragma unroll
-    for (int m = 0; m < NP; ++m) {
-      const R x[2] = {fr[0][m], fr[VPT - 1][m]};
-      fp[m] = pack(x);
-    }
-    eo_volume<M>([&](int n) { return fp[n]; }, pack(an), pack(dn), le[0], lo[0], [&](int n, T adv) {
-      R x[2];
-      if constexpr (kPacked) f2unpack(adv, x[0], x[1]);
-      else x[0] = adv;
-      finish(n, x);
+      // f itself from shared memory again: in registers next to its even and odd
+      // parts it would cost a resident CTA
+      const Pair f = value_pair<ST>(frow + n * Qp, w, ws);
+      const Pair eu = f2fma(ey, my, f2mul(ex, mx));
+      Pair feq = f2fma(ey, m2, f2fma(ex, m1, m0));
+      feq = f2fma(eu, f2mul(m3, eu), feq);
+      if (third) {
+        float2 t;
+        if constexpr (kDirect) t = reinterpret_cast<const float2*>(sm.mom + size_t(a.epc) * NP * kRecPairFloats)[node];
+        else t = reinterpret_cast<const float2*>(sm.mom + size_t(node) * 8)[3];
+        feq = f2fma(eu, f2fma(both(t.x), f2mul(eu, eu), both(t.y)), feq);
+      }
+      Pair r = f2fma(w, feq, f2fma(neg_k, f, adv));
+      if (read_res) r = f2fma(rkA2, *reinterpret_cast<const Pair*>(rrow + n * Qp), r);
+      *reinterpret_cast<Pair*>(rrow + n * Qp) = r;
+      const Pair fnew = f2fma(rkB2, r, f);
+      if constexpr (ST::dev) {
+        float q0, q1;
+        f2unpack(f2mul(EoPacked::sub(fnew, w), invw), q0, q1);
+        if constexpr (kTrack) {
+          dloc = fmaxf(dloc, fmaxf(fabsf(q0), fabsf(q1)));
+        } else {
+          __nv_bfloat162 q;
+          if (sr) {
+            const uint64_t gi = (uint64_t(k0 + e) * NP + n) * uint64_t(Qp) + uint64_t(i);
+            q.x = bf16_round_stochastic(q0, sr_hash(gi, sr_step, uint32_t(a.sr_stage)));
+            q.y = bf16_round_stochastic(q1, sr_hash(gi + 1, sr_step, uint32_t(a.sr_stage)));
+          } else {
+            q = __floats2bfloat162_rn(q0, q1);
+          }
+          *reinterpret_cast<__nv_bfloat162*>(frow + n * Qp) = q;
+        }
+      } else {
+        *reinterpret_cast<Pair*>(frow + n * Qp) = fnew;
+      }
     });
     if constexpr (kTrack) {
       if (e != emax) {
@@ -633,16 +775,13 @@ __device__ __forceinline__ void item_update(const StageArgs<typename ST::R>& a,
   }
 }
 
-// Minimum resident CTAs of 256 threads per SM: bounds the registers per thread
-// (65536 / (256 * min)) so that the unrolled node loop does not spill.  At
-// degree 4 the shared memory of the usual 128-thread tile already limits an SM
-// to four CTAs, so 128 registers cost no occupancy there (measured +4 %); at
-// degree 5, 128 registers measured slower than 85.
+// Registers per thread of the FMA kernel, so that the unrolled update does not
+// spill and the tile's shared memory, not the register file, bounds the resident
+// CTAs (tiles have 64 to 256 threads).
 template <class ST, int QT>
-__host__ __device__ constexpr int stage_min_blocks() {
-  return sizeof(typename ST::R) == 8 ? 2 : items_vpt<ST, QT>() == 2 ? 2 : (P <= 3 || P == 5 ? 3 : 2);
+__host__ __device__ constexpr int stage_max_regs() {
+  return sizeof(typename ST::R) == 8 ? 128 : P <= 2 ? 96 : P <= 4 ? 128 : 168;
 }
-
 
 // Bulk copies (TMA) of one tile into a shared-memory stage, issued by warp 0:
 // element tile, residual tile (stages 2..5), geometry and every neighbour face
@@ -680,9 +819,18 @@ __device__ void issue_tile_loads(const StageArgs<typename ST::R>& a, StageSmem<t
   uint64_t* bar_rt = sm.bar + 1;
   uint32_t bytes = 0;
   if (lane == 0) bytes += (read_res ? res_bytes : 0u);
-  for (int row = lane; row < ne * NF; row += 32) {
-    const int code = __ldg(a.nbr + (k0 + row / NF) * 3 + (row % NF) / NFP);
-    if (code >= 0) bytes += uint32_t(row_bytes);
+  if constexpr (direct_traces<ST, QT>()) {
+    // the update reads the traces itself: only their row numbers are left here
+    uint32_t* rows = reinterpret_cast<uint32_t*>(sm.tr);
+    for (int row = lane; row < ne * NF; row += 32) {
+      const int code = __ldg(a.nbr + (k0 + row / NF) * 3 + (row % NF) / NFP);
+      rows[row] = code >= 0 ? uint32_t(code >> 3) * NP + trace_node(code, row % NFP) : 0u;
+    }
+  } else {
+    for (int row = lane; row < ne * NF; row += 32) {
+      const int code = __ldg(a.nbr + (k0 + row / NF) * 3 + (row % NF) / NFP);
+      if (code >= 0) bytes += uint32_t(row_bytes);
+    }
   }
   mbar_arrive_expect_tx(sm.bar, lane == 0 ? tile_bytes + geo_bytes + a.extra_tx : 0u);
   mbar_arrive_expect_tx(bar_rt, bytes);
@@ -691,16 +839,13 @@ __device__ void issue_tile_loads(const StageArgs<typename ST::R>& a, StageSmem<t
     bulk_load(sm.geo, a.geo + k0 * kGeoStrideDev, geo_bytes, sm.bar);
     if (read_res) bulk_load(sm.res, a.res + k0 * NP * Qp, res_bytes, bar_rt);
   }
-  for (int row = lane; row < ne * NF; row += 32) {
-    const int e = row / NF, fc = (row % NF) / NFP, aa = row % NFP;
-    const int code = __ldg(a.nbr + (k0 + e) * 3 + fc);
-    if (code >= 0) {
-      const int64_t kn = code >> 3;
-      const int fn = (code >> 1) & 3;
-      const int a2 = (code & 1) ? NFP - 1 - aa : aa;
-      const int rs = a2 * (P + 1) - a2 * (a2 - 1) / 2;
-      const int node = fn == 0 ? a2 : (fn == 1 ? rs + (P - a2) : rs);
-      bulk_load(sm.tr + size_t(row) * Qp, fin + (kn * NP + node) * Qp, uint32_t(row_bytes), bar_rt);
+  if constexpr (!direct_traces<ST, QT>()) {
+    for (int row = lane; row < ne * NF; row += 32) {
+      const int e = row / NF, fc = (row % NF) / NFP, aa = row % NFP;
+      const int code = __ldg(a.nbr + (k0 + e) * 3 + fc);
+      if (code >= 0)
+        bulk_load(sm.tr + size_t(row) * Qp, fin + (int64_t(code >> 3) * NP + trace_node(code, aa)) * Qp,
+                  uint32_t(row_bytes), bar_rt);
     }
   }
 }
@@ -710,7 +855,7 @@ __device__ void issue_tile_loads(const StageArgs<typename ST::R>& a, StageSmem<t
 // QT > 0: the padded velocity count is the compile-time constant QT (all
 // shared-memory strides become immediate offsets); QT = 0: taken from a.Qp.
 template <class ST, int QT>
-__global__ void __launch_bounds__(256, stage_min_blocks<ST, QT>()) stage_kernel(const StageArgs<typename ST::R> a) {
+__global__ void __maxnreg__((stage_max_regs<ST, QT>())) stage_kernel(const StageArgs<typename ST::R> a) {
   using R = typename ST::R;
   using S = typename ST::S;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -719,8 +864,9 @@ __global__ void __launch_bounds__(256, stage_min_blocks<ST, QT>()) stage_kernel(
   const R rkA = a.rkA;
   const bool read_res = rkA != R(0);
   const int64_t ntiles = (a.K + epc - 1) / epc;
-  const size_t stage_bytes = stage_smem_stride(NP, NF, epc, Qp, sizeof(S), sizeof(R));
-  auto stage = [&](int sidx) { return carve_stage_smem<R, S>(smem + sidx * stage_bytes, NP, NF, epc, Qp); };
+  constexpr bool kDirect = direct_traces<ST, QT>();
+  const size_t stage_bytes = stage_smem_stride(NP, NF, epc, Qp, sizeof(S), sizeof(R), kDirect);
+  auto stage = [&](int sidx) { return carve_stage_smem<R, S>(smem + sidx * stage_bytes, NP, NF, epc, Qp, kDirect); };
   const size_t row_bytes = size_t(Qp) * sizeof(S);
 
   const bool two = a.nstages == 2;
@@ -789,7 +935,8 @@ __global__ void __launch_bounds__(256, stage_min_blocks<ST, QT>()) stage_kernel(
 
     // ---- 2. node moments ---------------------------------------------------------
     if (!a.collision) {
-      for (int v = tid; v < ne * NP * 8; v += nth) sm.mom[v] = R(0);
+      const int words = kDirect ? epc * NP * (kRecPairFloats + 2) : ne * NP * 8;
+      for (int v = tid; v < words; v += nth) sm.mom[v] = R(0);
     } else {
       // the usual large-Q tiles (one element, 128 or 256 threads) take the
       // moment reduction with compile-time lane groups and an unrolled loop
@@ -797,11 +944,11 @@ __global__ void __launch_bounds__(256, stage_min_blocks<ST, QT>()) stage_kernel(
         using Acc = decltype(acc);
         constexpr int kBig = QT >= 128 ? 1 : 0;
         if (kBig && epc == 1 && nth == 128)
-          tile_moments<ST, Acc, QT, kBig * 128, 1>(a, sm.f, sm.scale, sm.geo, sm.mom, ne, sm.vel);
+          tile_moments<ST, Acc, QT, kBig * 128, 1, record_form<ST, QT>()>(a, sm.f, sm.scale, sm.geo, sm.mom, ne, sm.vel);
         else if (kBig && epc == 1 && nth == 256)
-          tile_moments<ST, Acc, QT, kBig * 256, 1>(a, sm.f, sm.scale, sm.geo, sm.mom, ne, sm.vel);
+          tile_moments<ST, Acc, QT, kBig * 256, 1, record_form<ST, QT>()>(a, sm.f, sm.scale, sm.geo, sm.mom, ne, sm.vel);
         else
-          tile_moments<ST, Acc, QT>(a, sm.f, sm.scale, sm.geo, sm.mom, ne, sm.vel);
+          tile_moments<ST, Acc, QT, 0, 1, record_form<ST, QT>()>(a, sm.f, sm.scale, sm.geo, sm.mom, ne, sm.vel);
       };
       if constexpr (sizeof(R) == 8) {
         moments(AccD{});
@@ -828,7 +975,8 @@ __global__ void __launch_bounds__(256, stage_min_blocks<ST, QT>()) stage_kernel(
     // ---- 4. residual and update ----------------------------------------------------
     float dmax = 0.f;  // deviation forms: running max |f/w - 1| of element emax
     int emax = -1;
-    item_update<ST, QT, items_vpt<ST, QT>()>(a, sm, k0, ne, read_res, dmax, emax);
+    if constexpr (sizeof(R) == 8) value_update<ST, QT>(a, sm, ne, read_res);
+    else pair_update<ST, QT>(a, sm, k0, ne, read_res, dmax, emax);
 
     // ---- 5. deviation forms: the kept scale (BF16), or the new per-element
     // scale and the encoding in place (FP16) ------------------------------------

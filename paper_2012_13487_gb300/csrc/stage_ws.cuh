@@ -87,9 +87,6 @@ __device__ __forceinline__ bool wait_for_number(const int* word, int want, uint6
   return true;
 }
 
-using Pair = unsigned long long;  // two FP32 values, the lower velocity in the low half
-__device__ __forceinline__ Pair both(float x) { return f2pack(x, x); }
-
 // Node record: eight coefficients of dt f^eq / tau, each stored twice
 // (c0, c1, c2, c3, u_x, u_y, c6, c7; see node_record).
 constexpr int kRec = 16;
@@ -128,22 +125,6 @@ __host__ __device__ constexpr Layout layout() {
   o.wn = b;     b += up(size_t(2 * G) * NF * 4, 16);
   o.end = b;
   return o;
-}
-
-// Two adjacent stored values as an FP32 pair (decoded by the caller).
-template <class ST>
-__device__ __forceinline__ Pair load_raw(const typename ST::S* p) {
-  if constexpr (ST::dev) {
-    const uint32_t q = *reinterpret_cast<const uint32_t*>(p);  // BF16: the upper half of an FP32
-    return f2pack(__uint_as_float(q << 16), __uint_as_float(q & 0xffff0000u));
-  } else {
-    return *reinterpret_cast<const Pair*>(p);
-  }
-}
-template <class ST>
-__device__ __forceinline__ Pair load_pair(const typename ST::S* p, Pair w, Pair ws) {
-  if constexpr (ST::dev) return f2fma(ws, load_raw<ST>(p), w);
-  else return load_raw<ST>(p);
 }
 
 // Moments of every node of the element in `row0` and their records.  G lanes
@@ -438,7 +419,7 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
       const S* fcol = st_f(s) + i;
       Pair fr[NP];
 #pragma unroll
-      for (int m = 0; m < NP; ++m) fr[m] = load_pair<ST>(fcol + m * QT, w, ws);
+      for (int m = 0; m < NP; ++m) fr[m] = value_pair<ST>(fcol + m * QT, w, ws);
       // face fc carries flux for some velocity of this warp (warp-uniform; with
       // the upwind flux an outflow face's jump term is zero, so a face that is
       // outflow for all 64 velocities skips its traces and lift columns)
@@ -466,7 +447,7 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
           const S* trow = st_tr(s) + fc * NFP * QT + i;
 #pragma unroll
           for (int aa = 0; aa < NFP; ++aa)
-            flux[fc * NFP + aa] = f2mul(c, EoPacked::sub(fr[face_node(fc, aa)], load_pair<ST>(trow + aa * QT, w, wsn)));
+            flux[fc * NFP + aa] = f2mul(c, EoPacked::sub(fr[face_node(fc, aa)], value_pair<ST>(trow + aa * QT, w, wsn)));
         } else {
           const int slot = -code - 1;
           const Pair fb = *reinterpret_cast<const Pair*>(a.wall_feq + size_t(slot) * QT + i);
@@ -495,7 +476,7 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
       eo_volume<M>([&](int n) { return fr[n]; }, na, nd, le, lo, [&](int n, Pair adv) {
         const ulonglong2* mm = reinterpret_cast<const ulonglong2*>(rec + n * kRec);
         const ulonglong2 m01 = mm[0], m23 = mm[1], mu = mm[2];
-        const Pair f = load_pair<ST>(fcol + n * QT, w, ws);
+        const Pair f = value_pair<ST>(fcol + n * QT, w, ws);
         const Pair eu = f2fma(ey, mu.y, f2mul(ex, mu.x));
         Pair feq = f2fma(ey, m23.x, f2fma(ex, m01.y, m01.x));
         feq = f2fma(eu, f2mul(m23.y, eu), feq);
