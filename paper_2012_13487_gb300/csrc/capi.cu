@@ -1471,8 +1471,13 @@ struct Implicit {
   double* Rp = nullptr;     // R(Y + eps v)
   double* V = nullptr;      // GMRES basis [m+1][n]
   double* k = nullptr;      // stage derivatives [s][n]
-  double* partial = nullptr;  // [m+1][kDotBlocks]
+  double* partial = nullptr;  // two of [m+1][kMaxBlocks]: the two Gram-Schmidt passes
   double* hdev = nullptr;     // [m+2] dot results / combination coefficients
+  double* zpart = nullptr;    // [kMaxBlocks] partial sums of |M^-1 v|^2
+  double* step = nullptr;     // [1] step of the difference quotient
+  double* hcol = nullptr;     // [2 (m+1) + kMaxBlocks]: h of both passes, partial sums of |w|^2
+  double* hcol_host = nullptr;  // the same, pinned
+  cudaEvent_t column = nullptr; // hcol_host is complete
   void* x32 = nullptr;        // FP32 state: FP32 copy of the input of R
   void* r32 = nullptr;        // FP32 state: FP32 residual register
   void* scratch = nullptr;    // stage-kernel state output (unused values)
@@ -1487,8 +1492,11 @@ struct Implicit {
 
 void free_implicit(Implicit& im) {
   void* bufs[] = {im.u0, im.Y, im.base, im.RY, im.G, im.d, im.w, im.Yp, im.Rp, im.V, im.k, im.partial, im.hdev,
-                  im.x32, im.r32, im.scratch, im.geo_unit, im.minv, im.z, im.ops, im.fmask};
+                  im.x32, im.r32, im.scratch, im.geo_unit, im.minv, im.z, im.ops, im.fmask, im.zpart, im.step,
+                  im.hcol};
   for (void* p : bufs) cudaFree(p);
+  cudaFreeHost(im.hcol_host);
+  if (im.column) cudaEventDestroy(im.column);
   im = Implicit();
 }
 
@@ -1504,8 +1512,14 @@ int ensure_implicit(const Batch& b, const Group& g, Implicit& im, int m, int s) 
   for (double** v : vecs) FEDBM_CK(cudaMalloc(v, vb));
   FEDBM_CK(cudaMalloc(&im.V, vb * size_t(m + 1)));
   FEDBM_CK(cudaMalloc(&im.k, vb * size_t(s)));
-  FEDBM_CK(cudaMalloc(&im.partial, size_t(m + 1) * krylov::kDotBlocks * sizeof(double)));
+  FEDBM_CK(cudaMalloc(&im.partial, size_t(2) * (m + 1) * krylov::kMaxBlocks * sizeof(double)));
   FEDBM_CK(cudaMalloc(&im.hdev, size_t(m + 2) * sizeof(double)));
+  FEDBM_CK(cudaMalloc(&im.zpart, krylov::kMaxBlocks * sizeof(double)));
+  FEDBM_CK(cudaMalloc(&im.step, sizeof(double)));
+  const size_t col = (size_t(2) * (m + 1) + krylov::kMaxBlocks) * sizeof(double);
+  FEDBM_CK(cudaMalloc(&im.hcol, col));
+  FEDBM_CK(cudaMallocHost(&im.hcol_host, col));
+  FEDBM_CK(cudaEventCreateWithFlags(&im.column, cudaEventDisableTiming));
   const size_t rb = real_bytes(g.store);
   FEDBM_CK(cudaMalloc(&im.scratch, size_t(n) * rb));
   if (g.store == kStoreF32) {
@@ -1591,7 +1605,7 @@ int implicit_gmres(const Batch& b, const Group& g, Implicit& im, double dtg, dou
   const int m = im.m;
   cudaStream_t st = b.stream;
   FEDBM_CK(cudaMemsetAsync(im.d, 0, size_t(n) * sizeof(double), st));
-  std::vector<double> H(size_t(m + 1) * m, 0.0), cs(m), sn(m), gv(m + 1), y(m), h1(m + 1), h2(m + 1);
+  std::vector<double> H(size_t(m + 1) * m, 0.0), cs(m), sn(m), gv(m + 1), y(m);
   int total = 0;
   bool first = true;
   while (total < max_iter) {
@@ -1622,37 +1636,42 @@ int implicit_gmres(const Batch& b, const Group& g, Implicit& im, double dtg, dou
     gv[0] = beta;
     int jend = 0;
     double resid = beta;
-    for (int j = 0; j < m && total < max_iter; ++j, ++total) {
+    const int nb = krylov::blocks_of(n);
+    double* part1 = im.partial;
+    double* part2 = im.partial + size_t(m + 1) * krylov::kMaxBlocks;
+    double *dh1 = im.hcol, *dh2 = im.hcol + (m + 1), *dnorm = im.hcol + 2 * (m + 1);
+    // R(Y + e M^-1 v_j) for basis vector j (right preconditioning; M = I without a
+    // preconditioner), v_j = w / |w| where the iteration before left it in w
+    auto evaluate = [&](int j, bool from_w) -> int {
       double* vj = im.V + size_t(j) * n;
-      // w = A M^-1 v_j (right preconditioning; M = I without a preconditioner)
-      const double* xj = vj;
-      double ex = eps;
-      if (precond) {
-        FEDBM_CK(krylov::block_jacobi_apply(g.K, g.Np, g.Qp, im.minv, vj, im.z, st));
-        double zn = 0;
-        if ((rc = implicit_norm(b, im, im.z, &zn)) != FEDBM_OK) return rc;
-        xj = im.z;
-        ex = zn > 0 ? eps / zn : eps;
-      }
-      FEDBM_CK(krylov::axpby(n, 1.0, im.Y, ex, xj, im.Yp, st));
-      if ((rc = implicit_rhs(b, g, im, im.Yp, im.Rp)) != FEDBM_OK) return rc;
+      if (precond || from_w)
+        FEDBM_CK(krylov::direction(g.K, g.Np, g.Qp, precond ? im.minv : nullptr, from_w ? im.w : vj,
+                                   from_w ? dnorm : nullptr, vj, im.z, im.zpart, st));
+      FEDBM_CK(krylov::perturb(n, eps, precond ? im.zpart : nullptr, im.Y, precond ? im.z : vj, im.step, im.Yp, st));
+      return implicit_rhs(b, g, im, im.Yp, im.Rp);
+    };
+    if ((rc = evaluate(0, false)) != FEDBM_OK) return rc;
+    for (int j = 0; j < m && total < max_iter; ++j, ++total) {
       ++cnt.rhs;
-      FEDBM_CK(krylov::axpby(n, 1.0, im.Rp, -1.0, im.RY, im.w, st));
-      FEDBM_CK(krylov::axpby(n, 1.0, xj, -dtg / ex, im.w, im.w, st));
-      // two passes of classical Gram-Schmidt against v_0 .. v_j
-      for (int pass = 0; pass < 2; ++pass) {
-        std::vector<double>& hh = pass == 0 ? h1 : h2;
-        FEDBM_CK(krylov::multi_dot(n, j + 1, im.V, im.w, im.partial, im.hdev, st));
-        FEDBM_CK(krylov::sub_combination(n, j + 1, im.V, im.hdev, im.w, st));
-        FEDBM_CK(cudaMemcpyAsync(hh.data(), im.hdev, size_t(j + 1) * sizeof(double), cudaMemcpyDeviceToHost, st));
-      }
+      // w = A M^-1 v_j and two passes of classical Gram-Schmidt against v_0 .. v_j
+      const double* xj = precond ? im.z : im.V + size_t(j) * n;
+      FEDBM_CK(krylov::project_first(n, j + 1, xj, im.Rp, im.RY, im.step, dtg, im.V, im.w, part1, st));
+      FEDBM_CK(krylov::project_next(n, j + 1, im.V, part1, dh1, im.w, part2, false, st));
+      FEDBM_CK(krylov::project_next(n, j + 1, im.V, part2, dh2, im.w, dnorm, true, st));
+      FEDBM_CK(cudaMemcpyAsync(im.hcol_host, im.hcol, (size_t(2) * (m + 1) + nb) * sizeof(double),
+                               cudaMemcpyDeviceToHost, st));
+      FEDBM_CK(cudaEventRecord(im.column, st));
+      // the next evaluation is queued before the host has looked at this column: it
+      // covers the way to the host and back (not used if this column converges)
+      if (j + 1 < m && total + 1 < max_iter && (rc = evaluate(j + 1, true)) != FEDBM_OK) return rc;
+      FEDBM_CK(cudaEventSynchronize(im.column));
+      const double *h1 = im.hcol_host, *h2 = im.hcol_host + (m + 1);
       double hn = 0;
-      if ((rc = implicit_norm(b, im, im.w, &hn)) != FEDBM_OK) return rc;  // synchronises: h1, h2 are valid
+      for (int q = 0; q < nb; ++q) hn += im.hcol_host[2 * (m + 1) + q];
+      hn = std::sqrt(std::max(0.0, hn));
       ++cnt.gmres;
       for (int i = 0; i <= j; ++i) H[size_t(i) * m + j] = h1[i] + h2[i];
       H[size_t(j + 1) * m + j] = hn;
-      if (j + 1 <= m && hn > 0)
-        FEDBM_CK(krylov::axpby(n, 1.0 / hn, im.w, 0.0, im.w, im.V + size_t(j + 1) * n, st));
       // Givens rotations
       for (int i = 0; i < j; ++i) {
         const double a0 = H[size_t(i) * m + j], a1 = H[size_t(i + 1) * m + j];

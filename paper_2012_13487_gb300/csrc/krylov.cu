@@ -17,45 +17,163 @@ __global__ void axpby_kernel(int64_t n, double a, const double* x, double b, con
     out[i] = a * x[i] + b * y[i];
 }
 
-__global__ void combination_kernel(int64_t n, int m, const double* V, const double* c, double* y, double sign) {
+__global__ void combination_kernel(int64_t n, int m, const double* V, const double* c, double* y) {
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
     double acc = 0.0;
     for (int j = 0; j < m; ++j) acc += c[j] * V[size_t(j) * n + i];
-    y[i] += sign * acc;
+    y[i] += acc;
   }
 }
 
-// partial[j][block] = sum over this block's grid-stride share of V_j[i] w[i]
-__global__ void dot_partial_kernel(int64_t n, const double* V, const double* w, double* partial) {
-  __shared__ double red[kThreads / 32];
-  const int j = blockIdx.y;
-  const double* v = V + size_t(j) * n;
-  double acc = 0.0;
-  for (int64_t i = blockIdx.x * int64_t(kThreads) + threadIdx.x; i < n; i += int64_t(kDotBlocks) * kThreads)
-    acc += v[i] * w[i];
+// sum over the block's threads, in thread 0 (red: one double per warp)
+__device__ __forceinline__ double block_sum(double acc, double* red) {
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
+  double t = 0.0;
+  if (threadIdx.x == 0)
     for (int q = 0; q < kThreads / 32; ++q) t += red[q];
-    partial[size_t(j) * kDotBlocks + blockIdx.x] = t;
+  __syncthreads();
+  return t;
+}
+
+// sum of p[0 .. nb) over a warp, in every lane
+__device__ __forceinline__ double warp_sum(const double* p, int nb) {
+  double acc = 0.0;
+  for (int q = threadIdx.x & 31; q < nb; q += 32) acc += p[q];
+  for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+  return acc;
+}
+
+// This block's chunk [lo, hi) of n values (gridDim.x chunks).
+__device__ __forceinline__ void chunk_of(int64_t n, int64_t& lo, int64_t& hi) {
+  const int64_t len = ((n + gridDim.x - 1) / gridDim.x + kThreads - 1) / kThreads * kThreads;
+  lo = min(n, int64_t(blockIdx.x) * len);
+  hi = min(n, lo + len);
+}
+
+// part[j][block] = sum over the block's chunk of V_j w for j < m, eight j at a time so
+// that w is read once for them and one barrier serves them all.  FP64 arithmetic is
+// slow here, and a reduction of one value per thread was mostly the reduction (512
+// blocks a vector whatever its length: 21 us for 15 vectors of 82k values).
+__device__ void chunk_dots(int64_t n, int64_t lo, int64_t hi, int m, const double* V, const double* w, double* part) {
+  __shared__ double red[kThreads / 32][8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int j0 = 0; j0 < m; j0 += 8) {
+    double acc[8] = {};
+    for (int64_t i = lo + threadIdx.x; i < hi; i += kThreads) {
+      const double wi = w[i];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (j0 + j < m) acc[j] = fma(V[size_t(j0 + j) * n + i], wi, acc[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (j0 + j >= m) break;
+      for (int off = 16; off > 0; off >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], off);
+      if (lane == 0) red[warp][j] = acc[j];
+    }
+    __syncthreads();
+    if (threadIdx.x < 8 && j0 + int(threadIdx.x) < m) {
+      double t = 0.0;
+      for (int q = 0; q < kThreads / 32; ++q) t += red[q][threadIdx.x];
+      part[size_t(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
+    }
+    __syncthreads();
   }
 }
 
-// h[j] = sum of partial[j][*], one block per j
-__global__ void dot_final_kernel(const double* partial, double* h) {
+__global__ void dot_partial_kernel(int64_t n, int m, const double* V, const double* w, double* partial) {
+  int64_t lo, hi;
+  chunk_of(n, lo, hi);
+  chunk_dots(n, lo, hi, m, V, w, partial);
+}
+
+// h[j] = sum of partial[j][0 .. nb), one warp per j
+__global__ void dot_final_kernel(int m, int nb, const double* partial, double* h) {
+  const int j = (blockIdx.x * kThreads + threadIdx.x) >> 5;
+  if (j >= m) return;
+  const double t = warp_sum(partial + size_t(j) * nb, nb);
+  if ((threadIdx.x & 31) == 0) h[j] = t;
+}
+
+__global__ void direction_kernel(int64_t n, int Np, int Qp, const double* minv, const double* src,
+                                 const double* norm_part, int nb, double* v, double* z, double* zpart) {
   __shared__ double red[kThreads / 32];
-  const int j = blockIdx.x;
+  double s = 1.0;
+  if (norm_part) {
+    const double t = warp_sum(norm_part, nb);
+    s = t > 0.0 ? 1.0 / sqrt(t) : 0.0;
+  }
   double acc = 0.0;
-  for (int q = threadIdx.x; q < kDotBlocks; q += kThreads) acc += partial[size_t(j) * kDotBlocks + q];
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  for (int64_t t = blockIdx.x * int64_t(kThreads) + threadIdx.x; t < n; t += int64_t(gridDim.x) * kThreads) {
+    if (norm_part) v[t] = src[t] * s;
+    if (minv) {
+      // (element k, node r, velocity i): row r of the block times the column of v
+      const int64_t kn = t / Qp, k = kn / Np;
+      const int i = int(t - kn * Qp);
+      const double* col = src + k * Np * Qp + i;
+      const double* row = minv + kn * Np * Qp + i;
+      double a = 0.0;
+      for (int q = 0; q < Np; ++q) a = fma(row[size_t(q) * Qp], col[size_t(q) * Qp] * s, a);
+      z[t] = a;
+      acc = fma(a, a, acc);
+    }
+  }
+  if (minv && zpart) {
+    acc = block_sum(acc, red);
+    if (threadIdx.x == 0) zpart[blockIdx.x] = acc;
+  }
+}
+
+__global__ void perturb_kernel(int64_t n, double eps, const double* zpart, int nb, const double* Y, const double* x,
+                               double* step, double* out) {
+  double e = eps;
+  if (zpart) {
+    const double t = sqrt(warp_sum(zpart, nb));
+    e = t > 0.0 ? eps / t : eps;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) step[0] = e;
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+    out[i] = Y[i] + e * x[i];
+}
+
+__global__ void project_first_kernel(int64_t n, int m, const double* x, const double* Rp, const double* RY,
+                                     const double* step, double dtg, const double* V, double* w, double* part) {
+  int64_t lo, hi;
+  chunk_of(n, lo, hi);
+  const double c = -dtg / step[0];
+  for (int64_t i = lo + threadIdx.x; i < hi; i += kThreads) w[i] = x[i] + c * (Rp[i] - RY[i]);
+  chunk_dots(n, lo, hi, m, V, w, part);  // every thread reads back only what it wrote
+}
+
+__global__ void project_next_kernel(int64_t n, int m, const double* V, const double* part_in, double* h_out, double* w,
+                                    double* part_out, bool last) {
+  extern __shared__ double h[];
+  __shared__ double red[kThreads / 32];
+  for (int j = threadIdx.x >> 5; j < m; j += kThreads / 32) {
+    const double t = warp_sum(part_in + size_t(j) * gridDim.x, gridDim.x);
+    if ((threadIdx.x & 31) == 0) {
+      h[j] = t;
+      if (blockIdx.x == 0) h_out[j] = t;
+    }
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  int64_t lo, hi;
+  chunk_of(n, lo, hi);
+  double acc = 0.0;
+  for (int64_t i = lo + threadIdx.x; i < hi; i += kThreads) {
     double t = 0.0;
-    for (int q = 0; q < kThreads / 32; ++q) t += red[q];
-    h[j] = t;
+    for (int j = 0; j < m; ++j) t = fma(h[j], V[size_t(j) * n + i], t);
+    const double wi = w[i] - t;
+    w[i] = wi;
+    acc = fma(wi, wi, acc);
+  }
+  if (last) {
+    acc = block_sum(acc, red);
+    if (threadIdx.x == 0) part_out[blockIdx.x] = acc;
+  } else {
+    chunk_dots(n, lo, hi, m, V, w, part_out);
   }
 }
 
@@ -76,29 +194,61 @@ __global__ void set_geo_dt_kernel(int64_t K, int stride, int slot, double value,
 
 }  // namespace
 
+int blocks_of(int64_t n) {
+  const int64_t b = (n + 1023) / 1024;
+  return int(b < 1 ? 1 : b > kMaxBlocks ? kMaxBlocks : b);
+}
+
+int direction_blocks(int64_t n) {
+  const int64_t b = (n + kThreads - 1) / kThreads;
+  return int(b < 1 ? 1 : b > kMaxBlocks ? kMaxBlocks : b);
+}
+
+cudaError_t direction(int64_t K, int Np, int Qp, const double* minv, const double* src, const double* norm_part,
+                      double* v, double* z, double* zpart, cudaStream_t st) {
+  const int64_t n = K * Np * Qp;
+  direction_kernel<<<direction_blocks(n), kThreads, 0, st>>>(n, Np, Qp, minv, src, norm_part, blocks_of(n), v, z,
+                                                             zpart);
+  return cudaGetLastError();
+}
+
+cudaError_t perturb(int64_t n, double eps, const double* zpart, const double* Y, const double* x, double* step,
+                    double* out, cudaStream_t st) {
+  perturb_kernel<<<direction_blocks(n), kThreads, 0, st>>>(n, eps, zpart, direction_blocks(n), Y, x, step, out);
+  return cudaGetLastError();
+}
+
+cudaError_t project_first(int64_t n, int m, const double* x, const double* Rp, const double* RY, const double* step,
+                          double dtg, const double* V, double* w, double* part, cudaStream_t st) {
+  project_first_kernel<<<blocks_of(n), kThreads, 0, st>>>(n, m, x, Rp, RY, step, dtg, V, w, part);
+  return cudaGetLastError();
+}
+
+cudaError_t project_next(int64_t n, int m, const double* V, const double* part_in, double* h_out, double* w,
+                         double* part_out, bool last, cudaStream_t st) {
+  project_next_kernel<<<blocks_of(n), kThreads, size_t(m) * sizeof(double), st>>>(n, m, V, part_in, h_out, w, part_out,
+                                                                                 last);
+  return cudaGetLastError();
+}
+
 cudaError_t axpby(int64_t n, double a, const double* x, double b, const double* y, double* out, cudaStream_t st) {
   axpby_kernel<<<grid_of(n), kThreads, 0, st>>>(n, a, x, b, y, out);
   return cudaGetLastError();
 }
 
-cudaError_t sub_combination(int64_t n, int m, const double* V, const double* c_dev, double* y, cudaStream_t st) {
-  if (m < 1) return cudaSuccess;
-  combination_kernel<<<grid_of(n), kThreads, 0, st>>>(n, m, V, c_dev, y, -1.0);
-  return cudaGetLastError();
-}
-
 cudaError_t add_combination(int64_t n, int m, const double* V, const double* c_dev, double* out, cudaStream_t st) {
   if (m < 1) return cudaSuccess;
-  combination_kernel<<<grid_of(n), kThreads, 0, st>>>(n, m, V, c_dev, out, 1.0);
+  combination_kernel<<<grid_of(n), kThreads, 0, st>>>(n, m, V, c_dev, out);
   return cudaGetLastError();
 }
 
 cudaError_t multi_dot(int64_t n, int m, const double* V, const double* w, double* partial, double* h, cudaStream_t st) {
   if (m < 1) return cudaSuccess;
-  dot_partial_kernel<<<dim3(kDotBlocks, m), kThreads, 0, st>>>(n, V, w, partial);
+  const int nb = blocks_of(n);
+  dot_partial_kernel<<<nb, kThreads, 0, st>>>(n, m, V, w, partial);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  dot_final_kernel<<<m, kThreads, 0, st>>>(partial, h);
+  dot_final_kernel<<<(m * 32 + kThreads - 1) / kThreads, kThreads, 0, st>>>(m, nb, partial, h);
   return cudaGetLastError();
 }
 
@@ -199,20 +349,6 @@ __global__ void bj_build_kernel(int64_t K, int Np, int Nfp, int Qp, const R* geo
     for (int m = 0; m < Np; ++m) minv[((k * Np + n) * Np + m) * Qp + i] = B[n * Np + m];
 }
 
-__global__ void bj_apply_kernel(int64_t K, int Np, int Qp, const double* minv, const double* v, double* z) {
-  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (t >= K * Qp) return;
-  const int64_t k = t / Qp;
-  const int i = int(t % Qp);
-  double x[kMaxNp];
-  for (int m = 0; m < Np; ++m) x[m] = v[(k * Np + m) * Qp + i];
-  for (int n = 0; n < Np; ++n) {
-    double acc = 0.0;
-    for (int m = 0; m < Np; ++m) acc += minv[((k * Np + n) * Np + m) * Qp + i] * x[m];
-    z[(k * Np + n) * Qp + i] = acc;
-  }
-}
-
 }  // namespace
 
 cudaError_t block_jacobi_build(int64_t K, int Np, int Nfp, int Qp, const void* geo, int real_bytes,
@@ -240,9 +376,7 @@ cudaError_t block_jacobi_build(int64_t K, int Np, int Nfp, int Qp, const void* g
 
 cudaError_t block_jacobi_apply(int64_t K, int Np, int Qp, const double* minv, const double* v, double* z,
                                cudaStream_t st) {
-  const int64_t n = K * Qp;
-  bj_apply_kernel<<<int((n + 255) / 256), 256, 0, st>>>(K, Np, Qp, minv, v, z);
-  return cudaGetLastError();
+  return direction(K, Np, Qp, minv, v, nullptr, nullptr, z, nullptr, st);
 }
 
 }  // namespace krylov

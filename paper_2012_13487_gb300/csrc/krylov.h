@@ -8,17 +8,17 @@
 namespace fedbm {
 namespace krylov {
 
-// Blocks of the partial-sum reductions (one partial sum per block).
-constexpr int kDotBlocks = 512;
+// Most blocks of a partial-sum reduction (one partial sum per block); a vector of
+// n values takes blocks_of(n), at least 1,024 values each.
+constexpr int kMaxBlocks = 608;
 constexpr int kThreads = 256;
+int blocks_of(int64_t n);
 
 // out = a x + b y (out may alias x or y)
 cudaError_t axpby(int64_t n, double a, const double* x, double b, const double* y, double* out, cudaStream_t st);
-// y -= sum_i c[i] V_i for i < m; V holds m vectors of n values each, c is host memory
-cudaError_t sub_combination(int64_t n, int m, const double* V, const double* c_dev, double* y, cudaStream_t st);
-// out = sum_i c[i] V_i + b out (i < m); c in device memory
+// out += sum_i c[i] V_i for i < m; V holds m vectors of n values each, c in device memory
 cudaError_t add_combination(int64_t n, int m, const double* V, const double* c_dev, double* out, cudaStream_t st);
-// h[i] = <V_i, w> for i < m, through partial[m][kDotBlocks] (device); h in device memory
+// h[i] = <V_i, w> for i < m, through partial[m][blocks_of(n)] (device); h in device memory
 cudaError_t multi_dot(int64_t n, int m, const double* V, const double* w, double* partial, double* h, cudaStream_t st);
 // FP64 <-> FP32 copies
 cudaError_t to_f32(int64_t n, const double* x, float* y, cudaStream_t st);
@@ -43,6 +43,28 @@ cudaError_t block_jacobi_build(int64_t K, int Np, int Nfp, int Qp, const void* g
 // z = M^-1 v, blockwise
 cudaError_t block_jacobi_apply(int64_t K, int Np, int Qp, const double* minv, const double* v, double* z,
                                cudaStream_t st);
+
+// ---- one GMRES iteration ---------------------------------------------------------
+// The scalars between these kernels (norms, Gram-Schmidt coefficients, the step of
+// the difference quotient) stay on the device: a kernel leaves one partial sum per
+// block and the blocks of the next each add them up, in the same order.
+
+// v = src / sqrt(sum of norm_part) (norm_part == nullptr: v = src, not written) and z =
+// M^-1 v (minv == nullptr: no z); zpart[0 .. return value of direction_blocks) = partial
+// sums of z^2
+int direction_blocks(int64_t n);
+cudaError_t direction(int64_t K, int Np, int Qp, const double* minv, const double* src, const double* norm_part,
+                      double* v, double* z, double* zpart, cudaStream_t st);
+// step[0] = eps / sqrt(sum of zpart) (zpart == nullptr, or a zero sum: eps); out = Y + step x
+cudaError_t perturb(int64_t n, double eps, const double* zpart, const double* Y, const double* x, double* step,
+                    double* out, cudaStream_t st);
+// w = x - dtg / step[0] (Rp - RY); part[j][blocks_of(n)] = partial <V_j, w> for j < m
+cudaError_t project_first(int64_t n, int m, const double* x, const double* Rp, const double* RY, const double* step,
+                          double dtg, const double* V, double* w, double* part, cudaStream_t st);
+// h_out[j] = h_j = sum of part_in[j], w -= sum_j h_j V_j; then part_out[j] = partial
+// <V_j, w>, or with last: part_out[0] = partial <w, w>
+cudaError_t project_next(int64_t n, int m, const double* V, const double* part_in, double* h_out, double* w,
+                         double* part_out, bool last, cudaStream_t st);
 
 }  // namespace krylov
 }  // namespace fedbm
