@@ -129,12 +129,14 @@ __global__ void __launch_bounds__(kThreads, cl_min_blocks<ST>()) stage_kernel_cl
   const int64_t ntiles = (a.K + epc - 1) / epc;
   constexpr bool kImm = kHaveOpsTable && sizeof(R) == 4 && P <= 5;
 
+  pdl_launch_dependents();
   for (int v = tid; v < 3 * Qc; v += nth) s_vel[v] = a.vel[(v / Qc) * Qp + v0 + v % Qc];
   if (tid == 0) {
     mbar_init(bar, 32);
     fence_mbar_init();
     fence_proxy_async_smem();
   }
+  pdl_wait();
   __syncthreads();
 
   // warp 0: bulk copies of this CTA's slice of tile t (element rows, residual
@@ -409,19 +411,8 @@ cudaError_t with_cl_kernel(int store_kind, Fn fn) {
 
 template <class ST>
 cudaError_t launch_cl_as(const void* args, int nclusters, int ncl, size_t smem, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(nclusters * ncl), 1, 1);
-  cfg.blockDim = dim3(cl::kThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = unsigned(ncl);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, cl::stage_kernel_cl<ST>, *static_cast<const StageArgs<typename ST::R>*>(args));
+  return launch_stage_kernel(&cl::stage_kernel_cl<ST>, nclusters * ncl, cl::kThreads, smem, st,
+                             *static_cast<const StageArgs<typename ST::R>*>(args), ncl);
 }
 
 cudaError_t launch_cl(int store_kind, const void* args, int nclusters, int ncl, size_t smem, cudaStream_t st) {

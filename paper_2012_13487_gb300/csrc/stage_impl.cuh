@@ -101,6 +101,7 @@ __host__ __device__ constexpr bool ops_immediate() {
 struct AccD {
   double s = 0.0;
   __device__ void add(double v) { s += v; }
+  __device__ void add(float v) { s += widen(v); }
   __device__ void reduce(int G) {
     for (int off = G >> 1; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
   }
@@ -217,6 +218,36 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 }
 __device__ __forceinline__ void fence_mbar_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+// Programmatic dependent launch: a stage kernel may be put on the SMs while the one
+// before it still runs its last CTAs.  It lets its own successor do the same at once
+// (launch_dependents), sets up its barriers and tables, which no earlier kernel
+// writes, and waits for the kernels before it to have finished, with their writes
+// visible, before it touches the state, the residual or the scales.
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class R>
+cudaError_t launch_stage_kernel(void (*kernel)(StageArgs<R>), int grid, int block, size_t smem, cudaStream_t st,
+                                const StageArgs<R>& a, int cluster = 0) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(grid), 1, 1);
+  cfg.blockDim = dim3(unsigned(block), 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = sizeof(R) == 4;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cluster > 1) {
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = unsigned(cluster);
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+  }
+  return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
 // Vector of the storage type covering 16 bytes.
@@ -870,6 +901,7 @@ __global__ void __maxnreg__((stage_max_regs<ST, QT>())) stage_kernel(const Stage
   const size_t row_bytes = size_t(Qp) * sizeof(S);
 
   const bool two = a.nstages == 2;
+  pdl_launch_dependents();
   // velocity rows e_x, e_y, w into every stage's copy (read by the moment and
   // wall-numerator reductions)
   for (int sidx = 0; sidx < (two ? 2 : 1); ++sidx) {
@@ -886,6 +918,7 @@ __global__ void __maxnreg__((stage_max_regs<ST, QT>())) stage_kernel(const Stage
     fence_mbar_init();
     fence_proxy_async_smem();
   }
+  pdl_wait();
   __syncthreads();
 
   int64_t tile = blockIdx.x;
@@ -1039,8 +1072,7 @@ __global__ void __maxnreg__((stage_max_regs<ST, QT>())) stage_kernel(const Stage
 template <class ST, int QT>
 cudaError_t launch_one(const void* args, int grid, int block, size_t smem, cudaStream_t st) {
   const auto& a = *static_cast<const StageArgs<typename ST::R>*>(args);
-  stage_kernel<ST, QT><<<grid, block, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_stage_kernel(&stage_kernel<ST, QT>, grid, block, smem, st, a);
 }
 
 // Velocity counts with a specialised kernel (the GH D2Q16 and NC 16x16 /

@@ -252,6 +252,7 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
   auto full = [&](int s) { return reinterpret_cast<uint64_t*>(smem + s * o.stage + o.bars); };
   auto empty = [&](int s) { return reinterpret_cast<uint64_t*>(smem + s * o.stage + o.bars) + 1; };
 
+  pdl_launch_dependents();
   for (int v = threadIdx.x; v < QT; v += threads<G>()) {
     s_vel[v] = a.vel[kVelEx * QT + v];
     s_vel[QT + v] = a.vel[kVelEy * QT + v];
@@ -270,6 +271,7 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
     fence_mbar_init();
     fence_proxy_async_smem();
   }
+  pdl_wait();
   __syncthreads();
 
   if (producer) {
@@ -557,8 +559,7 @@ cudaError_t launch_ws(int store_kind, const void* args, int groups, int grid, si
   const auto& a = *static_cast<const StageArgs<float>*>(args);
   const ws::Form f = ws::form(store_kind, a.Qp, groups);
   if (!f.kernel) return cudaErrorInvalidValue;
-  f.kernel<<<grid, f.threads, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_stage_kernel(f.kernel, grid, f.threads, smem, st, a);
 }
 
 cudaError_t set_smem_ws(int store_kind, int Qp, int groups, size_t smem) {

@@ -17,16 +17,6 @@ constexpr size_t kSmemCap = 227 * 1024 - 64;  // dynamic; the encode kernel has 
 // stores.
 constexpr size_t kStageBytes = 48 * 1024;
 
-// FP32 -> FP64 with integer operations for zeros and normal numbers: the
-// conversion instruction to FP64 runs at the part's low FP64 rate (two lanes
-// per clock and SM), which bounded the FP32 decode at 31M values (90 us
-// against 56 us for its bytes).
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t u = __float_as_uint(x), e = u & 0x7f800000u, m = u & 0x7fffffffu;
-  if (m != 0u && (e == 0u || e == 0x7f800000u)) return double(x);  // denormal, infinity, NaN
-  const uint32_t hi = (u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
-  return __hiloint2double(int(hi), int(u << 29));
-}
 __device__ __forceinline__ double widen(double x) { return x; }
 
 // Work split shared by encode and decode: a group of G threads (a warp where
