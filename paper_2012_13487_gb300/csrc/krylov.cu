@@ -57,7 +57,7 @@ __device__ __forceinline__ void chunk_of(int64_t n, int64_t& lo, int64_t& hi) {
 // slow here, and a reduction of one value per thread was mostly the reduction (512
 // blocks a vector whatever its length: 21 us for 15 vectors of 82k values).
 __device__ void chunk_dots(int64_t n, int64_t lo, int64_t hi, int m, const double* V, const double* w, double* part) {
-  __shared__ double red[kThreads / 32][8];
+  __shared__ double red[8][kThreads + 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int j0 = 0; j0 < m; j0 += 8) {
     double acc[8] = {};
@@ -67,17 +67,17 @@ __device__ void chunk_dots(int64_t n, int64_t lo, int64_t hi, int m, const doubl
       for (int j = 0; j < 8; ++j)
         if (j0 + j < m) acc[j] = fma(V[size_t(j0 + j) * n + i], wi, acc[j]);
     }
+    // through shared memory, warp j adding up vector j: a third of the additions of a
+    // shuffle reduction in every warp
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (j0 + j >= m) break;
-      for (int off = 16; off > 0; off >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], off);
-      if (lane == 0) red[warp][j] = acc[j];
-    }
+    for (int j = 0; j < 8; ++j) red[j][threadIdx.x] = acc[j];
     __syncthreads();
-    if (threadIdx.x < 8 && j0 + int(threadIdx.x) < m) {
+    if (j0 + warp < m) {
       double t = 0.0;
-      for (int q = 0; q < kThreads / 32; ++q) t += red[q][threadIdx.x];
-      part[size_t(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
+#pragma unroll
+      for (int q = 0; q < kThreads / 32; ++q) t += red[warp][q * 32 + lane];
+      for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+      if (lane == 0) part[size_t(j0 + warp) * gridDim.x + blockIdx.x] = t;
     }
     __syncthreads();
   }
@@ -100,10 +100,15 @@ __global__ void dot_final_kernel(int m, int nb, const double* partial, double* h
 __global__ void direction_kernel(int64_t n, int Np, int Qp, const double* minv, const double* src,
                                  const double* norm_part, int nb, double* v, double* z, double* zpart) {
   __shared__ double red[kThreads / 32];
+  __shared__ double scale;
   double s = 1.0;
   if (norm_part) {
-    const double t = warp_sum(norm_part, nb);
-    s = t > 0.0 ? 1.0 / sqrt(t) : 0.0;
+    if (threadIdx.x < 32) {
+      const double t = warp_sum(norm_part, nb);
+      if (threadIdx.x == 0) scale = t > 0.0 ? 1.0 / sqrt(t) : 0.0;
+    }
+    __syncthreads();
+    s = scale;
   }
   double acc = 0.0;
   for (int64_t t = blockIdx.x * int64_t(kThreads) + threadIdx.x; t < n; t += int64_t(gridDim.x) * kThreads) {
@@ -115,6 +120,7 @@ __global__ void direction_kernel(int64_t n, int Np, int Qp, const double* minv, 
       const double* col = src + k * Np * Qp + i;
       const double* row = minv + kn * Np * Qp + i;
       double a = 0.0;
+#pragma unroll 8
       for (int q = 0; q < Np; ++q) a = fma(row[size_t(q) * Qp], col[size_t(q) * Qp] * s, a);
       z[t] = a;
       acc = fma(a, a, acc);
@@ -128,10 +134,15 @@ __global__ void direction_kernel(int64_t n, int Np, int Qp, const double* minv, 
 
 __global__ void perturb_kernel(int64_t n, double eps, const double* zpart, int nb, const double* Y, const double* x,
                                double* step, double* out) {
+  __shared__ double step_s;
   double e = eps;
   if (zpart) {
-    const double t = sqrt(warp_sum(zpart, nb));
-    e = t > 0.0 ? eps / t : eps;
+    if (threadIdx.x < 32) {
+      const double t = warp_sum(zpart, nb);
+      if (threadIdx.x == 0) step_s = t > 0.0 ? eps / sqrt(t) : eps;
+    }
+    __syncthreads();
+    e = step_s;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) step[0] = e;
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
@@ -142,7 +153,10 @@ __global__ void project_first_kernel(int64_t n, int m, const double* x, const do
                                      const double* step, double dtg, const double* V, double* w, double* part) {
   int64_t lo, hi;
   chunk_of(n, lo, hi);
-  const double c = -dtg / step[0];
+  __shared__ double c_s;
+  if (threadIdx.x == 0) c_s = -dtg / step[0];  // one quotient per block: FP64 is slow here
+  __syncthreads();
+  const double c = c_s;
   for (int64_t i = lo + threadIdx.x; i < hi; i += kThreads) w[i] = x[i] + c * (Rp[i] - RY[i]);
   chunk_dots(n, lo, hi, m, V, w, part);  // every thread reads back only what it wrote
 }
@@ -164,6 +178,7 @@ __global__ void project_next_kernel(int64_t n, int m, const double* V, const dou
   double acc = 0.0;
   for (int64_t i = lo + threadIdx.x; i < hi; i += kThreads) {
     double t = 0.0;
+#pragma unroll 8
     for (int j = 0; j < m; ++j) t = fma(h[j], V[size_t(j) * n + i], t);
     const double wi = w[i] - t;
     w[i] = wi;
@@ -195,7 +210,7 @@ __global__ void set_geo_dt_kernel(int64_t K, int stride, int slot, double value,
 }  // namespace
 
 int blocks_of(int64_t n) {
-  const int64_t b = (n + 1023) / 1024;
+  const int64_t b = (n + 511) / 512;
   return int(b < 1 ? 1 : b > kMaxBlocks ? kMaxBlocks : b);
 }
 

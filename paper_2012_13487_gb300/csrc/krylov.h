@@ -9,7 +9,7 @@ namespace fedbm {
 namespace krylov {
 
 // Most blocks of a partial-sum reduction (one partial sum per block); a vector of
-// n values takes blocks_of(n), at least 1,024 values each.
+// n values takes blocks_of(n), at least 512 values each.
 constexpr int kMaxBlocks = 608;
 constexpr int kThreads = 256;
 int blocks_of(int64_t n);
