@@ -140,9 +140,10 @@ typedef struct fedbm_params {
   int32_t pipeline_stages; /* stage-kernel tile buffers per CTA: 1, or 2 to load
                               the next tile while computing one (0 = auto: the
                               warp-specialised form where it measured faster,
-                              i.e. FP32 or BF16 state with 256 padded velocities
-                              at degree 1-5 or 1024 at degree 1-3, when the tile
-                              arguments are 0 too; else 1);
+                              i.e. FP32 or BF16 state at degree 1-5 with 256 or
+                              1024 padded velocities, and from 512 up at degree
+                              3-5 (FP32 2-5), when the tile arguments are 0 too;
+                              else 1);
                               3 = the warp-specialised form: a producer warp
                               keeps a ring of one-element tiles filled (bulk
                               copies) for consumer warps, two velocities per
@@ -174,7 +175,8 @@ typedef struct fedbm_params {
                              of CTAs sharing each element (FP64, FP32, BF16
                              state): 0 = automatic (used when one CTA cannot
                              hold all velocities of an element, e.g. D2Q1089
-                             at degree 5 and 6), 1 = never, 2, 4 or 8 = that
+                             at degree 6, or at degree 5 on fewer elements
+                             than fill the SMs twice), 1 = never, 2, 4 or 8 = that
                              cluster size (EINVAL where it does not divide
                              the padded velocity count into multiples of 8) */
   int32_t rounding;      /* encode of the new BF16 deviation state: 0 = round to

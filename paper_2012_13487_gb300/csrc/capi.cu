@@ -457,26 +457,28 @@ int auto_cluster(const Group& g) {
 // eight consumer warps (two velocities per thread) and one producer warp.
 // Consumer groups per CTA of the automatic choice: one with 256 velocities (three
 // CTAs share an SM), three with 1,024 (one CTA per SM: two ring stages of each of
-// three CTAs would not fit).
-int ws_groups(const Group& g) { return g.Qp == 1024 ? 3 : 1; }
+// three CTAs would not fit), 0 for the wide form.
+int ws_groups(const Group& g) { return g.Qp == 256 ? 1 : g.Qp == 1024 && g.p <= 3 ? 3 : 0; }
 bool ws_available(const Group& g) { return stage_entry(g.p).ws_smem(g.store, g.Qp, ws_groups(g)) > 0; }
 
-// The untuned default takes the warp-specialised form wherever it exists from
-// degree 1 up (with 1,024 velocities up to degree 3: at degree 4 two ring stages of
-// FP32 state do not fit and BF16 spills).  One step of 20M values on the GB300, the
-// FMA kernel or the former warp-specialised one (one velocity per thread, eight
-// consumer warps) against this one, us at degree 1..5: 256 velocities FP32 484, 341,
-// 334, 349, 524 -> 361, 272, 274, 299, 399; BF16 751, 546, 433, 386, 471 -> 437, 329,
-// 322, 386, 438; 1,024 velocities FP32 736, 628, 837 -> 350, 298, 400; BF16 471, 527,
-// 636 -> 419, 306, 300.
+// The untuned default takes the warp-specialised form from degree 1 up with 256 and
+// 1,024 velocities (with 1,024 up to degree 3: above, two ring stages of FP32 state do
+// not fit with the face rows), else its wide form from 512 velocities up at degree 3-5,
+// FP32 state also at degree 2.  One step of 20M values on the GB300, us at degree 1..5,
+// the FMA or velocity-split kernel or the former warp-specialised one (one velocity per
+// thread, eight consumer warps) against this one: 256 velocities FP32 484, 341, 334, 349,
+// 524 -> 361, 272, 274, 299, 399; BF16 751, 546, 433, 386, 471 -> 437, 329, 322, 386, 438;
+// 1,024 velocities FP32 736, 628, 837, 768, 1164 -> 344, 292, 395, 447, 664; BF16 471,
+// 527, 636, 953, 1901 -> 411, 296, 293, 718, 1093; D2Q1089 FP32 661, 718, 969, 839, 1195
+// -> 783 (not taken), 579, 540, 486, 700; BF16 688, 687, 765, 991, 2105 -> 1010, 770 (not
+// taken), 703, 717, 1065.
 bool ws_default(const Group& g) {
-  if (!ws_available(g)) return false;
-  if (g.Qp == 1024) return g.p <= 3;
-  return g.p >= 1;
+  if (!ws_available(g) || g.p < 1) return false;
+  return ws_groups(g) > 0 || g.p >= 3 || (g.p == 2 && g.store == kStoreF32);
 }
 
-int configure_ws(Batch& b, Group& g, int groups = 0) {
-  if (groups == 0) groups = ws_groups(g);
+int configure_ws(Batch& b, Group& g, int groups = -1) {
+  if (groups < 0) groups = ws_groups(g);
   const StageEntry e = stage_entry(g.p);
   const size_t smem = e.ws_smem(g.store, g.Qp, groups);
   if (smem == 0)
@@ -1085,10 +1087,15 @@ int create_batch(const fedbm_case_desc* cd, int ncases, void* stream, Batch** ou
            // degree 5 likewise); tensor cores on request (tensor_cores = 1) or
            // when the autotuner times them faster
            const bool want_tc = g.tc_mode > 0;
-           // the velocity-split form on request, or when one CTA cannot hold
-           // an element's velocities (automatic mode)
+           // the velocity-split form on request, or (automatic mode) when one CTA of the
+           // FMA kernel cannot hold an element: it spreads a few elements over more SMs
+           // than there are of them.  With elements enough to fill the SMs the wide
+           // warp-specialised form takes over where it exists (D2Q1089, degree 5, FP32:
+           // 700 us against 1103 us for a step of 20M values)
            const bool too_big = stage_smem_bytes(g.p, g.store, std::max(1, epc), g.Qp, 1) > kMaxSmem;
-           const int ncl = g.vsplit >= 2 ? g.vsplit : (g.vsplit == 0 && too_big && !want_tc ? auto_cluster(g) : 0);
+           const bool wide = epc == 0 && tpb == 0 && st == 0 && g.K >= 2 * 152 && ws_default(g);
+           const int ncl = g.vsplit >= 2 ? g.vsplit
+                           : g.vsplit == 0 && too_big && !want_tc && !wide ? auto_cluster(g) : 0;
            if (ncl >= 2) {
              if ((r = configure_cluster(*b, g, ncl)) != FEDBM_OK) return r;
            } else if (want_tc) {

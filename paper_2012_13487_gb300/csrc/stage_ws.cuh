@@ -1,5 +1,6 @@
 // Warp-specialised form of the FMA stage kernel for 256 and 1,024 velocities (the
-// NC 16 x 16 and 32 x 32 sets), FP32 or BF16 deviation state.  Included by
+// NC 16 x 16 and 32 x 32 sets) and, as its wide form, any count from 512 up; FP32 or BF16
+// deviation state.  Included by
 // stage_impl.cuh inside its namespace; the arithmetic of a stage is that of the
 // FMA kernel.
 //
@@ -35,6 +36,12 @@
 // us with two CTAs of eight consumer warps per SM and 96 registers; one CTA of three
 // groups of four has the call at 14.1 ms instead of 18.7 ms.
 //
+// Wide form (QT == 0): the ring holds the element's state only, 94 KB at 1,120
+// velocities and degree 5, and the consumers read the neighbour traces they enter
+// through straight from L2, so that two stages fit an SM and an element's velocities
+// need not be split over a cluster: D2Q1089 at degree 5, 2,048 elements, a call of
+// three steps 8146 -> 5212 us against the velocity-split kernel.
+//
 // Every wait is bounded by %globaltimer.  Consumer warp 0 waits on the full
 // barrier and the consumers agree on the outcome with a reducing named
 // barrier; on a timeout the consumers record it and leave, the producer stops
@@ -48,27 +55,37 @@ namespace ws {
 // and the warps are dealt out over them: four warps each leave 128 registers per
 // thread, five 96, three 168.
 constexpr int kGroupThreads = 128;
-template <int G>
-__host__ __device__ constexpr int threads() { return G * kGroupThreads + 32; }
-template <int G>
-__host__ __device__ constexpr int ctas() { return G > 1 ? 1 : P <= 2 ? 4 : P <= 4 ? 3 : 2; }
-template <int G>
-__host__ __device__ constexpr int max_regs() { return G == 3 ? 128 : G == 2 ? 168 : P <= 2 ? 96 : P <= 4 ? 128 : 168; }
+template <int QT, int G>
+__host__ __device__ constexpr int ctas() { return QT == 0 || G > 1 ? 1 : P <= 2 ? 4 : P <= 4 ? 3 : 2; }
+template <int QT, int G>
+__host__ __device__ constexpr int max_regs() {
+  return QT == 0 ? 168 : G == 3 ? 128 : G == 2 ? 168 : P <= 2 ? 96 : P <= 4 ? 128 : 168;
+}
+// Consumer threads of a group.  The wide form (QT == 0: the velocity count is taken
+// from the arguments) has one group of at most eleven warps, three warps per
+// sub-partition with the producer, and as few as cover the velocities in the same
+// number of passes.
+template <int QT>
+__host__ __device__ constexpr int group_threads(int Q) {
+  if (QT > 0) return kGroupThreads;
+  const int pairs = Q / 2, passes = (pairs + 351) / 352;
+  return ((pairs + passes - 1) / passes + 31) / 32 * 32;
+}
+template <int QT, int G>
+__host__ __device__ constexpr int threads(int Q) { return G * group_threads<QT>(Q) + 32; }
 
 // named barrier of a group's N threads, OR-reducing a predicate
-template <int N>
-__device__ __forceinline__ bool consumers_sync_or(int id, bool pred) {
+__device__ __forceinline__ bool consumers_sync_or(int id, int N, bool pred) {
   uint32_t r;
   asm volatile(
       "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.red.or.pred q, %3, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
       : "=r"(r)
-      : "r"(pred ? 1u : 0u), "n"(N), "r"(id)
+      : "r"(pred ? 1u : 0u), "r"(N), "r"(id)
       : "memory");
   return r != 0;
 }
-template <int N>
-__device__ __forceinline__ void consumers_sync(int id) {
-  asm volatile("barrier.sync %1, %0;" ::"n"(N), "r"(id) : "memory");
+__device__ __forceinline__ void consumers_sync(int id, int N) {
+  asm volatile("barrier.sync %1, %0;" ::"r"(N), "r"(id) : "memory");
 }
 // plain arrive (release) of this thread on a barrier
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
@@ -91,8 +108,8 @@ __device__ __forceinline__ bool wait_for_number(const int* word, int want, uint6
 // (c0, c1, c2, c3, u_x, u_y, c6, c7; see node_record).
 constexpr int kRec = 16;
 
-// Shared-memory layout: per ring stage the state tile [NP][QT], the neighbour
-// face rows [NF][QT], the geometry, face codes and scales, two barriers; once per
+// Shared-memory layout: per ring stage the state tile [NP][Q], the neighbour face
+// rows [NF][Q] (not in the wide form), the geometry, face codes and scales, two barriers; once per
 // CTA the velocity rows (e_x, e_y, w and, for the deviation forms, w e_x, w e_y)
 // and two alternating sets of node records and wall numerators.
 struct Layout {
@@ -102,25 +119,25 @@ struct Layout {
 };
 __host__ __device__ constexpr size_t up(size_t b, size_t a) { return (b + a - 1) / a * a; }
 template <class ST, int QT, int G>
-__host__ __device__ constexpr Layout layout() {
+__host__ __device__ constexpr Layout layout(int Q) {
   Layout o{};
   constexpr size_t sb = sizeof(typename ST::S);
   size_t b = 0;
-  o.f = b;      b += up(size_t(NP) * QT * sb, 16);
-  o.tr = b;     b += up(size_t(NF) * QT * sb, 16);
+  o.f = b;      b += up(size_t(NP) * Q * sb, 16);
+  o.tr = b;     b += QT == 0 ? 0 : up(size_t(NF) * Q * sb, 16);
   o.geo = b;    b += up(size_t(kGeoStrideDev) * 4, 16);
   o.nbr = b;    b += 16;
   o.scale = b;  b += 16;
   o.nscale = b; b += 16;
   o.bars = b;   b += 16;                   // full, empty
   o.stage = up(b, 128);
-  const size_t fixed = up(size_t(ST::dev ? 5 : 3) * QT * 4, 16) + size_t(2 * G) * NP * kRec * 4 + up(size_t(2 * G) * NF * 4, 16);
+  const size_t fixed = up(size_t(ST::dev ? 5 : 3) * Q * 4, 16) + size_t(2 * G) * NP * kRec * 4 + up(size_t(2 * G) * NF * 4, 16);
   // as many stages as let the CTAs share an SM (1 KB of each is the system's), two to four
-  const size_t room = (size_t(228) * 1024) / ctas<G>() - 1024 - fixed;
+  const size_t room = (size_t(228) * 1024) / ctas<QT, G>() - 1024 - fixed;
   o.stages = int(room / o.stage);
   o.stages = o.stages < 2 ? 2 : o.stages > 4 * G ? 4 * G : o.stages;
   b = o.stage * o.stages;
-  o.vel = b;    b += up(size_t(ST::dev ? 5 : 3) * QT * 4, 16);
+  o.vel = b;    b += up(size_t(ST::dev ? 5 : 3) * Q * 4, 16);
   o.mom = b;    b += size_t(2 * G) * NP * kRec * 4;
   o.wn = b;     b += up(size_t(2 * G) * NF * 4, 16);
   o.end = b;
@@ -132,16 +149,19 @@ __host__ __device__ constexpr Layout layout() {
 // compensated modes take one accumulator update per chunk).
 template <class ST, class Acc, int QT>
 __device__ __forceinline__ void element_moments(const StageArgs<float>& a, const typename ST::S* row0, float sc,
-                                                const float* s_vel, float kappa, float* rec, int tid) {
-  constexpr int NTH = kGroupThreads;
-  constexpr int V = Vec16<ST>::N, NCH = QT / V;
-  constexpr int G = moment_lanes(NTH, 1, NCH);
+                                                const float* s_vel, float kappa, float* rec, int tid, int nth) {
+  const int Q = QT > 0 ? QT : a.Qp, NTH = QT > 0 ? kGroupThreads : nth;
+  constexpr int V = Vec16<ST>::N;
+  const int NCH = Q / V;
+  // lanes per node: a power of two that divides the chunks' loop evenly for the
+  // compile-time counts; the wide form's last round of chunks may be partial
+  const int G = moment_lanes(NTH, 1, NCH);
   constexpr bool kFast = std::is_same<Acc, AccF>::value;
   const int grp = tid / G, lane = tid % G;
   const bool third = a.eq_order == 3;
-  const float* t0 = s_vel + 2 * QT;                       // w (deviation forms)
-  const float* t1 = s_vel + (ST::dev ? 3 : 0) * QT;       // (w) e_x
-  const float* t2 = s_vel + (ST::dev ? 4 : 1) * QT;       // (w) e_y
+  const float* t0 = s_vel + 2 * Q;                       // w (deviation forms)
+  const float* t1 = s_vel + (ST::dev ? 3 : 0) * Q;       // (w) e_x
+  const float* t2 = s_vel + (ST::dev ? 4 : 1) * Q;       // (w) e_y
 #pragma unroll 1
   for (int base = 0; base < NP; base += NTH / G) {
     const int n = base + grp;
@@ -149,9 +169,10 @@ __device__ __forceinline__ void element_moments(const StageArgs<float>& a, const
     Acc m0, m1, m2;
     Pair p0 = 0, p1 = 0, p2 = 0;
     if (valid) {
-      const typename ST::S* row = row0 + n * QT;
+      const typename ST::S* row = row0 + n * Q;
 #pragma unroll 8
       for (int c = 0; c < NCH; c += G) {
+        if (QT == 0 && c + lane >= NCH) break;
         const int i = (c + lane) * V;
         const uint4 x = *reinterpret_cast<const uint4*>(row + i);
         const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
@@ -228,11 +249,14 @@ __device__ __forceinline__ void element_moments(const StageArgs<float>& a, const
 }
 
 template <class ST, int QT, int G>
-__global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<float> a) {
+__global__ void __maxnreg__((max_regs<QT, G>())) stage_kernel_ws(const StageArgs<float> a) {
   using S = typename ST::S;
-  constexpr Layout o = layout<ST, QT, G>();
-  constexpr int NC = kGroupThreads, NST = o.stages;
-  constexpr int kPasses = QT / (2 * NC);
+  constexpr bool kWide = QT == 0;
+  const int Q = kWide ? a.Qp : QT;
+  constexpr Layout oc = layout<ST, QT, G>(kWide ? 512 : QT);
+  const Layout o = kWide ? layout<ST, QT, G>(Q) : oc;
+  const int NC = kWide ? int(blockDim.x) - 32 : kGroupThreads, NST = kWide ? o.stages : oc.stages;
+  const int kPasses = (Q + 2 * NC - 1) / (2 * NC);
   extern __shared__ __align__(128) unsigned char smem[];
   const bool producer = threadIdx.x >= G * NC;
   const int group = producer ? 0 : threadIdx.x / NC;
@@ -253,13 +277,13 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
   auto empty = [&](int s) { return reinterpret_cast<uint64_t*>(smem + s * o.stage + o.bars) + 1; };
 
   pdl_launch_dependents();
-  for (int v = threadIdx.x; v < QT; v += threads<G>()) {
-    s_vel[v] = a.vel[kVelEx * QT + v];
-    s_vel[QT + v] = a.vel[kVelEy * QT + v];
-    s_vel[2 * QT + v] = a.vel[kVelW * QT + v];
+  for (int v = threadIdx.x; v < Q; v += blockDim.x) {
+    s_vel[v] = a.vel[kVelEx * Q + v];
+    s_vel[Q + v] = a.vel[kVelEy * Q + v];
+    s_vel[2 * Q + v] = a.vel[kVelW * Q + v];
     if constexpr (ST::dev) {
-      s_vel[3 * QT + v] = a.vel[kVelWex * QT + v];
-      s_vel[4 * QT + v] = a.vel[kVelWey * QT + v];
+      s_vel[3 * Q + v] = a.vel[kVelWex * Q + v];
+      s_vel[4 * Q + v] = a.vel[kVelWey * Q + v];
     }
   }
   if (threadIdx.x == 0) {
@@ -277,7 +301,7 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
   if (producer) {
     // ---- producer warp: element k = blockIdx.x + j gridDim.x into stage j % NST
     const int lane = threadIdx.x - G * NC;
-    const size_t row_bytes = size_t(QT) * sizeof(S);
+    const size_t row_bytes = size_t(Q) * sizeof(S);
     int issued = 0;  // elements issued
     for (int64_t k = blockIdx.x; k < K; k += gridDim.x, ++issued) {
       const int s = issued % NST;
@@ -300,27 +324,27 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
       if constexpr (ST::dev)
         if (lane == 0) st_scale(s)[0] = __ldg(a.scale_in + k);
       uint32_t bytes = lane == 0 ? uint32_t(NP * row_bytes + kGeoStrideDev * 4) + a.extra_tx : 0u;
-      for (int row = lane; row < NF; row += 32)
+      for (int row = lane; row < NF && !kWide; row += 32)
         if (__ldg(a.nbr + k * 3 + row / NFP) >= 0) bytes += uint32_t(row_bytes);
       mbar_arrive_expect_tx(full(s), bytes);
       if (lane == 0) {
-        bulk_load(st_f(s), fin + size_t(k) * NP * QT, uint32_t(NP * row_bytes), full(s));
+        bulk_load(st_f(s), fin + size_t(k) * NP * Q, uint32_t(NP * row_bytes), full(s));
         bulk_load(st_geo(s), a.geo + k * kGeoStrideDev, uint32_t(kGeoStrideDev * 4), full(s));
         // the residual goes straight to the consumers' registers; bring it into L2
         // while the ring is ahead of them
         if (read_res)
-          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.res + size_t(k) * NP * QT),
-                       "r"(uint32_t(NP * QT * 4))
+          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.res + size_t(k) * NP * Q),
+                       "r"(uint32_t(NP * Q * 4))
                        : "memory");
       }
-      for (int row = lane; row < NF; row += 32) {
+      for (int row = lane; row < NF && !kWide; row += 32) {
         const int fc = row / NFP, aa = row % NFP;
         const int code = __ldg(a.nbr + k * 3 + fc);
         if (code >= 0) {
           const int64_t kn = code >> 3;
           const int fn = (code >> 1) & 3;
           const int a2 = (code & 1) ? NFP - 1 - aa : aa;
-          bulk_load(st_tr(s) + size_t(row) * QT, fin + (size_t(kn) * NP + face_node(fn, a2)) * QT,
+          bulk_load(st_tr(s) + size_t(row) * Q, fin + (size_t(kn) * NP + face_node(fn, a2)) * Q,
                     uint32_t(row_bytes), full(s));
         }
       }
@@ -351,11 +375,13 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
     // latency overlaps the copies and the reductions; asked for an element ahead
     // instead they measured slower, 4126 us against 3812 us for the 8-step call)
     Pair rold[NP];
-    const size_t col0 = size_t(k) * NP * QT + 2 * tid;
+    const size_t col0 = size_t(k) * NP * Q + 2 * tid;
     auto load_residual = [&](int pass) {
 #pragma unroll
       for (int n = 0; n < NP; ++n)
-        rold[n] = read_res ? *reinterpret_cast<const Pair*>(a.res + col0 + size_t(n) * QT + pass * 2 * NC) : 0ull;
+        rold[n] = read_res && (!kWide || 2 * tid + pass * 2 * NC < Q)
+                      ? *reinterpret_cast<const Pair*>(a.res + col0 + size_t(n) * Q + pass * 2 * NC)
+                      : 0ull;
     };
     load_residual(0);
     bool ok = true;
@@ -364,10 +390,10 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
       // barrier may not even be complete, and the parity alone would let this
       // group pass.  Its own number in the stage says that it is: the producer
       // writes it after that element's release.
-      if constexpr (NST % G != 0) ok = wait_for_number(st_nbr(s) + 3, j, 2000000000ull);
+      if (G > 1 && NST % G != 0) ok = wait_for_number(st_nbr(s) + 3, j, 2000000000ull);
       ok = ok && mbar_wait_bounded(full(s), ph, 2000000000ull);
     }
-    if (consumers_sync_or<NC>(bar_id, !ok)) {
+    if (consumers_sync_or(bar_id, NC, !ok)) {
       if (tid == 0 && a.err) atomicExch(a.err, 1);
       return;  // the producer waits for its copies in flight before it leaves
     }
@@ -383,11 +409,11 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
     if (!a.collision) {
       for (int v = tid; v < NP * kRec; v += NC) rec[v] = 0.f;
     } else if (a.red == kRedFP64) {
-      element_moments<ST, AccD, QT>(a, st_f(s), sc, s_vel, kappa, rec, tid);
+      element_moments<ST, AccD, QT>(a, st_f(s), sc, s_vel, kappa, rec, tid, NC);
     } else if (a.red == kRedCompFP32) {
-      element_moments<ST, AccN, QT>(a, st_f(s), sc, s_vel, kappa, rec, tid);
+      element_moments<ST, AccN, QT>(a, st_f(s), sc, s_vel, kappa, rec, tid, NC);
     } else {
-      element_moments<ST, AccF, QT>(a, st_f(s), sc, s_vel, kappa, rec, tid);
+      element_moments<ST, AccF, QT>(a, st_f(s), sc, s_vel, kappa, rec, tid, NC);
     }
     if (a.wall_any) {
       // one warp per wall face node: sum over outgoing velocities of (e.n) f^-
@@ -397,31 +423,52 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
         const int code = nb[fc];
         if (!(code < 0 && __ldg(a.wall_den_inv + (-code - 1)) > 0.f)) continue;
         const float nxf = g[4 + 3 * fc], nyf = g[5 + 3 * fc];
-        const S* row = st_f(s) + face_node(fc, aa) * QT;
+        const S* row = st_f(s) + face_node(fc, aa) * Q;
         float acc = 0.f;
-        for (int v = lane; v < QT; v += 32) {
-          const float en = s_vel[v] * nxf + s_vel[QT + v] * nyf;
-          const float wv = ST::dev ? s_vel[2 * QT + v] : 0.f;
+        for (int v = lane; v < Q; v += 32) {
+          const float en = s_vel[v] * nxf + s_vel[Q + v] * nyf;
+          const float wv = ST::dev ? s_vel[2 * Q + v] : 0.f;
           if (en > 0) acc += en * decode<ST>(row[v], wv, wv * sc);
         }
         for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(kFull, acc, off);
         if (lane == 0) wn[trip] = acc;
       }
     }
-    consumers_sync<NC>(bar_id);
+    consumers_sync(bar_id, NC);
 
     // ---- residual and update of velocities i, i + 1, all nodes -----------------
 #pragma unroll 1
     for (int pass = 0; pass < kPasses; ++pass) {
-      const int i = 2 * tid + pass * 2 * NC;
-      const Pair ex = *reinterpret_cast<const Pair*>(s_vel + i), ey = *reinterpret_cast<const Pair*>(s_vel + QT + i);
-      const Pair w = *reinterpret_cast<const Pair*>(s_vel + 2 * QT + i);
+      const int i_own = 2 * tid + pass * 2 * NC;
+      // the wide form's last pass: lanes past the last velocity take the first along and
+      // store nothing
+      const bool own = !kWide || i_own < Q;
+      const int i = own ? i_own : 0;
+      if (kWide && !__any_sync(kFull, own)) continue;
+      const Pair ex = *reinterpret_cast<const Pair*>(s_vel + i), ey = *reinterpret_cast<const Pair*>(s_vel + Q + i);
+      const Pair w = *reinterpret_cast<const Pair*>(s_vel + 2 * Q + i);
       const Pair ws = ST::dev ? f2mul(w, both(sc)) : 0ull;
       if (kPasses > 1 && pass > 0) load_residual(pass);
       const S* fcol = st_f(s) + i;
+      // wide form: the neighbour traces straight from global memory (L2), for the faces
+      // the pair enters through, all in flight before the first is used
+      Pair tr[kWide ? NF : 1];
+      if constexpr (kWide) {
+#pragma unroll
+        for (int fc = 0; fc < 3; ++fc) {
+          const int code = nb[fc];
+          float e0, e1;
+          f2unpack(f2fma(ey, both(g[5 + 3 * fc]), f2mul(ex, both(g[4 + 3 * fc]))), e0, e1);
+          const bool in = code >= 0 && (fmaf(-ab, fabsf(e0), e0) != 0.f || fmaf(-ab, fabsf(e1), e1) != 0.f);
+          const S* base = fin + size_t(code >= 0 ? code >> 3 : 0) * NP * Q + i;
+#pragma unroll
+          for (int aa = 0; aa < NFP; ++aa)
+            tr[fc * NFP + aa] = in ? raw_pair<ST>(base + size_t(trace_node(code, aa)) * Q) : 0ull;
+        }
+      }
       Pair fr[NP];
 #pragma unroll
-      for (int m = 0; m < NP; ++m) fr[m] = value_pair<ST>(fcol + m * QT, w, ws);
+      for (int m = 0; m < NP; ++m) fr[m] = value_pair<ST>(fcol + m * Q, w, ws);
       // face fc carries flux for some velocity of this warp (warp-uniform; with
       // the upwind flux an outflow face's jump term is zero, so a face that is
       // outflow for all 64 velocities skips its traces and lift columns)
@@ -446,13 +493,17 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
         const Pair c = f2pack(c0, c1);
         if (code >= 0) {
           const Pair wsn = ST::dev ? f2mul(w, both(st_nscale(s)[fc])) : 0ull;
-          const S* trow = st_tr(s) + fc * NFP * QT + i;
+          const S* trow = st_tr(s) + fc * NFP * Q + i;
 #pragma unroll
-          for (int aa = 0; aa < NFP; ++aa)
-            flux[fc * NFP + aa] = f2mul(c, EoPacked::sub(fr[face_node(fc, aa)], value_pair<ST>(trow + aa * QT, w, wsn)));
+          for (int aa = 0; aa < NFP; ++aa) {
+            Pair t;
+            if constexpr (kWide) t = ST::dev ? f2fma(wsn, tr[fc * NFP + aa], w) : tr[fc * NFP + aa];
+            else t = value_pair<ST>(trow + aa * Q, w, wsn);
+            flux[fc * NFP + aa] = f2mul(c, EoPacked::sub(fr[face_node(fc, aa)], t));
+          }
         } else {
           const int slot = -code - 1;
-          const Pair fb = *reinterpret_cast<const Pair*>(a.wall_feq + size_t(slot) * QT + i);
+          const Pair fb = *reinterpret_cast<const Pair*>(a.wall_feq + size_t(slot) * Q + i);
           const float den_inv = __ldg(a.wall_den_inv + slot);
           const bool diffuse = den_inv > 0.f;
           const Pair fd = diffuse ? f2mul(both(den_inv), fb) : fb;
@@ -471,14 +522,14 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
       const Pair na = f2mul(f2mul(half_dt, both(-1.f)), EoPacked::add(ar, as)), nd = f2mul(half_dt, EoPacked::sub(ar, as));
       Pair invw = 0ull;
       if constexpr (ST::dev)  // BF16 keeps the element's power-of-two scale: q = (f - w) / (w s)
-        invw = f2mul(*reinterpret_cast<const Pair*>(a.vel + kVelInvW * QT + i), both(1.0f / sc));
+        invw = f2mul(*reinterpret_cast<const Pair*>(a.vel + kVelInvW * Q + i), both(1.0f / sc));
       const size_t col = col0 + size_t(pass) * 2 * NC;
       // update and write-back of node n from dt times its advection term
       // -(e . grad) f + LIFT (flux)
       eo_volume<M>([&](int n) { return fr[n]; }, na, nd, le, lo, [&](int n, Pair adv) {
         const ulonglong2* mm = reinterpret_cast<const ulonglong2*>(rec + n * kRec);
         const ulonglong2 m01 = mm[0], m23 = mm[1], mu = mm[2];
-        const Pair f = value_pair<ST>(fcol + n * QT, w, ws);
+        const Pair f = value_pair<ST>(fcol + n * Q, w, ws);
         const Pair eu = f2fma(ey, mu.y, f2mul(ex, mu.x));
         Pair feq = f2fma(ey, m23.x, f2fma(ex, m01.y, m01.x));
         feq = f2fma(eu, f2mul(m23.y, eu), feq);
@@ -488,8 +539,8 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
         }
         const Pair r = f2fma(w, feq, f2fma(neg_k, f, f2fma(rkA2, rold[n], adv)));
         const Pair fnew = f2fma(rkB2, r, f);
-        const size_t gi = col + size_t(n) * QT;
-        *reinterpret_cast<Pair*>(a.res + gi) = r;
+        const size_t gi = col + size_t(n) * Q;
+        if (own) *reinterpret_cast<Pair*>(a.res + gi) = r;
         if constexpr (ST::dev) {
           float q0, q1;
           f2unpack(f2mul(EoPacked::sub(fnew, w), invw), q0, q1);
@@ -500,9 +551,9 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
           } else {
             q = __floats2bfloat162_rn(q0, q1);
           }
-          *reinterpret_cast<__nv_bfloat162*>(fout + gi) = q;
+          if (own) *reinterpret_cast<__nv_bfloat162*>(fout + gi) = q;
         } else {
-          *reinterpret_cast<Pair*>(fout + gi) = fnew;
+          if (own) *reinterpret_cast<Pair*>(fout + gi) = fnew;
         }
       });
     }
@@ -518,7 +569,8 @@ __global__ void __maxnreg__((max_regs<G>())) stage_kernel_ws(const StageArgs<flo
 template <class ST, int QT, int G>
 __host__ __device__ constexpr bool exists() {
   if constexpr (ST::kind != kStoreF32 && ST::kind != kStoreBF16) return false;
-  else if constexpr (QT == 1024) return P <= 4 && layout<ST, QT, G>().end <= size_t(227) * 1024;
+  else if constexpr (QT == 0) return P >= 1 && P <= 5;
+  else if constexpr (QT == 1024) return P <= 4 && layout<ST, QT, G>(QT).end <= size_t(227) * 1024;
   else return P <= 5;
 }
 
@@ -529,23 +581,26 @@ struct Form {
   int threads = 0;
 };
 template <class ST, int QT, int G>
-Form form_as() {
+Form form_as(int Q) {
   Form f;
   if constexpr (exists<ST, QT, G>()) {
+    const Layout o = layout<ST, QT, G>(Q);
+    if (o.end > size_t(227) * 1024) return f;
     f.kernel = &stage_kernel_ws<ST, QT, G>;
-    f.smem = layout<ST, QT, G>().end;
-    f.threads = threads<G>();
+    f.smem = o.end;
+    f.threads = threads<QT, G>(Q);
   }
   return f;
 }
-// The form of this state and velocity count with `groups` consumer groups;
-// kernel == nullptr where there is none.
+// The form of this state and velocity count with `groups` consumer groups (0: the
+// wide form, one group sized to the velocities); kernel == nullptr where there is none.
 inline Form form(int store_kind, int Qp, int groups) {
   const bool f32 = store_kind == kStoreF32;
   if (!f32 && store_kind != kStoreBF16) return Form();
-  if (Qp == 1024 && groups == 3) return f32 ? form_as<StoreF32, 1024, 3>() : form_as<StoreBF16, 1024, 3>();
-  if (Qp == 256 && groups == 1) return f32 ? form_as<StoreF32, 256, 1>() : form_as<StoreBF16, 256, 1>();
-  if (Qp == 256 && groups == 2) return f32 ? form_as<StoreF32, 256, 2>() : form_as<StoreBF16, 256, 2>();
+  if (Qp == 1024 && groups == 3) return f32 ? form_as<StoreF32, 1024, 3>(Qp) : form_as<StoreBF16, 1024, 3>(Qp);
+  if (Qp == 256 && groups == 1) return f32 ? form_as<StoreF32, 256, 1>(Qp) : form_as<StoreBF16, 256, 1>(Qp);
+  if (Qp == 256 && groups == 2) return f32 ? form_as<StoreF32, 256, 2>(Qp) : form_as<StoreBF16, 256, 2>(Qp);
+  if (Qp >= 512 && groups == 0) return f32 ? form_as<StoreF32, 0, 1>(Qp) : form_as<StoreBF16, 0, 1>(Qp);
   return Form();
 }
 
