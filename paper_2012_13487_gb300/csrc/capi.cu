@@ -1482,9 +1482,9 @@ struct Implicit {
   double* hdev = nullptr;     // [m+2] dot results / combination coefficients
   double* zpart = nullptr;    // [kMaxBlocks] partial sums of |M^-1 v|^2
   double* step = nullptr;     // [1] step of the difference quotient
-  double* hcol = nullptr;     // [2 (m+1) + kMaxBlocks]: h of both passes, partial sums of |w|^2
-  double* hcol_host = nullptr;  // the same, pinned
-  cudaEvent_t column = nullptr; // hcol_host is complete
+  double* npart = nullptr;    // [kMaxBlocks] partial sums of |w|^2
+  double* hcol = nullptr;     // pinned host memory [2 (m+1) + kMaxBlocks]: h of both passes, npart
+  cudaEvent_t column = nullptr; // hcol is complete
   void* x32 = nullptr;        // FP32 state: FP32 copy of the input of R
   void* r32 = nullptr;        // FP32 state: FP32 residual register
   void* scratch = nullptr;    // stage-kernel state output (unused values)
@@ -1500,9 +1500,9 @@ struct Implicit {
 void free_implicit(Implicit& im) {
   void* bufs[] = {im.u0, im.Y, im.base, im.RY, im.G, im.d, im.w, im.Yp, im.Rp, im.V, im.k, im.partial, im.hdev,
                   im.x32, im.r32, im.scratch, im.geo_unit, im.minv, im.z, im.ops, im.fmask, im.zpart, im.step,
-                  im.hcol};
+                  im.npart};
   for (void* p : bufs) cudaFree(p);
-  cudaFreeHost(im.hcol_host);
+  cudaFreeHost(im.hcol);
   if (im.column) cudaEventDestroy(im.column);
   im = Implicit();
 }
@@ -1524,8 +1524,8 @@ int ensure_implicit(const Batch& b, const Group& g, Implicit& im, int m, int s) 
   FEDBM_CK(cudaMalloc(&im.zpart, krylov::kMaxBlocks * sizeof(double)));
   FEDBM_CK(cudaMalloc(&im.step, sizeof(double)));
   const size_t col = (size_t(2) * (m + 1) + krylov::kMaxBlocks) * sizeof(double);
-  FEDBM_CK(cudaMalloc(&im.hcol, col));
-  FEDBM_CK(cudaMallocHost(&im.hcol_host, col));
+  FEDBM_CK(cudaMalloc(&im.npart, krylov::kMaxBlocks * sizeof(double)));
+  FEDBM_CK(cudaHostAlloc(&im.hcol, col, cudaHostAllocMapped));
   FEDBM_CK(cudaEventCreateWithFlags(&im.column, cudaEventDisableTiming));
   const size_t rb = real_bytes(g.store);
   FEDBM_CK(cudaMalloc(&im.scratch, size_t(n) * rb));
@@ -1646,14 +1646,14 @@ int implicit_gmres(const Batch& b, const Group& g, Implicit& im, double dtg, dou
     const int nb = krylov::blocks_of(n);
     double* part1 = im.partial;
     double* part2 = im.partial + size_t(m + 1) * krylov::kMaxBlocks;
-    double *dh1 = im.hcol, *dh2 = im.hcol + (m + 1), *dnorm = im.hcol + 2 * (m + 1);
+    double *h1 = im.hcol, *h2 = im.hcol + (m + 1), *hnorm = im.hcol + 2 * (m + 1);
     // R(Y + e M^-1 v_j) for basis vector j (right preconditioning; M = I without a
     // preconditioner), v_j = w / |w| where the iteration before left it in w
     auto evaluate = [&](int j, bool from_w) -> int {
       double* vj = im.V + size_t(j) * n;
       if (precond || from_w)
         FEDBM_CK(krylov::direction(g.K, g.Np, g.Qp, precond ? im.minv : nullptr, from_w ? im.w : vj,
-                                   from_w ? dnorm : nullptr, vj, im.z, im.zpart, st));
+                                   from_w ? im.npart : nullptr, vj, im.z, im.zpart, st));
       FEDBM_CK(krylov::perturb(n, eps, precond ? im.zpart : nullptr, im.Y, precond ? im.z : vj, im.step, im.Yp, st));
       return implicit_rhs(b, g, im, im.Yp, im.Rp);
     };
@@ -1663,18 +1663,15 @@ int implicit_gmres(const Batch& b, const Group& g, Implicit& im, double dtg, dou
       // w = A M^-1 v_j and two passes of classical Gram-Schmidt against v_0 .. v_j
       const double* xj = precond ? im.z : im.V + size_t(j) * n;
       FEDBM_CK(krylov::project_first(n, j + 1, xj, im.Rp, im.RY, im.step, dtg, im.V, im.w, part1, st));
-      FEDBM_CK(krylov::project_next(n, j + 1, im.V, part1, dh1, im.w, part2, false, st));
-      FEDBM_CK(krylov::project_next(n, j + 1, im.V, part2, dh2, im.w, dnorm, true, st));
-      FEDBM_CK(cudaMemcpyAsync(im.hcol_host, im.hcol, (size_t(2) * (m + 1) + nb) * sizeof(double),
-                               cudaMemcpyDeviceToHost, st));
+      FEDBM_CK(krylov::project_next(n, j + 1, im.V, part1, h1, im.w, part2, nullptr, st));
+      FEDBM_CK(krylov::project_next(n, j + 1, im.V, part2, h2, im.w, im.npart, hnorm, st));
       FEDBM_CK(cudaEventRecord(im.column, st));
       // the next evaluation is queued before the host has looked at this column: it
       // covers the way to the host and back (not used if this column converges)
       if (j + 1 < m && total + 1 < max_iter && (rc = evaluate(j + 1, true)) != FEDBM_OK) return rc;
       FEDBM_CK(cudaEventSynchronize(im.column));
-      const double *h1 = im.hcol_host, *h2 = im.hcol_host + (m + 1);
       double hn = 0;
-      for (int q = 0; q < nb; ++q) hn += im.hcol_host[2 * (m + 1) + q];
+      for (int q = 0; q < nb; ++q) hn += hnorm[q];
       hn = std::sqrt(std::max(0.0, hn));
       ++cnt.gmres;
       for (int i = 0; i <= j; ++i) H[size_t(i) * m + j] = h1[i] + h2[i];

@@ -161,15 +161,15 @@ __global__ void project_first_kernel(int64_t n, int m, const double* x, const do
   chunk_dots(n, lo, hi, m, V, w, part);  // every thread reads back only what it wrote
 }
 
-__global__ void project_next_kernel(int64_t n, int m, const double* V, const double* part_in, double* h_out, double* w,
-                                    double* part_out, bool last) {
+__global__ void project_next_kernel(int64_t n, int m, const double* V, const double* part_in, double* h_host, double* w,
+                                    double* part_out, double* norm_host) {
   extern __shared__ double h[];
   __shared__ double red[kThreads / 32];
   for (int j = threadIdx.x >> 5; j < m; j += kThreads / 32) {
     const double t = warp_sum(part_in + size_t(j) * gridDim.x, gridDim.x);
     if ((threadIdx.x & 31) == 0) {
       h[j] = t;
-      if (blockIdx.x == 0) h_out[j] = t;
+      if (blockIdx.x == 0) h_host[j] = t;
     }
   }
   __syncthreads();
@@ -184,9 +184,12 @@ __global__ void project_next_kernel(int64_t n, int m, const double* V, const dou
     w[i] = wi;
     acc = fma(wi, wi, acc);
   }
-  if (last) {
+  if (norm_host) {
     acc = block_sum(acc, red);
-    if (threadIdx.x == 0) part_out[blockIdx.x] = acc;
+    if (threadIdx.x == 0) {
+      part_out[blockIdx.x] = acc;
+      norm_host[blockIdx.x] = acc;
+    }
   } else {
     chunk_dots(n, lo, hi, m, V, w, part_out);
   }
@@ -239,10 +242,10 @@ cudaError_t project_first(int64_t n, int m, const double* x, const double* Rp, c
   return cudaGetLastError();
 }
 
-cudaError_t project_next(int64_t n, int m, const double* V, const double* part_in, double* h_out, double* w,
-                         double* part_out, bool last, cudaStream_t st) {
-  project_next_kernel<<<blocks_of(n), kThreads, size_t(m) * sizeof(double), st>>>(n, m, V, part_in, h_out, w, part_out,
-                                                                                 last);
+cudaError_t project_next(int64_t n, int m, const double* V, const double* part_in, double* h_host, double* w,
+                         double* part_out, double* norm_host, cudaStream_t st) {
+  project_next_kernel<<<blocks_of(n), kThreads, size_t(m) * sizeof(double), st>>>(n, m, V, part_in, h_host, w, part_out,
+                                                                                 norm_host);
   return cudaGetLastError();
 }
 

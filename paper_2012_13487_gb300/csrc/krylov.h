@@ -61,10 +61,12 @@ cudaError_t perturb(int64_t n, double eps, const double* zpart, const double* Y,
 // w = x - dtg / step[0] (Rp - RY); part[j][blocks_of(n)] = partial <V_j, w> for j < m
 cudaError_t project_first(int64_t n, int m, const double* x, const double* Rp, const double* RY, const double* step,
                           double dtg, const double* V, double* w, double* part, cudaStream_t st);
-// h_out[j] = h_j = sum of part_in[j], w -= sum_j h_j V_j; then part_out[j] = partial
-// <V_j, w>, or with last: part_out[0] = partial <w, w>
-cudaError_t project_next(int64_t n, int m, const double* V, const double* part_in, double* h_out, double* w,
-                         double* part_out, bool last, cudaStream_t st);
+// h_host[j] = h_j = sum of part_in[j], w -= sum_j h_j V_j; then part_out[j] = partial
+// <V_j, w>, or, where norm_host is given, part_out[0] = norm_host = partial <w, w>.
+// h_host and norm_host are pinned host memory, written by the kernel itself: a copy
+// behind it would hold up the kernels queued after it.
+cudaError_t project_next(int64_t n, int m, const double* V, const double* part_in, double* h_host, double* w,
+                         double* part_out, double* norm_host, cudaStream_t st);
 
 }  // namespace krylov
 }  // namespace fedbm
