@@ -110,7 +110,7 @@ constexpr int kRec = 16;
 
 // Shared-memory layout: per ring stage the state tile [NP][Q], the neighbour face
 // rows [NF][Q] (not in the wide form), the geometry, face codes and scales, two barriers; once per
-// CTA the velocity rows (e_x, e_y, w and, for the deviation forms, w e_x, w e_y)
+// CTA the velocity rows (e_x, e_y, w and, for the deviation forms, w e_x, w e_y, 1/w)
 // and two alternating sets of node records and wall numerators.
 struct Layout {
   size_t stage, f, tr, geo, nbr, scale, nscale, bars;
@@ -131,13 +131,13 @@ __host__ __device__ constexpr Layout layout(int Q) {
   o.nscale = b; b += 16;
   o.bars = b;   b += 16;                   // full, empty
   o.stage = up(b, 128);
-  const size_t fixed = up(size_t(ST::dev ? 5 : 3) * Q * 4, 16) + size_t(2 * G) * NP * kRec * 4 + up(size_t(2 * G) * NF * 4, 16);
+  const size_t fixed = up(size_t(ST::dev ? 6 : 3) * Q * 4, 16) + size_t(2 * G) * NP * kRec * 4 + up(size_t(2 * G) * NF * 4, 16);
   // as many stages as let the CTAs share an SM (1 KB of each is the system's), two to four
   const size_t room = (size_t(228) * 1024) / ctas<QT, G>() - 1024 - fixed;
   o.stages = int(room / o.stage);
   o.stages = o.stages < 2 ? 2 : o.stages > 4 * G ? 4 * G : o.stages;
   b = o.stage * o.stages;
-  o.vel = b;    b += up(size_t(ST::dev ? 5 : 3) * Q * 4, 16);
+  o.vel = b;    b += up(size_t(ST::dev ? 6 : 3) * Q * 4, 16);
   o.mom = b;    b += size_t(2 * G) * NP * kRec * 4;
   o.wn = b;     b += up(size_t(2 * G) * NF * 4, 16);
   o.end = b;
@@ -284,6 +284,7 @@ __global__ void __maxnreg__((max_regs<QT, G>())) stage_kernel_ws(const StageArgs
     if constexpr (ST::dev) {
       s_vel[3 * Q + v] = a.vel[kVelWex * Q + v];
       s_vel[4 * Q + v] = a.vel[kVelWey * Q + v];
+      s_vel[5 * Q + v] = a.vel[kVelInvW * Q + v];
     }
   }
   if (threadIdx.x == 0) {
@@ -522,7 +523,7 @@ __global__ void __maxnreg__((max_regs<QT, G>())) stage_kernel_ws(const StageArgs
       const Pair na = f2mul(f2mul(half_dt, both(-1.f)), EoPacked::add(ar, as)), nd = f2mul(half_dt, EoPacked::sub(ar, as));
       Pair invw = 0ull;
       if constexpr (ST::dev)  // BF16 keeps the element's power-of-two scale: q = (f - w) / (w s)
-        invw = f2mul(*reinterpret_cast<const Pair*>(a.vel + kVelInvW * Q + i), both(1.0f / sc));
+        invw = f2mul(*reinterpret_cast<const Pair*>(s_vel + 5 * Q + i), both(1.0f / sc));
       const size_t col = col0 + size_t(pass) * 2 * NC;
       // update and write-back of node n from dt times its advection term
       // -(e . grad) f + LIFT (flux)
