@@ -205,6 +205,66 @@ __device__ __forceinline__ void eo_volume(F f, typename M::T na, typename M::T n
   }
 }
 
+// The same for the outputs q = part, part + nparts, .. only (a warp-uniform choice), with
+// the lift of those; every sum in the same order as above.
+template <class M, class F, class Fin>
+__device__ __forceinline__ void eo_part(F f, const typename M::T (&flux)[NF], typename M::T na, typename M::T nd,
+                                        int part, int nparts, Fin fin) {
+  using T = typename M::T;
+  constexpr EoPairs pr = eo_pairs();
+  T E[NE], O[at_least_1(NO)], g[NLE], h[NLO];
+#pragma unroll
+  for (int q = 0; q < NE; ++q) {
+    const T fa = f(pr.a[q]);
+    if (q < NO) {
+      const T fb = f(pr.b[q]);
+      E[q] = M::add(fa, fb);
+      O[q] = M::sub(fa, fb);
+    } else {
+      E[q] = fa;
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < NFP; ++a) {
+    g[a] = M::add(flux[a], flux[2 * NFP + a]);
+    h[a] = M::sub(flux[a], flux[2 * NFP + a]);
+  }
+#pragma unroll
+  for (int a = 0; a < NF1E; ++a) {
+    const int b = P - a;
+    g[NFP + a] = a == b ? flux[NFP + a] : M::add(flux[NFP + a], flux[NFP + b]);
+    if (a < NF1O) h[NFP + a] = M::sub(flux[NFP + a], flux[NFP + b]);
+  }
+#pragma unroll
+  for (int q = 0; q < NE; ++q) {
+    if (q % nparts != part) continue;
+    T le = M::zero(), se = M::zero(), dv = M::zero();
+#pragma unroll
+    for (int a = 0; a < NLE; ++a) le = M::fmac(EO_LE + q * NLE + a, g[a], le);
+#pragma unroll
+    for (int m = 0; m < NE; ++m) se = M::fmac(EO_SE + q * NE + m, E[m], se);
+#pragma unroll
+    for (int m = 0; m < NO; ++m)
+      if (!pr.hyp[q] || pr.hyp[m]) dv = M::fmac(EO_DO + q * NO + m, O[m], dv);
+    const T oe = M::fmat(na, se, M::fmat(nd, dv, le));
+    if (q < NO) {
+      T lo = M::zero(), so = M::zero(), de = M::zero();
+#pragma unroll
+      for (int a = 0; a < NLO; ++a) lo = M::fmac(EO_LO + q * NLO + a, h[a], lo);
+#pragma unroll
+      for (int m = 0; m < NO; ++m) so = M::fmac(EO_SO + q * NO + m, O[m], so);
+#pragma unroll
+      for (int m = 0; m < NE; ++m)
+        if (!pr.hyp[q] || pr.hyp[m]) de = M::fmac(EO_DE + q * NE + m, E[m], de);
+      const T oo = M::fmat(na, so, M::fmat(nd, de, lo));
+      fin(pr.a[q], M::add(oe, oo));
+      fin(pr.b[q], M::sub(oe, oo));
+    } else {
+      fin(pr.a[q], oe);
+    }
+  }
+}
+
 // Host side: the coefficients from the FP64 operators (row-major Dr, Ds
 // [Np][Np], LIFT [Np][3 Nfp]).
 inline void eo_coefficients(const double* Dr, const double* Ds, const double* LIFT, double (&t)[EO_N]) {

@@ -463,7 +463,7 @@ __device__ void tile_wall_numerators(const StageArgs<typename ST::R>& a, const t
   const int Qp = QT > 0 ? QT : a.Qp, tid = threadIdx.x, nth = blockDim.x;
   // lanes per wall node: a fixed number, so that the sum has one order whatever the tile
   const int G = Qp < 128 ? 8 : 32;
-  const int ngroups = nth / G, grp = tid / G, lane = tid % G;
+  const int grp = tid / G, lane = tid % G, step = G < 32 ? 32 / G : nth / G;
   const R* ex = s_vel + kVelEx * Qp;  // shared-memory copy of the velocity rows
   const R* ey = s_vel + kVelEy * Qp;
   const R* wv = s_vel + kVelW * Qp;
@@ -475,13 +475,16 @@ __device__ void tile_wall_numerators(const StageArgs<typename ST::R>& a, const t
       const int code = s_nbr[mine];
       wall = code < 0 && __ldg(a.wall_den_inv + (-code - 1)) > R(0);
     }
-    for (unsigned mask = __ballot_sync(kFull, wall); mask; mask &= mask - 1) {
+    int nth_wall = 0;
+    for (unsigned mask = __ballot_sync(kFull, wall); mask; mask &= mask - 1, ++nth_wall) {
+      // short rows: a warp per face; long ones: a warp per node of each face
+      if (G < 32 && nth_wall % (nth / 32) != tid / 32) continue;
       const int face = f0 + __ffs(mask) - 1, e = face / 3, fc = face - 3 * e;
       const R nxf = s_geo[e * kGeoStrideDev + 4 + 3 * fc];
       const R nyf = s_geo[e * kGeoStrideDev + 5 + 3 * fc];
       const R sc = ST::dev ? s_scale[e] : R(0);
-      for (int base = 0; base < NFP; base += ngroups) {
-        const int aa = base + grp;
+      for (int base = 0; base < NFP; base += step) {
+        const int aa = base + (G < 32 ? (tid & 31) / G : grp);
         R acc = 0;
         if (aa < NFP) {
           const int rs = aa * (P + 1) - aa * (aa - 1) / 2;
@@ -553,7 +556,10 @@ __host__ __device__ constexpr RecordForm record_form() {
 
 // Phase 4, FP64 state: residual, 2N-storage update and write-back of every
 // (element, velocity) value of the tile, one velocity of one element per thread, f
-// and the residual updated in place in shared memory.
+// and the residual updated in place in shared memory.  A tile of at most one warp's
+// items run by four warps or more (fewer elements than SMs) splits the nodes over the warps,
+// one per SM sub-partition: FP64 instructions take 64 cycles a warp there, and a stage is
+// one element's chain of them (8x8x2, degree 2, GH D2Q16: see auto_tile).
 template <class ST, int QT>
 __device__ __forceinline__ void value_update(const StageArgs<typename ST::R>& a,
                                              StageSmem<typename ST::R, typename ST::S>& sm, int ne, bool read_res) {
@@ -562,8 +568,12 @@ __device__ __forceinline__ void value_update(const StageArgs<typename ST::R>& a,
   const int Qp = QT > 0 ? QT : a.Qp;
   const R rkA = a.rkA, rkB = a.rkB, ab = a.ab;
   const bool third = a.eq_order == 3;
-  for (int item = threadIdx.x; item < ne * Qp; item += blockDim.x) {
-    const int e = item / Qp, i = item - e * Qp;
+  const bool split = a.epc * Qp <= 32 && blockDim.x >= 128;
+  const int part = split ? threadIdx.x / 32 : 0, nparts = split ? blockDim.x / 32 : 1;
+  const int first = split ? threadIdx.x % 32 : threadIdx.x, stride = split ? 32 : blockDim.x;
+  for (int item = first; split ? item < 32 : item < ne * Qp; item += stride) {
+    const bool own = item < ne * Qp;  // split: every thread comes to the barrier below
+    const int e = own ? item / Qp : 0, i = own ? item - e * Qp : 0;
     const R ex = a.vel[kVelEx * Qp + i], ey = a.vel[kVelEy * Qp + i], w = a.vel[kVelW * Qp + i];
     const R* g = sm.geo + e * kGeoStrideDev;
     const R dt = g[kGeoDt], inv_tau = g[kGeoInvTau];  // per element: cases of a batch differ
@@ -598,9 +608,7 @@ __device__ __forceinline__ void value_update(const StageArgs<typename ST::R>& a,
       }
     }
     using M = EoScalar<R, false>;
-    R le[NE], lo[at_least_1(NO)];
-    eo_lift<M>(flux, true, true, le, lo);
-    eo_volume<M>([&](int n) { return fr[n]; }, R(-0.5) * (ar + as), R(0.5) * (ar - as), le, lo, [&](int n, R adv) {
+    auto finish = [&](int n, R adv) {
       // f itself from shared memory again, which keeps the registers within two
       // resident CTAs of 256 threads
       const R f = frow[n * Qp];
@@ -609,7 +617,17 @@ __device__ __forceinline__ void value_update(const StageArgs<typename ST::R>& a,
       if (read_res) r = fma(rkA, rrow[n * Qp], r);
       rrow[n * Qp] = r;
       frow[n * Qp] = new_f<ST>(f, rkB, r);
-    });
+    };
+    auto value = [&](int n) { return fr[n]; };
+    const R na = R(-0.5) * (ar + as), nd = R(0.5) * (ar - as);
+    if (split) {
+      __syncthreads();  // every warp has read f before one updates its nodes
+      if (own) eo_part<M>(value, flux, na, nd, part, nparts, finish);
+    } else {
+      R le[NE], lo[at_least_1(NO)];
+      eo_lift<M>(flux, true, true, le, lo);
+      eo_volume<M>(value, na, nd, le, lo, finish);
+    }
   }
 }
 
