@@ -527,7 +527,7 @@ void auto_tile(const Group& g, int* epc, int* tpb) {
   const int spread = int(std::min<int64_t>(4, (K + 303) / 304));  // elements per CTA, two CTAs per SM
   if (g.Qp == 16 && f64) {
     *epc = !few ? 8 : K <= 304 ? 1 : 2;
-    *tpb = !few || K <= 152 ? 128 : K <= 1216 ? 64 : 32;
+    *tpb = !few || K <= 608 ? 128 : K <= 1216 ? 64 : 32;
   } else if (g.Qp == 16) {
     *epc = few ? spread : K < 32768 ? 4 : g.p <= 3 ? 8 : 4;
     if (K >= 32768 && g.p == 1 && g.store >= kStoreBF16) *epc = 16;
