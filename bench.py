@@ -111,8 +111,9 @@ def stage_kernel_sha():
     """Hash of the stage-kernel sources with comments and blank space removed,
     so that only code changes void a recorded ncu traffic figure."""
     h = hashlib.sha256()
-    for n in ("stage_impl.cuh", "stage_tc.cuh", "stage_cluster.cuh", "stage_ws.cuh", "device_common.cuh"):
-        with open(os.path.join(ROOT, "paper_2012_13487_gb300", "csrc", n)) as fh:
+    csrc = os.path.join(ROOT, "paper_2012_13487_gb300", "csrc")
+    for n in sorted(n for n in os.listdir(csrc) if n.startswith("stage_") and n.endswith(".cuh")) + ["device_common.cuh"]:
+        with open(os.path.join(csrc, n)) as fh:
             code = re.sub(r"//[^\n]*", "", fh.read())
         h.update(" ".join(code.split()).encode())
     return h.hexdigest()[:16]
