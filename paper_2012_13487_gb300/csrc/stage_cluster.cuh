@@ -146,10 +146,10 @@ __global__ void __launch_bounds__(kThreads, cl_min_blocks<ST>()) stage_kernel_cl
     for (int v = lane; v < ne * 3; v += 32) {
       const int code = __ldg(a.nbr + k0 * 3 + v);
       s_nbr[v] = code;
-      if constexpr (ST::dev) s_nscale[v] = code >= 0 ? __ldg(a.scale_in + (code >> 3)) : 0.f;
+      if constexpr (ST::dev) s_nscale[v] = code >= 0 ? a.scale_in[code >> 3] : 0.f;
     }
     if constexpr (ST::dev)
-      for (int v = lane; v < ne; v += 32) s_scale[v] = __ldg(a.scale_in + k0 + v);
+      for (int v = lane; v < ne; v += 32) s_scale[v] = a.scale_in[k0 + v];
     uint32_t bytes = lane == 0 ? uint32_t(size_t(ne) * kGeoStrideDev * sizeof(R)) + a.extra_tx : 0u;
     for (int row = lane; row < ne * NP; row += 32) bytes += uint32_t(row_bytes + (read_res ? rrow_bytes : 0));
     for (int row = lane; row < ne * NF; row += 32) {

@@ -224,7 +224,14 @@ __device__ __forceinline__ void fence_mbar_init() {
 // before it still runs its last CTAs.  It lets its own successor do the same at once
 // (launch_dependents), sets up its barriers and tables, which no earlier kernel
 // writes, and waits for the kernels before it to have finished, with their writes
-// visible, before it touches the state, the residual or the scales.
+// visible, before it touches the state, the residual or the scales.  Its lifetime so
+// overlaps its predecessors' writes of those three: they are read with ordinary loads
+// or bulk copies, never through the non-coherent path (__ldg), which is specified only
+// for data that nothing writes while the kernel lives and whose lines an older stage on
+// the same SM may have brought in.  Face codes, velocity rows and wall tables are
+// written by no kernel; the step counter of the stochastic rounding only by a kernel
+// between two steps, which starts after the last stage of one has finished and finishes
+// before the first of the next starts.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class R>
@@ -856,11 +863,11 @@ __device__ void issue_tile_loads(const StageArgs<typename ST::R>& a, StageSmem<t
   for (int v = lane; v < ne * 3; v += 32) {
     const int code = __ldg(a.nbr + k0 * 3 + v);
     sm.nbr[v] = code;
-    if constexpr (ST::dev) sm.nscale[v] = code >= 0 ? __ldg(a.scale_in + (code >> 3)) : 0.f;
+    if constexpr (ST::dev) sm.nscale[v] = code >= 0 ? a.scale_in[code >> 3] : 0.f;
   }
   if constexpr (ST::dev) {
     for (int v = lane; v < ne; v += 32) {
-      sm.scale[v] = __ldg(a.scale_in + k0 + v);
+      sm.scale[v] = a.scale_in[k0 + v];
       sm.dmax[v] = 0u;
     }
   }

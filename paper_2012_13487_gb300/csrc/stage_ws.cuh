@@ -320,10 +320,10 @@ __global__ void __maxnreg__((max_regs<QT, G>())) stage_kernel_ws(const StageArgs
       for (int v = lane; v < 3; v += 32) {
         const int code = __ldg(a.nbr + k * 3 + v);
         nb[v] = code;
-        if constexpr (ST::dev) st_nscale(s)[v] = code >= 0 ? __ldg(a.scale_in + (code >> 3)) : 0.f;
+        if constexpr (ST::dev) st_nscale(s)[v] = code >= 0 ? a.scale_in[code >> 3] : 0.f;
       }
       if constexpr (ST::dev)
-        if (lane == 0) st_scale(s)[0] = __ldg(a.scale_in + k);
+        if (lane == 0) st_scale(s)[0] = a.scale_in[k];
       uint32_t bytes = lane == 0 ? uint32_t(NP * row_bytes + kGeoStrideDev * 4) + a.extra_tx : 0u;
       for (int row = lane; row < NF && !kWide; row += 32)
         if (__ldg(a.nbr + k * 3 + row / NFP) >= 0) bytes += uint32_t(row_bytes);
