@@ -14,6 +14,7 @@
 #include "device_common.cuh"
 #include "fedbm.h"
 #include "host_setup.h"
+#include "implicit_space.h"
 #include "krylov.h"
 #include "stage_dispatch.h"
 #include "transfer.h"
@@ -1463,96 +1464,65 @@ bool make_tableau(const fedbm_implicit_params& ip, Tableau& t, std::string& err)
   return false;
 }
 
-// Device work space of the implicit solver of a single-group solver.
-struct Implicit {
-  int64_t n = 0;        // K * Np * Qp
-  int m = 0, s = 0;     // GMRES restart length, stages
-  double* u0 = nullptr;     // state at the start of the step
-  double* Y = nullptr;      // stage value (Newton iterate)
-  double* base = nullptr;   // u0 + dt sum_{j<i} a_ij k_j
-  double* RY = nullptr;     // R(Y)
-  double* G = nullptr;      // Newton residual, then the GMRES right-hand side -G
-  double* d = nullptr;      // Newton update
-  double* w = nullptr;      // GMRES work vector
-  double* Yp = nullptr;     // Y + eps v
-  double* Rp = nullptr;     // R(Y + eps v)
-  double* V = nullptr;      // GMRES basis [m+1][n]
-  double* k = nullptr;      // stage derivatives [s][n]
-  double* partial = nullptr;  // two of [m+1][kMaxBlocks]: the two Gram-Schmidt passes
-  double* hdev = nullptr;     // [m+2] dot results / combination coefficients
-  double* zpart = nullptr;    // [kMaxBlocks] partial sums of |M^-1 v|^2
-  double* step = nullptr;     // [1] step of the difference quotient
-  double* npart = nullptr;    // [kMaxBlocks] partial sums of |w|^2
-  double* hcol = nullptr;     // pinned host memory [2 (m+1) + kMaxBlocks]: h of both passes, npart
-  cudaEvent_t column = nullptr; // hcol is complete
-  void* x32 = nullptr;        // FP32 state: FP32 copy of the input of R
-  void* r32 = nullptr;        // FP32 state: FP32 residual register
-  void* scratch = nullptr;    // stage-kernel state output (unused values)
-  void* geo_unit = nullptr;   // geometry with dt = 1
-  // element-and-velocity block-Jacobi preconditioner (right preconditioning)
-  double* minv = nullptr;     // [K][Np][Np][Qp] block inverses of (I - dt gamma J)
-  double* z = nullptr;        // M^-1 v
-  double* ops = nullptr;      // FP64 Dr | Ds | LIFT of the degree
-  int* fmask = nullptr;       // [3][Nfp]
-  double minv_dtg = 0;        // dt gamma the inverses were built for (0 = none)
-};
+// Work space of the implicit solver of a single-group solver (implicit_space.h).
+struct Implicit : ImplicitSpace {};
 
-void free_implicit(Implicit& im) {
-  void* bufs[] = {im.u0, im.Y, im.base, im.RY, im.G, im.d, im.w, im.Yp, im.Rp, im.V, im.k, im.partial, im.hdev,
-                  im.x32, im.r32, im.scratch, im.geo_unit, im.minv, im.z, im.ops, im.fmask, im.zpart, im.step,
-                  im.npart};
-  for (void* p : bufs) cudaFree(p);
-  cudaFreeHost(im.hcol);
-  if (im.column) cudaEventDestroy(im.column);
-  im = Implicit();
+int space_device(void** p, size_t bytes) { return int(cudaMalloc(p, bytes)); }
+int space_pinned(void** p, size_t bytes) { return int(cudaHostAlloc(p, bytes, cudaHostAllocMapped)); }
+int space_event(void** e) {
+  return int(cudaEventCreateWithFlags(reinterpret_cast<cudaEvent_t*>(e), cudaEventDisableTiming));
+}
+const SpaceMemory kSpaceMemory = {&space_device,
+                                  &space_pinned,
+                                  &space_event,
+                                  [](void* p) { cudaFree(p); },
+                                  [](void* p) { cudaFreeHost(p); },
+                                  [](void* e) { cudaEventDestroy(static_cast<cudaEvent_t>(e)); }};
+
+// A request of the work space that failed: the runtime's pending error is taken, so
+// that the next launch check does not report it again.
+int space_failed(int rc) {
+  cudaGetLastError();
+  return fail(rc == int(cudaErrorMemoryAllocation) ? FEDBM_ENOMEM : FEDBM_ECUDA,
+              std::string("implicit work space: ") + cudaGetErrorString(cudaError_t(rc)));
 }
 
 int ensure_implicit(const Batch& b, const Group& g, Implicit& im, int m, int s) {
   const int64_t n = g.K * g.Np * g.Qp;
-  if (im.n == n && im.m >= m && im.s >= s) return FEDBM_OK;
-  free_implicit(im);
-  im.n = n;
-  im.m = m;
-  im.s = s;
-  const size_t vb = size_t(n) * sizeof(double);
-  double** vecs[] = {&im.u0, &im.Y, &im.base, &im.RY, &im.G, &im.d, &im.w, &im.Yp, &im.Rp};
-  for (double** v : vecs) FEDBM_CK(cudaMalloc(v, vb));
-  FEDBM_CK(cudaMalloc(&im.V, vb * size_t(m + 1)));
-  FEDBM_CK(cudaMalloc(&im.k, vb * size_t(s)));
-  FEDBM_CK(cudaMalloc(&im.partial, size_t(2) * (m + 1) * krylov::kMaxBlocks * sizeof(double)));
-  FEDBM_CK(cudaMalloc(&im.hdev, size_t(m + 2) * sizeof(double)));
-  FEDBM_CK(cudaMalloc(&im.zpart, krylov::kMaxBlocks * sizeof(double)));
-  FEDBM_CK(cudaMalloc(&im.step, sizeof(double)));
-  const size_t col = (size_t(2) * (m + 1) + krylov::kMaxBlocks) * sizeof(double);
-  FEDBM_CK(cudaMalloc(&im.npart, krylov::kMaxBlocks * sizeof(double)));
-  FEDBM_CK(cudaHostAlloc(&im.hcol, col, cudaHostAllocMapped));
-  FEDBM_CK(cudaEventCreateWithFlags(&im.column, cudaEventDisableTiming));
-  const size_t rb = real_bytes(g.store);
-  FEDBM_CK(cudaMalloc(&im.scratch, size_t(n) * rb));
-  if (g.store == kStoreF32) {
-    FEDBM_CK(cudaMalloc(&im.x32, size_t(n) * 4));
-    FEDBM_CK(cudaMalloc(&im.r32, size_t(n) * 4));
-  }
-  FEDBM_CK(cudaMalloc(&im.geo_unit, size_t(g.K) * kGeoStrideDev * rb));
-  FEDBM_CK(cudaMemcpyAsync(im.geo_unit, g.geo, size_t(g.K) * kGeoStrideDev * rb, cudaMemcpyDeviceToDevice, b.stream));
-  FEDBM_CK(krylov::set_geo_dt(g.K, kGeoStrideDev, kGeoDt, 1.0, im.geo_unit, int(rb), b.stream));
-  return FEDBM_OK;
+  const size_t rb = real_bytes(g.store), geo = size_t(g.K) * kGeoStrideDev * rb;
+  bool fresh = false;
+  int rc = im.reserve(kSpaceMemory, n, m, s, krylov::kMaxBlocks, rb, geo, &fresh);
+  if (rc) return space_failed(rc);
+  if (!fresh) return FEDBM_OK;
+  rc = int(cudaMemcpyAsync(im.geo_unit, g.geo, geo, cudaMemcpyDeviceToDevice, b.stream));
+  if (rc == 0) rc = int(krylov::set_geo_dt(g.K, kGeoStrideDev, kGeoDt, 1.0, im.geo_unit, int(rb), b.stream));
+  if (rc == 0) return FEDBM_OK;
+  im.release(kSpaceMemory);
+  return space_failed(rc);
 }
 
 // The block-Jacobi inverses for this dt gamma (built on first use, rebuilt
 // when dt gamma changes).
 int ensure_block_jacobi(const Batch& b, const Group& g, Implicit& im, double dtg) {
-  if (im.minv && im.minv_dtg == dtg) return FEDBM_OK;
-  if (!im.minv) {
-    FEDBM_CK(cudaMalloc(&im.minv, size_t(im.n) * g.Np * sizeof(double)));
-    FEDBM_CK(cudaMalloc(&im.z, size_t(im.n) * sizeof(double)));
-    std::vector<double> ops(g.ops.Dr);
-    ops.insert(ops.end(), g.ops.Ds.begin(), g.ops.Ds.end());
-    ops.insert(ops.end(), g.ops.LIFT.begin(), g.ops.LIFT.end());
-    int rc = upload_vec(ops, reinterpret_cast<void**>(&im.ops));
-    if (rc) return rc;
-    if ((rc = upload_vec(g.ops.fmask, reinterpret_cast<void**>(&im.fmask))) != FEDBM_OK) return rc;
+  const size_t nn = g.ops.Dr.size();
+  bool fresh = false;
+  int rc = im.reserve_blocks(kSpaceMemory, g.Np, 2 * nn + g.ops.LIFT.size(), g.ops.fmask.size(), &fresh);
+  if (rc) return space_failed(rc);
+  if (fresh) {
+    auto put = [&](void* dst, const void* src, size_t bytes) {
+      if (rc == 0) rc = int(cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice));
+    };
+    put(im.ops, g.ops.Dr.data(), nn * sizeof(double));
+    put(im.ops + nn, g.ops.Ds.data(), nn * sizeof(double));
+    put(im.ops + 2 * nn, g.ops.LIFT.data(), g.ops.LIFT.size() * sizeof(double));
+    put(im.fmask, g.ops.fmask.data(), g.ops.fmask.size() * sizeof(int32_t));
+    if (rc) {
+      im.release_blocks(kSpaceMemory);
+      return space_failed(rc);
+    }
   }
+  if (im.minv_dtg == dtg) return FEDBM_OK;
+  im.minv_dtg = 0;  // until the new inverses are queued
   FEDBM_CK(krylov::block_jacobi_build(g.K, g.Np, g.Nfp, g.Qp, g.geo, int(real_bytes(g.store)), g.vel64, im.ops,
                                       im.fmask, dtg, 2.0 * g.beta - 1.0, im.minv, b.stream));
   im.minv_dtg = dtg;
@@ -1665,11 +1635,11 @@ int implicit_gmres(const Batch& b, const Group& g, Implicit& im, double dtg, dou
       FEDBM_CK(krylov::project_first(n, j + 1, xj, im.Rp, im.RY, im.step, dtg, im.V, im.w, part1, st));
       FEDBM_CK(krylov::project_next(n, j + 1, im.V, part1, h1, im.w, part2, nullptr, st));
       FEDBM_CK(krylov::project_next(n, j + 1, im.V, part2, h2, im.w, im.npart, hnorm, st));
-      FEDBM_CK(cudaEventRecord(im.column, st));
+      FEDBM_CK(cudaEventRecord(static_cast<cudaEvent_t>(im.column), st));
       // the next evaluation is queued before the host has looked at this column: it
       // covers the way to the host and back (not used if this column converges)
       if (j + 1 < m && total + 1 < max_iter && (rc = evaluate(j + 1, true)) != FEDBM_OK) return rc;
-      FEDBM_CK(cudaEventSynchronize(im.column));
+      FEDBM_CK(cudaEventSynchronize(static_cast<cudaEvent_t>(im.column)));
       double hn = 0;
       for (int q = 0; q < nb; ++q) hn += hnorm[q];
       hn = std::sqrt(std::max(0.0, hn));
@@ -1720,7 +1690,7 @@ int implicit_gmres(const Batch& b, const Group& g, Implicit& im, double dtg, dou
 
 void free_implicit_of(Batch* b) {
   if (b->implicit) {
-    free_implicit(*b->implicit);
+    b->implicit->release(kSpaceMemory);
     delete b->implicit;
     b->implicit = nullptr;
   }
