@@ -408,7 +408,8 @@ int fedbm_batch_set_tiles(fedbm_batch* b, int32_t group, int32_t elems_per_cta,
  * onwards. */
 int fedbm_batch_set_tensor_cores(fedbm_batch* b, int32_t group, int32_t on);
 
-/* Tile autotuner: for every kernel group, time each candidate stage-kernel
+/* Tile autotuner: for every kernel group, time the configuration it has, the
+ * library's own choice and each candidate stage-kernel
  * tile (elements per CTA 1..32, threads per CTA 64/128/256, one or two
  * pipeline stages, the tensor-core form where the group has it and was not
  * created with tensor_cores = -1, and from 256 padded velocities up the
@@ -417,8 +418,9 @@ int fedbm_batch_set_tensor_cores(fedbm_batch* b, int32_t group, int32_t on);
  * velocity-split form because no FMA tile fits keep it.
  * The current state is left unchanged.  With a cache_path (NULL or "" for
  * none), results are read from and written to a JSON object keyed by device
- * name, degree, padded velocity count, precision, reduction and element
- * count.  Synchronous.  Errors: ECUDA if no candidate runs. */
+ * name, generation of the kernels, degree, padded velocity count, precision,
+ * reduction and element count; an entry also holds the time of the library's
+ * own choice in the same run (auto_us).  Synchronous.  Errors: ECUDA if no candidate runs. */
 int fedbm_batch_autotune(fedbm_batch* b, const char* cache_path, int32_t trials);
 int fedbm_autotune(fedbm_solver* s, const char* cache_path, int32_t trials);
 
