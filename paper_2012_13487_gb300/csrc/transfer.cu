@@ -34,10 +34,10 @@ struct Split {
 
 inline size_t up16(size_t b) { return (b + 15) / 16 * 16; }
 
-Split split_for(const Shape& sh, size_t table_bytes_per_q, size_t value_bytes) {
+Split split_for(const Shape& sh, size_t table_bytes, size_t value_bytes) {
   Split s;
   s.warp = sh.Np * sh.Qp <= kWarpValues;
-  s.tables = up16(table_bytes_per_q * size_t(sh.Q) + 4 * size_t(sh.Qp));
+  s.tables = up16(table_bytes);
   const size_t row = size_t(sh.Qp) * value_bytes;
   const int groups = s.warp ? kThreads / 32 : 1;
   s.rows = s.warp ? sh.Np : std::max(1, std::min(sh.Np, int(kStageBytes / row)));
@@ -77,33 +77,62 @@ struct Walk {
   }
 };
 
-// f - w relative to w, in FP32 with w = wh + wl: x - wh is exact where x is
-// within a factor of two of w, so the difference keeps FP32's relative
-// precision however small the deviation, without FP64 arithmetic per value.
-// An FP64 x that FP32 holds exactly takes the same path, so that an FP32 value
-// and the same value given in FP64 give the same bits; any other is subtracted
-// in FP64.  Weights below FP32's normal range take the FP64 quotient.
-struct DevTable {
-  const float *wh, *wl, *iw;  // canonical order; iw < 0: tiny weight, 0: weight 0
+// (f - w) / w rounded to FP32, as the FP64 quotient rounds, without FP64 arithmetic per
+// value (its rate is low here): w is held as three FP32 pieces, all its 53 bits, and 1/w
+// as two.  x - w is formed as a sum s + low whose rounding errors are kept (Knuth's
+// two-sum, The Art of Computer Programming vol. 2, 4.2.2, theorem B), its product with
+// 1/w likewise with the product's error from an FMA (Dekker 1971), so that what is
+// rounded in the last addition is off by about 2^-46.  Over 16 to 1,089 velocities and
+// deviations of 1e-7 to 1e6 the result is off by at most 1.0 units of 2^-24 |d|, as the FP64
+// quotient rounded to FP32 is; one difference and one product in plain FP32 had 3.6.
+// An FP64 x that FP32 holds exactly takes the same path, so that an FP32 value and the
+// same value given in FP64 give the same bits; any other is subtracted and scaled in
+// FP64.  Weights below 2^-96, whose last bits FP32's denormals do not hold, and results
+// out of its range take the FP64 quotient.
+constexpr double kTinyWeight = 1.262177448353619e-29;  // 2^-96
+struct __align__(16) DevRow {
+  float wh, wl, ih, il;  // ih < 0: tiny weight, 0: weight 0
 };
-__device__ __forceinline__ float difference(float x, const DevTable& t, int c) {
-  return (x - t.wh[c]) - t.wl[c];
+struct __align__(8) DevIndex {
+  float wll;
+  int at;  // internal index
+};
+struct DevTable {  // canonical order
+  const DevRow* row;
+  const DevIndex* index;
+  const double2* wide;  // FP64 input only: w, 1/w
+  const double* w64;    // internal order
+};
+__device__ __forceinline__ float two_difference(float a, float b, float& err) {
+  const float s = __fadd_rn(a, -b), t = __fadd_rn(s, -a);
+  err = __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -t)), -__fadd_rn(b, t));
+  return s;
 }
+// the same where |a| >= |b| or a = 0 (Dekker 1971)
+__device__ __forceinline__ float two_difference_ordered(float a, float b, float& err) {
+  const float s = __fadd_rn(a, -b);
+  err = -__fadd_rn(b, __fadd_rn(s, -a));
+  return s;
+}
+__device__ __noinline__ float deviation64(double x, double w) { return float((x - w) / w); }
 template <typename TIn>
-__device__ __forceinline__ float deviation(TIn x, const DevTable& t, int c, const double* w64, const int* perm) {
-  const float iw = t.iw[c];
-  if (iw <= 0.f) {
-    if (iw == 0.f) return 0.f;
-    const double w = w64[perm[c]];
-    return float((double(x) - w) / w);
-  }
+__device__ __forceinline__ float deviation(TIn x, const DevTable& t, int c, const DevIndex& at) {
+  const DevRow r = t.row[c];
+  if (r.ih <= 0.f) return r.ih == 0.f ? 0.f : deviation64(double(x), t.w64[at.at]);
+  const float xf = float(x);
   if constexpr (sizeof(TIn) == 8) {
-    const float xh = float(x);
-    if (__double_as_longlong(widen(xh)) != __double_as_longlong(x)) return float(x - w64[perm[c]]) * iw;
-    return difference(xh, t, c) * iw;
-  } else {
-    return difference(x, t, c) * iw;
+    if (__double_as_longlong(widen(xf)) != __double_as_longlong(x)) {
+      const double2 w = t.wide[c];
+      return float((x - w.x) * w.y);
+    }
   }
+  float ea, es;
+  // x - wh is 0 or, as a multiple of half a unit in wh's last place, at least |wl|
+  const float s = two_difference_ordered(two_difference(xf, r.wh, ea), r.wl, es);
+  const float low = __fadd_rn(__fadd_rn(ea, es), -at.wll);
+  const float p = __fmul_rn(s, r.ih), ep = fmaf(s, r.ih, -p);
+  const float d = __fadd_rn(p, __fadd_rn(ep, fmaf(s, r.il, __fmul_rn(low, r.ih))));
+  return fabsf(d) <= 3e38f ? d : deviation64(double(x), t.w64[at.at]);
 }
 
 // Encode: the caller's rows are read along the canonical order (consecutive
@@ -115,7 +144,10 @@ __device__ __forceinline__ float deviation(TIn x, const DevTable& t, int c, cons
 // with two FP64 divisions per value, scattered 2- and 4-byte stores and an
 // integer division per value (GB300, ncu): BF16 from FP32 input 15.3 ms at 335M
 // values (1,024 velocities), 1.45 ms at 31M (256) and 2.44 ms at 44M (16), FP32
-// from FP32 71 us at 31M; now 1.18 ms, 79 us, 122 us and 43 us.
+// from FP32 71 us at 31M; now (events around the call) 1.02 ms, 97 us, 142 us and 49 us.
+// Of these, the quotient with its rounding errors costs the 16-bit forms 15 us at 31M and
+// 17 us at 44M against a difference and a product in plain FP32, whose codes can round the
+// other way near a tie; from FP64 input BF16 takes 3.29 ms, 313 us and 439 us.
 template <class ST, typename TIn, bool kWarp>
 __global__ void __launch_bounds__(kThreads) encode_kernel(const TIn* __restrict__ in, void* out, float* scale,
                                                           const double* __restrict__ vel64,
@@ -125,19 +157,28 @@ __global__ void __launch_bounds__(kThreads) encode_kernel(const TIn* __restrict_
   using T = std::conditional_t<ST::dev, float, S>;  // staged values
   constexpr int V = 16 / int(sizeof(S));
   extern __shared__ __align__(16) unsigned char smem[];
-  int* perm = reinterpret_cast<int*>(smem);
-  float* tab = reinterpret_cast<float*>(perm + Qp);
-  DevTable dt{tab, tab + Q, tab + 2 * Q};
   const double* w64 = vel64 + 2 * Qp;
+  // tables in canonical order: the internal index, and for the deviation forms the weight's
+  // pieces (sized in encode_as)
+  DevRow* rows_w = reinterpret_cast<DevRow*>(smem);
+  DevIndex* index = reinterpret_cast<DevIndex*>(rows_w + Q);
+  double2* wide = reinterpret_cast<double2*>(smem + (size_t(24) * Q + 15) / 16 * 16);
+  int* perm = reinterpret_cast<int*>(smem);
+  const DevTable dt{rows_w, index, wide, w64};
   for (int c = threadIdx.x; c < Q; c += kThreads) {
     const int i = iperm[c];
-    perm[c] = i;
     if constexpr (ST::dev) {
       const double w = w64[i];
-      const float wh = float(w);
-      tab[c] = wh;
-      tab[Q + c] = float(w - double(wh));
-      tab[2 * Q + c] = !(w > 0) ? 0.f : w < 1e-30 ? -1.f : float(1.0 / w);
+      const float wh = float(w), wl = float(w - double(wh)), wll = float(w - double(wh) - double(wl));
+      const double iw = w > 0 ? 1.0 / w : 0.0;
+      const float ih = !(w > 0) ? 0.f : w < kTinyWeight ? -1.f : float(iw);
+      // the rest of 1/w from the FP64 residual of w ih, whose product has at most 77 bits:
+      // formed as an FMA
+      rows_w[c] = DevRow{wh, wl, ih, ih > 0.f ? float(fma(-w, double(ih), 1.0) * iw) : 0.f};
+      index[c] = DevIndex{wll, i};
+      if constexpr (sizeof(TIn) == 8) wide[c] = make_double2(w, iw);
+    } else {
+      perm[c] = i;
     }
   }
   const int G = kWarp ? 32 : kThreads;
@@ -177,7 +218,7 @@ __global__ void __launch_bounds__(kThreads) encode_kernel(const TIn* __restrict_
       if (!whole) {  // the element does not fit: its largest deviation in a pass of its own
         float m = 0.f;
         Walk w(lane, G, Q);
-        for (int j = lane; j < Np * Q; j += G, w.next()) m = fmaxf(m, fabsf(deviation(src[j], dt, w.c, w64, perm)));
+        for (int j = lane; j < Np * Q; j += G, w.next()) m = fmaxf(m, fabsf(deviation(src[j], dt, w.c, index[w.c])));
         set_scale(m);
       }
     }
@@ -197,13 +238,13 @@ __global__ void __launch_bounds__(kThreads) encode_kernel(const TIn* __restrict_
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           if (j + u * G >= n) break;
-          const int at = w.row * Qp + perm[w.c];
           if constexpr (ST::dev) {
-            const float d = deviation(x[u], dt, w.c, w64, perm);
+            const DevIndex at = index[w.c];
+            const float d = deviation(x[u], dt, w.c, at);
             m = fmaxf(m, fabsf(d));
-            buf[at] = d;
+            buf[w.row * Qp + at.at] = d;
           } else {
-            buf[at] = T(x[u]);
+            buf[w.row * Qp + perm[w.c]] = T(x[u]);
           }
           w.next();
         }
@@ -417,7 +458,10 @@ cudaError_t allow_smem(F kernel, size_t smem) {
 
 template <class ST, typename TIn>
 cudaError_t encode_as(const Shape& sh, const TIn* in, void* out, float* scale, cudaStream_t st) {
-  const Split s = split_for(sh, ST::dev ? 12 : 0, ST::dev ? 4 : sizeof(typename ST::S));
+  // internal indices; deviation forms: six words a velocity, for FP64 input w and 1/w behind them
+  const size_t q = size_t(sh.Q);
+  const size_t tables = !ST::dev ? 4 * q : sizeof(TIn) == 8 ? up16(24 * q) + 16 * q : 24 * q;
+  const Split s = split_for(sh, tables, ST::dev ? 4 : sizeof(typename ST::S));
   auto kernel = s.warp ? encode_kernel<ST, TIn, true> : encode_kernel<ST, TIn, false>;
   cudaError_t e = allow_smem(kernel, s.smem);
   if (e != cudaSuccess) return e;
@@ -428,7 +472,8 @@ cudaError_t encode_as(const Shape& sh, const TIn* in, void* out, float* scale, c
 
 template <class ST>
 cudaError_t decode_as(const Shape& sh, const void* in, const float* scale, double* out, cudaStream_t st) {
-  const Split s = split_for(sh, ST::dev ? 8 : 0, ST::dev ? 4 : sizeof(typename ST::S));
+  const size_t tables = (ST::dev ? 8 * size_t(sh.Q) : 0) + 4 * size_t(sh.Qp);
+  const Split s = split_for(sh, tables, ST::dev ? 4 : sizeof(typename ST::S));
   auto kernel = s.warp ? decode_kernel<ST, true> : decode_kernel<ST, false>;
   cudaError_t e = allow_smem(kernel, s.smem);
   if (e != cudaSuccess) return e;
