@@ -264,6 +264,7 @@ struct Group {
   std::vector<int> cases;
   int epc = 0, tpb = 0, nstages = 1, grid = 0;
   int ws_groups = 1;  // warp-specialised form: consumer groups per CTA
+  int lanes = 2;      // FMA kernel, FP32 arithmetic: velocities per thread
   size_t smem = 0;
   RefOps ops;
   VelocitySet vs;
@@ -354,7 +355,7 @@ cudaError_t launch_args(const Group& g, const void* args, cudaStream_t st, int g
   if (g.ncl > 1) return e.launch_cl(g.store, args, g.grid / g.ncl, g.ncl, g.smem, st);
   if (g.tc) return e.launch_tc(g.store, args, grid, g.smem, st);
   if (g.nstages == 3) return e.launch_ws(g.store, args, g.ws_groups, grid, g.smem, st);
-  return e.launch(g.store, args, grid, g.tpb, g.smem, st);
+  return e.launch(g.store, args, g.lanes, grid, g.tpb, g.smem, st);
 }
 
 cudaError_t launch_stage(const Group& g, int stage, int from, cudaStream_t st, int grid = 0) {
@@ -545,6 +546,25 @@ void auto_tile(const Group& g, int* epc, int* tpb) {
   }
 }
 
+// Velocities per thread of the FMA kernel's update (FP32 arithmetic) on a tile of epc
+// elements and tpb threads: two, the faster where the tile has a pair for every thread, as
+// the automatic tiles of enough elements have; one on a tile that a caller gives a thread
+// for every value, or a warp without a pair, and that has neighbours to share its SM with
+// (from 16 elements per SM up, or tiles of one element where they are more than two per
+// SM).  There idle threads would hold registers that keep other CTAs off the SM: one step of
+// 20M values, us, with one kernel of one velocity per thread (before), two, one: 256
+// velocities, 256 threads, FP32 degree 3, 4, 5 468, 450, 460; 532, 491, 769; 406, 377, 362;
+// 16 velocities, 8 elements on 128 threads, BF16 degree 4, 5 793, 753; 681, 822; 506, 526;
+// 36 velocities, 4 elements on 128 threads, degree 3 FP32, FP16 572, 803; 708, 915; 538,
+// 797.  Below those counts two was as fast or faster (36 velocities, 264 elements, 4 on 128
+// threads, degree 5 FP32 88; 53; 59).
+int stage_lanes(const Group& g, int epc, int tpb) {
+  const int values = epc * g.Qp, pairs = values / 2;
+  const bool idle = tpb >= values || tpb > (pairs + 31) / 32 * 32;
+  const bool shared = g.K >= 16 * 152 || (epc == 1 && g.K > 2 * 152);
+  return g.store != kStoreF64 && idle && shared ? 1 : 2;
+}
+
 // Tile shape, pipeline depth and persistent grid of a group's stage kernel.
 int configure_tiles(Batch& b, Group& g, int epc, int tpb, int stages) {
   if (stages == 3) {
@@ -576,16 +596,18 @@ int configure_tiles(Batch& b, Group& g, int epc, int tpb, int stages) {
   const StageEntry e = stage_entry(g.p);
   // the kernel's dynamic shared-memory limit stays at the maximum, so that
   // groups of one batch sharing this kernel with other tiles keep launching
-  FEDBM_CK(e.set_smem(g.store, g.Qp, kMaxSmem));
+  const int lanes = stage_lanes(g, e_pc, t_pb);
+  FEDBM_CK(e.set_smem(g.store, g.Qp, lanes, kMaxSmem));
   int nsm = 0;
   FEDBM_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b.device));
-  const int per_sm = e.occupancy(g.store, g.Qp, t_pb, smem);
+  const int per_sm = e.occupancy(g.store, g.Qp, lanes, t_pb, smem);
   if (per_sm < 1) return fail(FEDBM_EINVAL, "stage tile cannot be resident on an SM");
   const int64_t ntiles = (g.K + e_pc - 1) / e_pc;
   g.tc = 0;
   g.ncl = 0;
   g.epc = e_pc;
   g.tpb = t_pb;
+  g.lanes = lanes;
   g.nstages = nst;
   g.smem = smem;
   g.grid = int(std::min<int64_t>(ntiles, int64_t(per_sm) * nsm));

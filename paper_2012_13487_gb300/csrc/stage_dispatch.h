@@ -7,10 +7,11 @@
 namespace fedbm {
 
 struct StageEntry {
-  cudaError_t (*launch)(int store_kind, const void* args, int grid, int block, size_t smem, cudaStream_t st);
-  cudaError_t (*set_smem)(int store_kind, int Qp, size_t smem);
+  // lanes: velocities per thread of the FP32-arithmetic kernels, 1 or 2
+  cudaError_t (*launch)(int store_kind, const void* args, int lanes, int grid, int block, size_t smem, cudaStream_t st);
+  cudaError_t (*set_smem)(int store_kind, int Qp, int lanes, size_t smem);
   cudaError_t (*upload)(const double* Dr, const double* Ds, const double* LIFT);
-  int (*occupancy)(int store_kind, int Qp, int block, size_t smem);  // resident CTAs per SM
+  int (*occupancy)(int store_kind, int Qp, int lanes, int block, size_t smem);  // resident CTAs per SM
   // tensor-core form (FP32, BF16 or FP16 state; 128, 256 or 1024 velocities;
   // one element per CTA)
   size_t (*tc_smem)(int store_kind, int Qp);  // dynamic shared memory; 0 = no such form

@@ -23,7 +23,7 @@
 //      Dr, Ds, LIFT as instruction immediates (compile-time tables) or
 //      constant-memory operands of unrolled FMAs on the even and odd parts of f
 //      and of the flux (stage_eo.cuh); the FP32 and 16-bit states take two
-//      velocities per thread as packed FP32 pairs;
+//      velocities per thread as packed FP32 pairs, or one (stage_lanes);
 //   5. deviation forms only: per-element scale from max |f/w - 1|, encode;
 //   6. bulk-store the new state and residual tiles.
 #include "device_common.cuh"
@@ -498,9 +498,10 @@ __device__ void tile_wall_numerators(const StageArgs<typename ST::R>& a, const t
           const int node = (fc == 0) ? aa : (fc == 1 ? rs + (P - aa) : rs);
           const typename ST::S* row = s_f + (size_t(e) * NP + node) * Qp;
           for (int i = lane; i < Qp; i += G) {
-            const R en = ex[i] * nxf + ey[i] * nyf;
+            // the FMAs spelled out: left to the compiler they differ between kernels in the last bit
+            const R en = fma(ex[i], nxf, ey[i] * nyf);
             const R w = ST::dev ? wv[i] : R(0);  // the plain forms do not use (or hold) the w row
-            if (en > 0) acc += en * decode<ST>(row[i], w, w * sc);
+            if (en > 0) acc = fma(en, decode<ST>(row[i], w, w * sc), acc);
           }
         }
         for (int off = G >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(kFull, acc, off);
@@ -638,51 +639,132 @@ __device__ __forceinline__ void value_update(const StageArgs<typename ST::R>& a,
   }
 }
 
-// Two adjacent stored values as an FP32 pair, the lower velocity in the low half.
+// The velocities of a thread in the FP32-arithmetic update: two adjacent ones as packed
+// FP32 pairs (the lower in the low half), or one.  Every operation rounds a velocity the
+// same way in both, so that a value does not depend on which the tile has.  (A product
+// that is added or subtracted is written as the FMA: the assembler fuses a packed product
+// with the sum behind it in some places and not in others.)
 using Pair = unsigned long long;
-__device__ __forceinline__ Pair both(float x) { return f2pack(x, x); }
-template <class ST>
-__device__ __forceinline__ Pair raw_pair(const typename ST::S* p) {
-  if constexpr (ST::kind == kStoreBF16) {
-    const uint32_t q = *reinterpret_cast<const uint32_t*>(p);  // BF16: the upper half of an FP32
-    return f2pack(__uint_as_float(q << 16), __uint_as_float(q & 0xffff0000u));
-  } else if constexpr (ST::kind == kStoreF16) {
-    const float2 x = __half22float2(*reinterpret_cast<const __half2*>(p));
-    return f2pack(x.x, x.y);
-  } else {
-    return *reinterpret_cast<const Pair*>(p);
+template <int N>
+struct Lanes;
+template <>
+struct Lanes<2> : EoDual<kHaveOpsTable> {
+  static __device__ __forceinline__ T both(float x) { return f2pack(x, x); }
+  static __device__ __forceinline__ T mul(T x, T y) { return f2mul(x, y); }
+  static __device__ __forceinline__ T load(const float* p) { return *reinterpret_cast<const T*>(p); }
+  static __device__ __forceinline__ void store(float* p, T x) { *reinterpret_cast<T*>(p) = x; }
+  template <class F>
+  static __device__ __forceinline__ T map(T x, F f) {
+    float a, b;
+    f2unpack(x, a, b);
+    return f2pack(f(a), f(b));
   }
-}
+  static __device__ __forceinline__ bool any(T x) {
+    float a, b;
+    f2unpack(x, a, b);
+    return a != 0.f || b != 0.f;
+  }
+  static __device__ __forceinline__ float max_abs(T x) {
+    float a, b;
+    f2unpack(x, a, b);
+    return fmaxf(fabsf(a), fabsf(b));
+  }
+  // two adjacent values of a node record that holds every value twice
+  static __device__ __forceinline__ void record(const float* p, T& a, T& b) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
+    a = v.x;
+    b = v.y;
+  }
+  // stored values as FP32
+  template <class ST>
+  static __device__ __forceinline__ T raw(const typename ST::S* p) {
+    if constexpr (ST::kind == kStoreBF16) {
+      const uint32_t q = *reinterpret_cast<const uint32_t*>(p);  // BF16: the upper half of an FP32
+      return f2pack(__uint_as_float(q << 16), __uint_as_float(q & 0xffff0000u));
+    } else if constexpr (ST::kind == kStoreF16) {
+      const float2 x = __half22float2(*reinterpret_cast<const __half2*>(p));
+      return f2pack(x.x, x.y);
+    } else {
+      return *reinterpret_cast<const T*>(p);
+    }
+  }
+  using Code = __nv_bfloat162;
+  static __device__ __forceinline__ Code to_bf16(T x) {
+    float a, b;
+    f2unpack(x, a, b);
+    return __floats2bfloat162_rn(a, b);
+  }
+  // stochastic rounding; idx: the first value's index
+  static __device__ __forceinline__ Code to_bf16(T x, uint64_t idx, uint32_t step, uint32_t stage) {
+    float a, b;
+    f2unpack(x, a, b);
+    Code q;
+    q.x = bf16_round_stochastic(a, sr_hash(idx, step, stage));
+    q.y = bf16_round_stochastic(b, sr_hash(idx + 1, step, stage));
+    return q;
+  }
+};
+template <>
+struct Lanes<1> : EoScalar<float, kHaveOpsTable> {
+  static __device__ __forceinline__ T both(float x) { return x; }
+  // not contracted into FMAs, as the packed ones are not
+  static __device__ __forceinline__ T mul(T x, T y) { return __fmul_rn(x, y); }
+  static __device__ __forceinline__ T add(T x, T y) { return __fadd_rn(x, y); }
+  static __device__ __forceinline__ T sub(T x, T y) { return __fsub_rn(x, y); }
+  static __device__ __forceinline__ T load(const float* p) { return *p; }
+  static __device__ __forceinline__ void store(float* p, T x) { *p = x; }
+  template <class F>
+  static __device__ __forceinline__ T map(T x, F f) { return f(x); }
+  static __device__ __forceinline__ bool any(T x) { return x != 0.f; }
+  static __device__ __forceinline__ float max_abs(T x) { return fabsf(x); }
+  static __device__ __forceinline__ void record(const float* p, T& a, T& b) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    a = v.x;
+    b = v.z;
+  }
+  template <class ST>
+  static __device__ __forceinline__ T raw(const typename ST::S* p) {
+    if constexpr (ST::dev) return ST::to_r(*p);
+    else return *p;
+  }
+  using Code = __nv_bfloat16;
+  static __device__ __forceinline__ Code to_bf16(T x) { return __float2bfloat16_rn(x); }
+  static __device__ __forceinline__ Code to_bf16(T x, uint64_t idx, uint32_t step, uint32_t stage) {
+    return bf16_round_stochastic(x, sr_hash(idx, step, stage));
+  }
+};
 // decoded: f, or w + (w s) q
-template <class ST>
-__device__ __forceinline__ Pair value_pair(const typename ST::S* p, Pair w, Pair ws) {
-  if constexpr (ST::dev) return f2fma(ws, raw_pair<ST>(p), w);
-  else return raw_pair<ST>(p);
+template <class L, class ST>
+__device__ __forceinline__ typename L::T lane_value(const typename ST::S* p, typename L::T w, typename L::T ws) {
+  if constexpr (ST::dev) return L::fmat(ws, L::template raw<ST>(p), w);
+  else return L::template raw<ST>(p);
 }
 
 // Phase 4, FP32 arithmetic: residual, 2N-storage update and write-back of every
-// (element, velocity) value of the tile; each thread owns two adjacent velocities
-// of one element.  Additions, collision, update, loads and stores act on packed
+// (element, velocity) value of the tile; each thread owns N adjacent velocities of one
+// element.  With two, additions, collision, update, loads and stores act on packed
 // FP32 pairs, the contractions on their halves with the operators as immediates;
 // the time step is folded into the operators' factors, the flux coefficients and
 // the node records.  Bound by instruction issue: 16 velocities at degree 5 in FP32 took
 // 111 warp instructions per value and 239 us per stage of 44M values with one velocity
 // per thread (98 us for the bytes), the whole four-step call 5169 us, with two 3730 us;
-// BF16 5897 and 4630 us.  Plain forms and BF16 (kept element scale) update f in place
-// in shared memory; FP16 only tracks max |f/w - 1| per element (the encoding pass
+// BF16 5897 and 4630 us.  One velocity per thread serves tiles that a caller gives more
+// threads than pairs (stage_lanes).  Plain forms and BF16 (kept element scale) update f in
+// place in shared memory; FP16 only tracks max |f/w - 1| per element (the encoding pass
 // recomputes f with the new scale).
-template <class ST, int QT>
-__device__ __forceinline__ void pair_update(const StageArgs<float>& a, StageSmem<float, typename ST::S>& sm,
+template <class ST, int QT, int N>
+__device__ __forceinline__ void lane_update(const StageArgs<float>& a, StageSmem<float, typename ST::S>& sm,
                                             int64_t k0, int ne, bool read_res, float& dmax, int& emax) {
   using S = typename ST::S;
-  using M = EoDual<kHaveOpsTable>;
+  using L = Lanes<N>;
+  using T = typename L::T;
   constexpr bool kDirect = direct_traces<ST, QT>();
   constexpr bool kKeep = keeps_scale<ST>();
   constexpr bool kTrack = ST::dev && !kKeep;
   // outflow faces skipped per warp where a warp's items belong to one element
   constexpr bool kSkip = QT >= 128;
-  const int Qp = QT > 0 ? QT : a.Qp, Qv = Qp / 2;
-  const Pair rkA2 = both(a.rkA), rkB2 = both(a.rkB);
+  const int Qp = QT > 0 ? QT : a.Qp, Qv = Qp / N;
+  const T rkA2 = L::both(a.rkA), rkB2 = L::both(a.rkB), zero = L::zero();
   const float ab = a.ab;
   const bool third = a.eq_order == 3;
   const S* fin = static_cast<const S*>(a.f_in);
@@ -690,137 +772,135 @@ __device__ __forceinline__ void pair_update(const StageArgs<float>& a, StageSmem
   const bool sr = kKeep && a.sr_step != nullptr;
   const uint32_t sr_step = sr ? __ldg(a.sr_step) : 0u;
   for (int item = threadIdx.x; item < ne * Qv; item += blockDim.x) {
-    const int e = item / Qv, i = 2 * (item - e * Qv);
-    const Pair ex = *reinterpret_cast<const Pair*>(sm.vel + kVelEx * Qp + i);
-    const Pair ey = *reinterpret_cast<const Pair*>(sm.vel + kVelEy * Qp + i);
-    const Pair w = *reinterpret_cast<const Pair*>(sm.vel + kVelW * Qp + i);
+    const int e = item / Qv, i = N * (item - e * Qv);
+    const T ex = L::load(sm.vel + kVelEx * Qp + i), ey = L::load(sm.vel + kVelEy * Qp + i);
+    const T w = L::load(sm.vel + kVelW * Qp + i);
     const float* g = sm.geo + e * kGeoStrideDev;
     const float dt = g[kGeoDt];  // per element: cases of a batch differ
     const int* nb = sm.nbr + e * 3;
     // flux coefficients dt (e.n - ab |e.n|) Fscale / 2 of the three faces
-    Pair c[3];
+    T c[3];
     bool on[3], nz[3];
 #pragma unroll
     for (int fc = 0; fc < 3; ++fc) {
-      float e0, e1;
-      f2unpack(f2fma(ey, both(g[5 + 3 * fc]), f2mul(ex, both(g[4 + 3 * fc]))), e0, e1);
+      const T en = L::fmat(ey, L::both(g[5 + 3 * fc]), L::mul(ex, L::both(g[4 + 3 * fc])));
       const float h = 0.5f * dt * g[6 + 3 * fc];
-      float c0 = h * fmaf(-ab, fabsf(e0), e0), c1 = h * fmaf(-ab, fabsf(e1), e1);
-      if (nb[fc] < 0) {  // incoming velocities take the wall state; outgoing ones have no jump
-        c0 = e0 < 0.f ? c0 : 0.f;
-        c1 = e1 < 0.f ? c1 : 0.f;
-      }
-      c[fc] = f2pack(c0, c1);
-      nz[fc] = c0 != 0.f || c1 != 0.f;
+      const bool wall = nb[fc] < 0;  // incoming velocities take the wall state; outgoing ones have no jump
+      c[fc] = L::map(en, [&](float v) {
+        const float x = h * fmaf(-ab, fabsf(v), v);
+        return wall && !(v < 0.f) ? 0.f : x;
+      });
+      nz[fc] = L::any(c[fc]);
       on[fc] = kSkip ? __any_sync(__activemask(), nz[fc]) : true;
     }
     // 16 velocities: the traces of the faces with flux straight from global memory,
     // all of them in flight before the first is used
-    Pair tr[kDirect ? NF : 1];
+    T tr[kDirect ? NF : 1];
     if constexpr (kDirect) {
       const uint32_t* rows = reinterpret_cast<const uint32_t*>(sm.tr) + e * NF;
 #pragma unroll
       for (int fc = 0; fc < 3; ++fc)
 #pragma unroll
         for (int aa = 0; aa < NFP; ++aa)
-          tr[fc * NFP + aa] = nz[fc] && nb[fc] >= 0 ? raw_pair<ST>(fin + size_t(rows[fc * NFP + aa]) * QT + i) : 0ull;
+          tr[fc * NFP + aa] =
+              nz[fc] && nb[fc] >= 0 ? L::template raw<ST>(fin + size_t(rows[fc * NFP + aa]) * QT + i) : zero;
     }
-    const Pair ws = ST::dev ? f2mul(w, both(sm.scale[e])) : 0ull;
+    const T ws = ST::dev ? L::mul(w, L::both(sm.scale[e])) : zero;
     S* frow = sm.f + size_t(e) * NP * Qp + i;
     float* rrow = sm.res + size_t(e) * NP * Qp + i;
-    Pair fr[NP];
+    T fr[NP];
 #pragma unroll
-    for (int m = 0; m < NP; ++m) fr[m] = value_pair<ST>(frow + m * Qp, w, ws);
-    Pair flux[NF];
+    for (int m = 0; m < NP; ++m) fr[m] = lane_value<L, ST>(frow + m * Qp, w, ws);
+    T flux[NF];
 #pragma unroll
     for (int fc = 0; fc < 3; ++fc) {
       const int code = nb[fc];
       if constexpr (kSkip) {
 #pragma unroll
-        for (int aa = 0; aa < NFP; ++aa) flux[fc * NFP + aa] = 0ull;
+        for (int aa = 0; aa < NFP; ++aa) flux[fc * NFP + aa] = zero;
         if (!on[fc]) continue;
       }
       if (code >= 0) {
-        const Pair wsn = ST::dev ? f2mul(w, both(sm.nscale[e * 3 + fc])) : 0ull;
+        const T wsn = ST::dev ? L::mul(w, L::both(sm.nscale[e * 3 + fc])) : zero;
         const S* trow = sm.tr + size_t(e * NF + fc * NFP) * Qp + i;
 #pragma unroll
         for (int aa = 0; aa < NFP; ++aa) {
-          Pair t;
-          if constexpr (kDirect) t = ST::dev ? f2fma(wsn, tr[fc * NFP + aa], w) : tr[fc * NFP + aa];
-          else t = value_pair<ST>(trow + aa * Qp, w, wsn);
-          flux[fc * NFP + aa] = f2mul(c[fc], EoPacked::sub(fr[face_node(fc, aa)], t));
+          T t;
+          if constexpr (kDirect) t = ST::dev ? L::fmat(wsn, tr[fc * NFP + aa], w) : tr[fc * NFP + aa];
+          else t = lane_value<L, ST>(trow + aa * Qp, w, wsn);
+          flux[fc * NFP + aa] = L::mul(c[fc], L::sub(fr[face_node(fc, aa)], t));
         }
       } else {
         const int slot = -code - 1;  // wall slot: 4 * case + side
-        const Pair fb = *reinterpret_cast<const Pair*>(a.wall_feq + size_t(slot) * Qp + i);
+        const T fb = L::load(a.wall_feq + size_t(slot) * Qp + i);
         const float den_inv = __ldg(a.wall_den_inv + slot);
         const bool diffuse = den_inv > 0.f;
-        const Pair fd = f2mul(both(den_inv), fb);
+        const T fd = diffuse ? L::mul(L::both(den_inv), fb) : fb;
 #pragma unroll
         for (int aa = 0; aa < NFP; ++aa) {
-          const Pair fp = diffuse ? f2mul(both(sm.wn[e * NF + fc * NFP + aa]), fd) : fb;
-          flux[fc * NFP + aa] = f2mul(c[fc], EoPacked::sub(fr[face_node(fc, aa)], fp));
+          const float m = diffuse ? -sm.wn[e * NF + fc * NFP + aa] : -1.f;
+          flux[fc * NFP + aa] = L::mul(c[fc], L::fmat(L::both(m), fd, fr[face_node(fc, aa)]));
         }
       }
     }
-    Pair le[NE], lo[at_least_1(NO)];
-    eo_lift<M>(flux, on[0] || on[2], on[1], le, lo);
-    const Pair neg_k = both(-dt * g[kGeoInvTau]);
-    const Pair ar = f2fma(ey, both(g[2]), f2mul(ex, both(g[0]))), as = f2fma(ey, both(g[3]), f2mul(ex, both(g[1])));
-    const Pair na = f2mul(both(-0.5f * dt), EoPacked::add(ar, as)), nd = f2mul(both(0.5f * dt), EoPacked::sub(ar, as));
-    Pair invw = 0ull;
+    T le[NE], lo[at_least_1(NO)];
+    eo_lift<L>(flux, on[0] || on[2], on[1], le, lo);
+    const T neg_k = L::both(-dt * g[kGeoInvTau]);
+    const T ar = L::fmat(ey, L::both(g[2]), L::mul(ex, L::both(g[0])));
+    const T as = L::fmat(ey, L::both(g[3]), L::mul(ex, L::both(g[1])));
+    const T na = L::mul(L::both(-0.5f * dt), L::add(ar, as)), nd = L::mul(L::both(0.5f * dt), L::sub(ar, as));
+    T invw = zero;
     if constexpr (ST::dev)  // BF16 keeps the element's power-of-two scale: q = (f - w) / (w s)
-      invw = f2mul(*reinterpret_cast<const Pair*>(a.vel + kVelInvW * Qp + i),
-                   both(kKeep ? 1.0f / sm.scale[e] : 1.0f));
+      invw = L::mul(L::load(a.vel + kVelInvW * Qp + i), L::both(kKeep ? 1.0f / sm.scale[e] : 1.0f));
     float dloc = 0.f;
     // update and write-back of node n from dt times its advection term
     // -(e . grad) f + LIFT (flux)
-    eo_volume<M>([&](int n) { return fr[n]; }, na, nd, le, lo, [&](int n, Pair adv) {
-      Pair m0, m1, m2, m3, mx, my;
+    eo_volume<L>([&](int n) { return fr[n]; }, na, nd, le, lo, [&](int n, T adv) {
+      T m0, m1, m2, m3, mx, my;
       const int node = e * NP + n;
       if constexpr (kDirect) {
-        const ulonglong2* mm = reinterpret_cast<const ulonglong2*>(sm.mom + size_t(node) * kRecPairFloats);
-        const ulonglong2 u = mm[0], v = mm[1], x = mm[2];
-        m0 = u.x; m1 = u.y; m2 = v.x; m3 = v.y; mx = x.x; my = x.y;
+        const float* mm = sm.mom + size_t(node) * kRecPairFloats;
+        L::record(mm, m0, m1);
+        L::record(mm + 4, m2, m3);
+        L::record(mm + 8, mx, my);
       } else {
         const float4* mm = reinterpret_cast<const float4*>(sm.mom + size_t(node) * 8);
         const float4 u = mm[0], v = mm[1];
-        m0 = both(u.x); m1 = both(u.y); m2 = both(u.z); m3 = both(u.w); mx = both(v.x); my = both(v.y);
+        m0 = L::both(u.x); m1 = L::both(u.y); m2 = L::both(u.z); m3 = L::both(u.w);
+        mx = L::both(v.x); my = L::both(v.y);
       }
       // f itself from shared memory again: in registers next to its even and odd
       // parts it would cost a resident CTA
-      const Pair f = value_pair<ST>(frow + n * Qp, w, ws);
-      const Pair eu = f2fma(ey, my, f2mul(ex, mx));
-      Pair feq = f2fma(ey, m2, f2fma(ex, m1, m0));
-      feq = f2fma(eu, f2mul(m3, eu), feq);
+      const T f = lane_value<L, ST>(frow + n * Qp, w, ws);
+      const T eu = L::fmat(ey, my, L::mul(ex, mx));
+      T feq = L::fmat(ey, m2, L::fmat(ex, m1, m0));
+      feq = L::fmat(eu, L::mul(m3, eu), feq);
       if (third) {
         float2 t;
         if constexpr (kDirect) t = reinterpret_cast<const float2*>(sm.mom + size_t(a.epc) * NP * kRecPairFloats)[node];
         else t = reinterpret_cast<const float2*>(sm.mom + size_t(node) * 8)[3];
-        feq = f2fma(eu, f2fma(both(t.x), f2mul(eu, eu), both(t.y)), feq);
+        feq = L::fmat(eu, L::fmat(L::both(t.x), L::mul(eu, eu), L::both(t.y)), feq);
       }
-      Pair r = f2fma(w, feq, f2fma(neg_k, f, adv));
-      if (read_res) r = f2fma(rkA2, *reinterpret_cast<const Pair*>(rrow + n * Qp), r);
-      *reinterpret_cast<Pair*>(rrow + n * Qp) = r;
-      const Pair fnew = f2fma(rkB2, r, f);
+      T r = L::fmat(w, feq, L::fmat(neg_k, f, adv));
+      if (read_res) r = L::fmat(rkA2, L::load(rrow + n * Qp), r);
+      L::store(rrow + n * Qp, r);
+      const T fnew = L::fmat(rkB2, r, f);
       if constexpr (ST::dev) {
-        float q0, q1;
-        f2unpack(f2mul(EoPacked::sub(fnew, w), invw), q0, q1);
+        const T q = L::mul(L::sub(fnew, w), invw);
         if constexpr (kTrack) {
-          dloc = fmaxf(dloc, fmaxf(fabsf(q0), fabsf(q1)));
+          dloc = fmaxf(dloc, L::max_abs(q));
         } else {
-          __nv_bfloat162 q;
+          typename L::Code code;
           if (sr) {
             const uint64_t gi = (uint64_t(k0 + e) * NP + n) * uint64_t(Qp) + uint64_t(i);
-            q.x = bf16_round_stochastic(q0, sr_hash(gi, sr_step, uint32_t(a.sr_stage)));
-            q.y = bf16_round_stochastic(q1, sr_hash(gi + 1, sr_step, uint32_t(a.sr_stage)));
+            code = L::to_bf16(q, gi, sr_step, uint32_t(a.sr_stage));
           } else {
-            q = __floats2bfloat162_rn(q0, q1);
+            code = L::to_bf16(q);
           }
-          *reinterpret_cast<__nv_bfloat162*>(frow + n * Qp) = q;
+          *reinterpret_cast<typename L::Code*>(frow + n * Qp) = code;
         }
       } else {
-        *reinterpret_cast<Pair*>(frow + n * Qp) = fnew;
+        L::store(frow + n * Qp, fnew);
       }
     });
     if constexpr (kTrack) {
@@ -834,12 +914,14 @@ __device__ __forceinline__ void pair_update(const StageArgs<float>& a, StageSmem
   }
 }
 
-// Registers per thread of the FMA kernel, so that the unrolled update does not
-// spill and the tile's shared memory, not the register file, bounds the resident
-// CTAs (tiles have 64 to 256 threads).
-template <class ST, int QT>
+// Registers per thread of the FMA kernel, so that the tile's shared memory, not the
+// register file, bounds the resident CTAs and the unrolled update spills little: at most
+// 48 bytes in FP32 arithmetic (FP16, degree 5), 56, 32 and 108 bytes stored in FP64 at degree
+// 3, 4 and 5.  One velocity per thread needs fewer: 80 let three CTAs of 256 threads share
+// an SM (degree 4, 256 velocities, FP32, a step of 20M values 377 us, with 128 461 us).
+template <class ST, int N>
 __host__ __device__ constexpr int stage_max_regs() {
-  return sizeof(typename ST::R) == 8 ? 128 : P <= 2 ? 96 : P <= 4 ? 128 : 168;
+  return sizeof(typename ST::R) == 8 ? 128 : N == 1 ? 80 : P <= 2 ? 96 : P <= 4 ? 128 : 168;
 }
 
 // Bulk copies (TMA) of one tile into a shared-memory stage, issued by warp 0:
@@ -913,8 +995,9 @@ __device__ void issue_tile_loads(const StageArgs<typename ST::R>& a, StageSmem<t
 // shared-memory stages, loading tile j+1 while it computes tile j.
 // QT > 0: the padded velocity count is the compile-time constant QT (all
 // shared-memory strides become immediate offsets); QT = 0: taken from a.Qp.
-template <class ST, int QT>
-__global__ void __maxnreg__((stage_max_regs<ST, QT>())) stage_kernel(const StageArgs<typename ST::R> a) {
+// N: velocities per thread of the update (FP32 arithmetic; the FP64 state has one).
+template <class ST, int QT, int N>
+__global__ void __maxnreg__((stage_max_regs<ST, N>())) stage_kernel(const StageArgs<typename ST::R> a) {
   using R = typename ST::R;
   using S = typename ST::S;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -1037,7 +1120,7 @@ __global__ void __maxnreg__((stage_max_regs<ST, QT>())) stage_kernel(const Stage
     float dmax = 0.f;  // deviation forms: running max |f/w - 1| of element emax
     int emax = -1;
     if constexpr (sizeof(R) == 8) value_update<ST, QT>(a, sm, ne, read_res);
-    else pair_update<ST, QT>(a, sm, k0, ne, read_res, dmax, emax);
+    else lane_update<ST, QT, N>(a, sm, k0, ne, read_res, dmax, emax);
 
     // ---- 5. deviation forms: the kept scale (BF16), or the new per-element
     // scale and the encoding in place (FP16) ------------------------------------
@@ -1097,12 +1180,6 @@ __global__ void __maxnreg__((stage_max_regs<ST, QT>())) stage_kernel(const Stage
 #include "stage_cluster.cuh"
 #include "stage_ws.cuh"
 
-template <class ST, int QT>
-cudaError_t launch_one(const void* args, int grid, int block, size_t smem, cudaStream_t st) {
-  const auto& a = *static_cast<const StageArgs<typename ST::R>*>(args);
-  return launch_stage_kernel(&stage_kernel<ST, QT>, grid, block, smem, st, a);
-}
-
 // Velocity counts with a specialised kernel (the GH D2Q16 and NC 16x16 /
 // 32x32 sets; the larger sets only at the degrees their workloads use, which
 // keeps the high-degree translation units quick to compile); other counts use
@@ -1111,82 +1188,55 @@ constexpr bool specialised_q(int Qp) {
   return (Qp == 16 && P <= 5) || (Qp == 256 && P <= 5) || (Qp == 1024 && P <= 4);
 }
 
-template <class ST>
-cudaError_t launch_q(int Qp, const void* args, int grid, int block, size_t smem, cudaStream_t st) {
+// fn(kernel) for the stage kernel of this state, velocity count and velocities per thread.
+// (One velocity per thread needs more threads than pairs: never 1,024 velocities.)
+template <class ST, int N, class Fn>
+auto with_stage_kernel(int Qp, Fn fn) {
   if constexpr (ST::kind != kStoreF64) {
     if constexpr (specialised_q(16))
-      if (Qp == 16) return launch_one<ST, 16>(args, grid, block, smem, st);
+      if (Qp == 16) return fn(&stage_kernel<ST, 16, N>);
     if constexpr (specialised_q(256))
-      if (Qp == 256) return launch_one<ST, 256>(args, grid, block, smem, st);
-    if constexpr (specialised_q(1024))
-      if (Qp == 1024) return launch_one<ST, 1024>(args, grid, block, smem, st);
+      if (Qp == 256) return fn(&stage_kernel<ST, 256, N>);
+    if constexpr (specialised_q(1024) && N == 2)
+      if (Qp == 1024) return fn(&stage_kernel<ST, 1024, N>);
   }
-  return launch_one<ST, 0>(args, grid, block, smem, st);
+  return fn(&stage_kernel<ST, 0, N>);
 }
-
-template <class ST>
-int occupancy_q(int Qp, int block, size_t smem) {
-  int n = 0;
-  auto occ = [&](auto kernel) { cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, block, smem); };
-  if constexpr (ST::kind != kStoreF64) {
-    if constexpr (specialised_q(16))
-      if (Qp == 16) { occ(stage_kernel<ST, 16>); return n; }
-    if constexpr (specialised_q(256))
-      if (Qp == 256) { occ(stage_kernel<ST, 256>); return n; }
-    if constexpr (specialised_q(1024))
-      if (Qp == 1024) { occ(stage_kernel<ST, 1024>); return n; }
+template <class Fn>
+auto with_f32_kernel(int store_kind, int Qp, int lanes, Fn fn) {
+  switch (store_kind) {
+    case kStoreF32: return lanes == 1 ? with_stage_kernel<StoreF32, 1>(Qp, fn) : with_stage_kernel<StoreF32, 2>(Qp, fn);
+    case kStoreBF16: return lanes == 1 ? with_stage_kernel<StoreBF16, 1>(Qp, fn) : with_stage_kernel<StoreBF16, 2>(Qp, fn);
+    default: return lanes == 1 ? with_stage_kernel<StoreF16, 1>(Qp, fn) : with_stage_kernel<StoreF16, 2>(Qp, fn);
   }
-  occ(stage_kernel<ST, 0>);
-  return n;
 }
 
 // resident CTAs per SM of the kernel a launch with these parameters uses
-int occupancy(int store_kind, int Qp, int block, size_t smem) {
-  switch (store_kind) {
-    case kStoreF64: return occupancy_q<StoreF64>(Qp, block, smem);
-    case kStoreF32: return occupancy_q<StoreF32>(Qp, block, smem);
-    case kStoreBF16: return occupancy_q<StoreBF16>(Qp, block, smem);
-    case kStoreF16: return occupancy_q<StoreF16>(Qp, block, smem);
-  }
-  return 0;
+int occupancy(int store_kind, int Qp, int lanes, int block, size_t smem) {
+  int n = 0;
+  auto occ = [&](auto kernel) { return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, block, smem); };
+  if (store_kind == kStoreF64) with_stage_kernel<StoreF64, 1>(Qp, occ);
+  else with_f32_kernel(store_kind, Qp, lanes, occ);
+  return n;
 }
 
-template <class ST>
-cudaError_t set_smem_q(int Qp, size_t smem) {
+cudaError_t launch(int store_kind, const void* args, int lanes, int grid, int block, size_t smem, cudaStream_t st) {
+  if (store_kind == kStoreF64) {
+    const auto& a = *static_cast<const StageArgs<double>*>(args);
+    return with_stage_kernel<StoreF64, 1>(
+        a.Qp, [&](auto kernel) { return launch_stage_kernel(kernel, grid, block, smem, st, a); });
+  }
+  const auto& a = *static_cast<const StageArgs<float>*>(args);
+  return with_f32_kernel(store_kind, a.Qp, lanes,
+                         [&](auto kernel) { return launch_stage_kernel(kernel, grid, block, smem, st, a); });
+}
+
+cudaError_t set_smem(int store_kind, int Qp, int lanes, size_t smem) {
   auto set = [smem](auto kernel) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   };
-  if constexpr (ST::kind != kStoreF64) {
-    if constexpr (specialised_q(16))
-      if (Qp == 16) return set(stage_kernel<ST, 16>);
-    if constexpr (specialised_q(256))
-      if (Qp == 256) return set(stage_kernel<ST, 256>);
-    if constexpr (specialised_q(1024))
-      if (Qp == 1024) return set(stage_kernel<ST, 1024>);
-  }
-  return set(stage_kernel<ST, 0>);
-}
-
-cudaError_t launch(int store_kind, const void* args, int grid, int block, size_t smem, cudaStream_t st) {
-  const int Qp = store_kind == kStoreF64 ? static_cast<const StageArgs<double>*>(args)->Qp
-                                         : static_cast<const StageArgs<float>*>(args)->Qp;
-  switch (store_kind) {
-    case kStoreF64: return launch_q<StoreF64>(Qp, args, grid, block, smem, st);
-    case kStoreF32: return launch_q<StoreF32>(Qp, args, grid, block, smem, st);
-    case kStoreBF16: return launch_q<StoreBF16>(Qp, args, grid, block, smem, st);
-    case kStoreF16: return launch_q<StoreF16>(Qp, args, grid, block, smem, st);
-  }
-  return cudaErrorInvalidValue;
-}
-
-cudaError_t set_smem(int store_kind, int Qp, size_t smem) {
-  switch (store_kind) {
-    case kStoreF64: return set_smem_q<StoreF64>(Qp, smem);
-    case kStoreF32: return set_smem_q<StoreF32>(Qp, smem);
-    case kStoreBF16: return set_smem_q<StoreBF16>(Qp, smem);
-    case kStoreF16: return set_smem_q<StoreF16>(Qp, smem);
-  }
-  return cudaErrorInvalidValue;
+  if (store_kind == kStoreF64) return with_stage_kernel<StoreF64, 1>(Qp, set);
+  return with_f32_kernel(store_kind, Qp, lanes, set);
 }
 
 cudaError_t upload(const double* Dr, const double* Ds, const double* LIFT) {

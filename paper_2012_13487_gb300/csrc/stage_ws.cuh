@@ -54,10 +54,11 @@ namespace ws {
 // register file of each of the SM's four sub-partitions holds 16,384 registers
 // and the warps are dealt out over them: four warps each leave 128 registers per
 // thread, five 96, three 168.
-constexpr int kGroupThreads = 128;
-template <int QT, int G>
-__host__ __device__ constexpr int ctas() { return QT == 0 || G > 1 ? 1 : P <= 2 ? 4 : P <= 4 ? 3 : 2; }
-template <int QT, int G>
+template <int QT, int G, int N>
+__host__ __device__ constexpr int ctas() {
+  return QT == 0 || G > 1 ? 1 : P <= 2 ? 4 : P <= 4 ? 3 : 2;
+}
+template <int QT, int G, int N>
 __host__ __device__ constexpr int max_regs() {
   return QT == 0 ? 168 : G == 3 ? 128 : G == 2 ? 168 : P <= 2 ? 96 : P <= 4 ? 128 : 168;
 }
@@ -65,14 +66,14 @@ __host__ __device__ constexpr int max_regs() {
 // from the arguments) has one group of at most eleven warps, three warps per
 // sub-partition with the producer, and as few as cover the velocities in the same
 // number of passes.
-template <int QT>
+template <int QT, int N>
 __host__ __device__ constexpr int group_threads(int Q) {
-  if (QT > 0) return kGroupThreads;
+  if (QT > 0) return N == 1 ? 256 : 128;
   const int pairs = Q / 2, passes = (pairs + 351) / 352;
   return ((pairs + passes - 1) / passes + 31) / 32 * 32;
 }
-template <int QT, int G>
-__host__ __device__ constexpr int threads(int Q) { return G * group_threads<QT>(Q) + 32; }
+template <int QT, int G, int N>
+__host__ __device__ constexpr int threads(int Q) { return G * group_threads<QT, N>(Q) + 32; }
 
 // named barrier of a group's N threads, OR-reducing a predicate
 __device__ __forceinline__ bool consumers_sync_or(int id, int N, bool pred) {
@@ -118,7 +119,7 @@ struct Layout {
   int stages;
 };
 __host__ __device__ constexpr size_t up(size_t b, size_t a) { return (b + a - 1) / a * a; }
-template <class ST, int QT, int G>
+template <class ST, int QT, int G, int N>
 __host__ __device__ constexpr Layout layout(int Q) {
   Layout o{};
   constexpr size_t sb = sizeof(typename ST::S);
@@ -133,7 +134,7 @@ __host__ __device__ constexpr Layout layout(int Q) {
   o.stage = up(b, 128);
   const size_t fixed = up(size_t(ST::dev ? 6 : 3) * Q * 4, 16) + size_t(2 * G) * NP * kRec * 4 + up(size_t(2 * G) * NF * 4, 16);
   // as many stages as let the CTAs share an SM (1 KB of each is the system's), two to four
-  const size_t room = (size_t(228) * 1024) / ctas<QT, G>() - 1024 - fixed;
+  const size_t room = (size_t(228) * 1024) / ctas<QT, G, N>() - 1024 - fixed;
   o.stages = int(room / o.stage);
   o.stages = o.stages < 2 ? 2 : o.stages > 4 * G ? 4 * G : o.stages;
   b = o.stage * o.stages;
@@ -147,10 +148,10 @@ __host__ __device__ constexpr Layout layout(int Q) {
 // Moments of every node of the element in `row0` and their records.  G lanes
 // share a node; a lane sums packed pairs over its 16-byte chunks (the FP64 and
 // compensated modes take one accumulator update per chunk).
-template <class ST, class Acc, int QT>
+template <class ST, class Acc, int QT, int NT>
 __device__ __forceinline__ void element_moments(const StageArgs<float>& a, const typename ST::S* row0, float sc,
                                                 const float* s_vel, float kappa, float* rec, int tid, int nth) {
-  const int Q = QT > 0 ? QT : a.Qp, NTH = QT > 0 ? kGroupThreads : nth;
+  const int Q = QT > 0 ? QT : a.Qp, NTH = QT > 0 ? NT : nth;
   constexpr int V = Vec16<ST>::N;
   const int NCH = Q / V;
   // lanes per node: a power of two that divides the chunks' loop evenly for the
@@ -248,15 +249,18 @@ __device__ __forceinline__ void element_moments(const StageArgs<float>& a, const
   }
 }
 
-template <class ST, int QT, int G>
-__global__ void __maxnreg__((max_regs<QT, G>())) stage_kernel_ws(const StageArgs<float> a) {
+template <class ST, int QT, int G, int N>
+__global__ void __maxnreg__((max_regs<QT, G, N>())) stage_kernel_ws(const StageArgs<float> a) {
   using S = typename ST::S;
+  using L = Lanes<N>;
+  using T = typename L::T;
   constexpr bool kWide = QT == 0;
   const int Q = kWide ? a.Qp : QT;
-  constexpr Layout oc = layout<ST, QT, G>(kWide ? 512 : QT);
-  const Layout o = kWide ? layout<ST, QT, G>(Q) : oc;
-  const int NC = kWide ? int(blockDim.x) - 32 : kGroupThreads, NST = kWide ? o.stages : oc.stages;
-  const int kPasses = (Q + 2 * NC - 1) / (2 * NC);
+  constexpr Layout oc = layout<ST, QT, G, N>(kWide ? 512 : QT);
+  const Layout o = kWide ? layout<ST, QT, G, N>(Q) : oc;
+  constexpr int kThreadsOf = group_threads<QT, N>(QT > 0 ? QT : 512);
+  const int NC = kWide ? int(blockDim.x) - 32 : kThreadsOf, NST = kWide ? o.stages : oc.stages;
+  const int kPasses = (Q + N * NC - 1) / (N * NC);
   extern __shared__ __align__(128) unsigned char smem[];
   const bool producer = threadIdx.x >= G * NC;
   const int group = producer ? 0 : threadIdx.x / NC;
@@ -362,12 +366,16 @@ __global__ void __maxnreg__((max_regs<QT, G>())) stage_kernel_ws(const StageArgs
     return;
   }
 
-  // ---- consumers: thread = velocities i, i + 1 of each element of this CTA --------
-  using M = EoDual<kHaveOpsTable>;
-  const Pair rkA2 = both(a.rkA), rkB2 = both(a.rkB);
+  // ---- consumers: thread = N adjacent velocities from i on, of each element of this CTA ----
+  const T rkA2 = L::both(a.rkA), rkB2 = L::both(a.rkB), zero = L::zero();
   const float ab = a.ab;
   const uint32_t sr_step = (ST::dev && a.sr_step) ? __ldg(a.sr_step) : 0u;
   const int bar_id = 1 + group;
+  // one velocity per thread: its own rows stay in registers
+  constexpr bool kOwnRows = N == 1;
+  const T ex1 = kOwnRows ? L::load(s_vel + tid) : zero, ey1 = kOwnRows ? L::load(s_vel + Q + tid) : zero;
+  const T w1 = kOwnRows ? L::load(s_vel + 2 * Q + tid) : zero;
+  const T iw1 = kOwnRows && ST::dev ? L::load(s_vel + 5 * Q + tid) : zero;
   int j = group;  // element of the CTA
   for (int64_t k = blockIdx.x + int64_t(group) * gridDim.x; k < K; k += int64_t(G) * gridDim.x, j += G) {
     const int s = j % NST;
@@ -375,14 +383,14 @@ __global__ void __maxnreg__((max_regs<QT, G>())) stage_kernel_ws(const StageArgs
     // the residual columns of this element's first pass (before the wait: their
     // latency overlaps the copies and the reductions; asked for an element ahead
     // instead they measured slower, 4126 us against 3812 us for the 8-step call)
-    Pair rold[NP];
-    const size_t col0 = size_t(k) * NP * Q + 2 * tid;
+    T rold[NP];
+    const size_t col0 = size_t(k) * NP * Q + N * tid;
     auto load_residual = [&](int pass) {
 #pragma unroll
       for (int n = 0; n < NP; ++n)
-        rold[n] = read_res && (!kWide || 2 * tid + pass * 2 * NC < Q)
-                      ? *reinterpret_cast<const Pair*>(a.res + col0 + size_t(n) * Q + pass * 2 * NC)
-                      : 0ull;
+        rold[n] = read_res && (!kWide || N * tid + pass * N * NC < Q)
+                      ? L::load(a.res + col0 + size_t(n) * Q + pass * N * NC)
+                      : zero;
     };
     load_residual(0);
     bool ok = true;
@@ -410,11 +418,11 @@ __global__ void __maxnreg__((max_regs<QT, G>())) stage_kernel_ws(const StageArgs
     if (!a.collision) {
       for (int v = tid; v < NP * kRec; v += NC) rec[v] = 0.f;
     } else if (a.red == kRedFP64) {
-      element_moments<ST, AccD, QT>(a, st_f(s), sc, s_vel, kappa, rec, tid, NC);
+      element_moments<ST, AccD, QT, kThreadsOf>(a, st_f(s), sc, s_vel, kappa, rec, tid, NC);
     } else if (a.red == kRedCompFP32) {
-      element_moments<ST, AccN, QT>(a, st_f(s), sc, s_vel, kappa, rec, tid, NC);
+      element_moments<ST, AccN, QT, kThreadsOf>(a, st_f(s), sc, s_vel, kappa, rec, tid, NC);
     } else {
-      element_moments<ST, AccF, QT>(a, st_f(s), sc, s_vel, kappa, rec, tid, NC);
+      element_moments<ST, AccF, QT, kThreadsOf>(a, st_f(s), sc, s_vel, kappa, rec, tid, NC);
     }
     if (a.wall_any) {
       // one warp per wall face node: sum over outgoing velocities of (e.n) f^-
@@ -437,124 +445,120 @@ __global__ void __maxnreg__((max_regs<QT, G>())) stage_kernel_ws(const StageArgs
     }
     consumers_sync(bar_id, NC);
 
-    // ---- residual and update of velocities i, i + 1, all nodes -----------------
+    // ---- residual and update of velocities i .. i + N - 1, all nodes -----------------
 #pragma unroll 1
     for (int pass = 0; pass < kPasses; ++pass) {
-      const int i_own = 2 * tid + pass * 2 * NC;
+      const int i_own = N * tid + pass * N * NC;
       // the wide form's last pass: lanes past the last velocity take the first along and
       // store nothing
       const bool own = !kWide || i_own < Q;
       const int i = own ? i_own : 0;
       if (kWide && !__any_sync(kFull, own)) continue;
-      const Pair ex = *reinterpret_cast<const Pair*>(s_vel + i), ey = *reinterpret_cast<const Pair*>(s_vel + Q + i);
-      const Pair w = *reinterpret_cast<const Pair*>(s_vel + 2 * Q + i);
-      const Pair ws = ST::dev ? f2mul(w, both(sc)) : 0ull;
+      const T ex = kOwnRows ? ex1 : L::load(s_vel + i), ey = kOwnRows ? ey1 : L::load(s_vel + Q + i);
+      const T w = kOwnRows ? w1 : L::load(s_vel + 2 * Q + i);
+      const T ws = ST::dev ? L::mul(w, L::both(sc)) : zero;
       if (kPasses > 1 && pass > 0) load_residual(pass);
       const S* fcol = st_f(s) + i;
+      auto normal_speed = [&](int fc) {
+        return L::fmat(ey, L::both(g[5 + 3 * fc]), L::mul(ex, L::both(g[4 + 3 * fc])));
+      };
       // wide form: the neighbour traces straight from global memory (L2), for the faces
       // the pair enters through, all in flight before the first is used
-      Pair tr[kWide ? NF : 1];
+      T tr[kWide ? NF : 1];
       if constexpr (kWide) {
 #pragma unroll
         for (int fc = 0; fc < 3; ++fc) {
           const int code = nb[fc];
-          float e0, e1;
-          f2unpack(f2fma(ey, both(g[5 + 3 * fc]), f2mul(ex, both(g[4 + 3 * fc]))), e0, e1);
-          const bool in = code >= 0 && (fmaf(-ab, fabsf(e0), e0) != 0.f || fmaf(-ab, fabsf(e1), e1) != 0.f);
+          const bool in = code >= 0 && L::any(L::map(normal_speed(fc), [&](float v) { return fmaf(-ab, fabsf(v), v); }));
           const S* base = fin + size_t(code >= 0 ? code >> 3 : 0) * NP * Q + i;
 #pragma unroll
           for (int aa = 0; aa < NFP; ++aa)
-            tr[fc * NFP + aa] = in ? raw_pair<ST>(base + size_t(trace_node(code, aa)) * Q) : 0ull;
+            tr[fc * NFP + aa] = in ? L::template raw<ST>(base + size_t(trace_node(code, aa)) * Q) : zero;
         }
       }
-      Pair fr[NP];
+      T fr[NP];
 #pragma unroll
-      for (int m = 0; m < NP; ++m) fr[m] = value_pair<ST>(fcol + m * Q, w, ws);
+      for (int m = 0; m < NP; ++m) fr[m] = lane_value<L, ST>(fcol + m * Q, w, ws);
       // face fc carries flux for some velocity of this warp (warp-uniform; with
       // the upwind flux an outflow face's jump term is zero, so a face that is
-      // outflow for all 64 velocities skips its traces and lift columns)
-      Pair flux[NF];
+      // outflow for all the warp's velocities skips its traces and lift columns)
+      T flux[NF];
       bool on[3];
 #pragma unroll
       for (int fc = 0; fc < 3; ++fc) {
-        const Pair en = f2fma(ey, both(g[5 + 3 * fc]), f2mul(ex, both(g[4 + 3 * fc])));
-        float e0, e1;
-        f2unpack(en, e0, e1);
         const float h = 0.5f * dt * g[6 + 3 * fc];
         const int code = nb[fc];
-        float c0 = h * fmaf(-ab, fabsf(e0), e0), c1 = h * fmaf(-ab, fabsf(e1), e1);
-        if (code < 0) {  // incoming velocities take the wall state; outgoing ones have no jump
-          c0 = e0 < 0.f ? c0 : 0.f;
-          c1 = e1 < 0.f ? c1 : 0.f;
-        }
-        on[fc] = __any_sync(kFull, c0 != 0.f || c1 != 0.f);
+        const T c = L::map(normal_speed(fc), [&](float v) {
+          const float x = h * fmaf(-ab, fabsf(v), v);
+          return code < 0 && !(v < 0.f) ? 0.f : x;  // a wall: incoming velocities take its state, no other jump
+        });
+        on[fc] = __any_sync(kFull, L::any(c));
 #pragma unroll
-        for (int aa = 0; aa < NFP; ++aa) flux[fc * NFP + aa] = 0ull;
+        for (int aa = 0; aa < NFP; ++aa) flux[fc * NFP + aa] = zero;
         if (!on[fc]) continue;
-        const Pair c = f2pack(c0, c1);
         if (code >= 0) {
-          const Pair wsn = ST::dev ? f2mul(w, both(st_nscale(s)[fc])) : 0ull;
+          const T wsn = ST::dev ? L::mul(w, L::both(st_nscale(s)[fc])) : zero;
           const S* trow = st_tr(s) + fc * NFP * Q + i;
 #pragma unroll
           for (int aa = 0; aa < NFP; ++aa) {
-            Pair t;
-            if constexpr (kWide) t = ST::dev ? f2fma(wsn, tr[fc * NFP + aa], w) : tr[fc * NFP + aa];
-            else t = value_pair<ST>(trow + aa * Q, w, wsn);
-            flux[fc * NFP + aa] = f2mul(c, EoPacked::sub(fr[face_node(fc, aa)], t));
+            T t;
+            if constexpr (kWide) t = ST::dev ? L::fmat(wsn, tr[fc * NFP + aa], w) : tr[fc * NFP + aa];
+            else t = lane_value<L, ST>(trow + aa * Q, w, wsn);
+            flux[fc * NFP + aa] = L::mul(c, L::sub(fr[face_node(fc, aa)], t));
           }
         } else {
           const int slot = -code - 1;
-          const Pair fb = *reinterpret_cast<const Pair*>(a.wall_feq + size_t(slot) * Q + i);
+          const T fb = L::load(a.wall_feq + size_t(slot) * Q + i);
           const float den_inv = __ldg(a.wall_den_inv + slot);
           const bool diffuse = den_inv > 0.f;
-          const Pair fd = diffuse ? f2mul(both(den_inv), fb) : fb;
+          const T fd = diffuse ? L::mul(L::both(den_inv), fb) : fb;
 #pragma unroll
           for (int aa = 0; aa < NFP; ++aa) {
-            const Pair fp = diffuse ? f2mul(both(wn[fc * NFP + aa]), fd) : fb;
-            flux[fc * NFP + aa] = f2mul(c, EoPacked::sub(fr[face_node(fc, aa)], fp));
+            const T fp = diffuse ? L::mul(L::both(wn[fc * NFP + aa]), fd) : fb;
+            flux[fc * NFP + aa] = L::mul(c, L::sub(fr[face_node(fc, aa)], fp));
           }
         }
       }
-      Pair le[NE], lo[at_least_1(NO)];
-      eo_lift<M>(flux, on[0] || on[2], on[1], le, lo);
-      const Pair neg_k = both(-kappa);
-      const Pair ar = f2fma(ey, both(g[2]), f2mul(ex, both(g[0]))), as = f2fma(ey, both(g[3]), f2mul(ex, both(g[1])));
-      const Pair half_dt = both(0.5f * dt);
-      const Pair na = f2mul(f2mul(half_dt, both(-1.f)), EoPacked::add(ar, as)), nd = f2mul(half_dt, EoPacked::sub(ar, as));
-      Pair invw = 0ull;
+      T le[NE], lo[at_least_1(NO)];
+      eo_lift<L>(flux, on[0] || on[2], on[1], le, lo);
+      const T neg_k = L::both(-kappa);
+      const T ar = L::fmat(ey, L::both(g[2]), L::mul(ex, L::both(g[0])));
+      const T as = L::fmat(ey, L::both(g[3]), L::mul(ex, L::both(g[1])));
+      const T half_dt = L::both(0.5f * dt);
+      const T na = L::mul(L::mul(half_dt, L::both(-1.f)), L::add(ar, as)), nd = L::mul(half_dt, L::sub(ar, as));
+      T invw = zero;
       if constexpr (ST::dev)  // BF16 keeps the element's power-of-two scale: q = (f - w) / (w s)
-        invw = f2mul(*reinterpret_cast<const Pair*>(s_vel + 5 * Q + i), both(1.0f / sc));
-      const size_t col = col0 + size_t(pass) * 2 * NC;
+        invw = L::mul(kOwnRows ? iw1 : L::load(s_vel + 5 * Q + i), L::both(1.0f / sc));
+      const size_t col = col0 + size_t(pass) * N * NC;
       // update and write-back of node n from dt times its advection term
       // -(e . grad) f + LIFT (flux)
-      eo_volume<M>([&](int n) { return fr[n]; }, na, nd, le, lo, [&](int n, Pair adv) {
-        const ulonglong2* mm = reinterpret_cast<const ulonglong2*>(rec + n * kRec);
-        const ulonglong2 m01 = mm[0], m23 = mm[1], mu = mm[2];
-        const Pair f = value_pair<ST>(fcol + n * Q, w, ws);
-        const Pair eu = f2fma(ey, mu.y, f2mul(ex, mu.x));
-        Pair feq = f2fma(ey, m23.x, f2fma(ex, m01.y, m01.x));
-        feq = f2fma(eu, f2mul(m23.y, eu), feq);
+      eo_volume<L>([&](int n) { return fr[n]; }, na, nd, le, lo, [&](int n, T adv) {
+        const float* mm = rec + n * kRec;
+        T m0, m1, m2, m3, mx, my;
+        L::record(mm, m0, m1);
+        L::record(mm + 4, m2, m3);
+        L::record(mm + 8, mx, my);
+        const T f = N == 1 && P <= 4 ? fr[n] : lane_value<L, ST>(fcol + n * Q, w, ws);
+        const T eu = L::fmat(ey, my, L::mul(ex, mx));
+        T feq = L::fmat(ey, m2, L::fmat(ex, m1, m0));
+        feq = L::fmat(eu, L::mul(m3, eu), feq);
         if (third) {
-          const ulonglong2 m67 = mm[3];
-          feq = f2fma(eu, f2fma(m67.x, f2mul(eu, eu), m67.y), feq);
+          T m6, m7;
+          L::record(mm + 12, m6, m7);
+          feq = L::fmat(eu, L::fmat(m6, L::mul(eu, eu), m7), feq);
         }
-        const Pair r = f2fma(w, feq, f2fma(neg_k, f, f2fma(rkA2, rold[n], adv)));
-        const Pair fnew = f2fma(rkB2, r, f);
+        const T r = L::fmat(w, feq, L::fmat(neg_k, f, L::fmat(rkA2, rold[n], adv)));
+        const T fnew = L::fmat(rkB2, r, f);
         const size_t gi = col + size_t(n) * Q;
-        if (own) *reinterpret_cast<Pair*>(a.res + gi) = r;
+        if (own) L::store(a.res + gi, r);
         if constexpr (ST::dev) {
-          float q0, q1;
-          f2unpack(f2mul(EoPacked::sub(fnew, w), invw), q0, q1);
-          __nv_bfloat162 q;
-          if (a.sr_step) {
-            q.x = bf16_round_stochastic(q0, sr_hash(gi, sr_step, uint32_t(a.sr_stage)));
-            q.y = bf16_round_stochastic(q1, sr_hash(gi + 1, sr_step, uint32_t(a.sr_stage)));
-          } else {
-            q = __floats2bfloat162_rn(q0, q1);
-          }
-          if (own) *reinterpret_cast<__nv_bfloat162*>(fout + gi) = q;
+          const T q = L::mul(L::sub(fnew, w), invw);
+          typename L::Code code;
+          if (a.sr_step) code = L::to_bf16(q, gi, sr_step, uint32_t(a.sr_stage));
+          else code = L::to_bf16(q);
+          if (own) *reinterpret_cast<typename L::Code*>(fout + gi) = code;
         } else {
-          if (own) *reinterpret_cast<Pair*>(fout + gi) = fnew;
+          if (own) L::store(fout + gi, fnew);
         }
       });
     }
@@ -567,11 +571,11 @@ __global__ void __maxnreg__((max_regs<QT, G>())) stage_kernel_ws(const StageArgs
 
 // The form exists for these states, velocity counts and degrees (two ring
 // stages have to fit a CTA's shared memory).
-template <class ST, int QT, int G>
+template <class ST, int QT, int G, int N>
 __host__ __device__ constexpr bool exists() {
   if constexpr (ST::kind != kStoreF32 && ST::kind != kStoreBF16) return false;
   else if constexpr (QT == 0) return P >= 1 && P <= 5;
-  else if constexpr (QT == 1024) return P <= 4 && layout<ST, QT, G>(QT).end <= size_t(227) * 1024;
+  else if constexpr (QT == 1024) return P <= 3;
   else return P <= 5;
 }
 
@@ -581,27 +585,29 @@ struct Form {
   size_t smem = 0;
   int threads = 0;
 };
-template <class ST, int QT, int G>
+template <class ST, int QT, int G, int N>
 Form form_as(int Q) {
   Form f;
-  if constexpr (exists<ST, QT, G>()) {
-    const Layout o = layout<ST, QT, G>(Q);
+  if constexpr (exists<ST, QT, G, N>()) {
+    const Layout o = layout<ST, QT, G, N>(Q);
     if (o.end > size_t(227) * 1024) return f;
-    f.kernel = &stage_kernel_ws<ST, QT, G>;
+    f.kernel = &stage_kernel_ws<ST, QT, G, N>;
     f.smem = o.end;
-    f.threads = threads<QT, G>(Q);
+    f.threads = threads<QT, G, N>(Q);
   }
   return f;
 }
-// The form of this state and velocity count with `groups` consumer groups (0: the
-// wide form, one group sized to the velocities); kernel == nullptr where there is none.
+template <class ST>
+Form form_of(int Qp, int groups) {
+  if (Qp == 1024 && groups == 3) return form_as<ST, 1024, 3, 2>(Qp);
+  if (Qp == 256 && groups == 1) return form_as<ST, 256, 1, 2>(Qp);
+  if (Qp == 256 && groups == 2) return form_as<ST, 256, 2, 2>(Qp);
+  if (Qp >= 512 && groups == 0) return form_as<ST, 0, 1, 2>(Qp);
+  return Form();
+}
 inline Form form(int store_kind, int Qp, int groups) {
-  const bool f32 = store_kind == kStoreF32;
-  if (!f32 && store_kind != kStoreBF16) return Form();
-  if (Qp == 1024 && groups == 3) return f32 ? form_as<StoreF32, 1024, 3>(Qp) : form_as<StoreBF16, 1024, 3>(Qp);
-  if (Qp == 256 && groups == 1) return f32 ? form_as<StoreF32, 256, 1>(Qp) : form_as<StoreBF16, 256, 1>(Qp);
-  if (Qp == 256 && groups == 2) return f32 ? form_as<StoreF32, 256, 2>(Qp) : form_as<StoreBF16, 256, 2>(Qp);
-  if (Qp >= 512 && groups == 0) return f32 ? form_as<StoreF32, 0, 1>(Qp) : form_as<StoreBF16, 0, 1>(Qp);
+  if (store_kind == kStoreF32) return form_of<StoreF32>(Qp, groups);
+  if (store_kind == kStoreBF16) return form_of<StoreBF16>(Qp, groups);
   return Form();
 }
 
