@@ -146,12 +146,12 @@ typedef struct fedbm_params {
                               else 1);
                               3 = the warp-specialised form: a producer warp
                               keeps a ring of one-element tiles filled (bulk
-                              copies) for consumer warps, two velocities per
-                              thread (tile arguments ignored); asked for by
-                              number it has two groups of four consumer warps,
-                              288 threads per CTA, and serves FP32 or BF16 state
-                              with 256 padded velocities at degree <= 5, else
-                              EINVAL.  The autotuner times the automatic
+                              copies) for consumer warps (tile arguments
+                              ignored); asked for by number it has eight
+                              consumer warps, 288 threads per CTA, and serves
+                              FP32 or BF16 state with 256 padded velocities at
+                              degree <= 5, else EINVAL (the automatic choice's
+                              shape of it is mostly the faster one).  The autotuner times the automatic
                               choice's form where it exists              */
   int32_t tensor_cores;  /* stage-kernel form: 0 = the FMA kernel (the
                             faster form on every measured shape), with the

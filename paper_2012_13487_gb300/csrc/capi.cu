@@ -455,8 +455,8 @@ int auto_cluster(const Group& g) {
   return best;
 }
 
-// The warp-specialised form of a group: one element per ring stage, four or
-// eight consumer warps (two velocities per thread) and one producer warp.
+// The warp-specialised form of a group: one element per ring stage, consumer warps and
+// one producer warp.
 // Consumer groups per CTA of the automatic choice: one with 256 velocities (three
 // CTAs share an SM), three with 1,024 (one CTA per SM: two ring stages of each of
 // three CTAs would not fit), 0 for the wide form.

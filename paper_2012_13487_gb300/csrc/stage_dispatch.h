@@ -26,9 +26,9 @@ struct StageEntry {
   cudaError_t (*set_smem_cl)(int store_kind, size_t smem);
   int (*occupancy_cl)(int store_kind, int ncl, size_t smem);  // resident clusters on the device
   // warp-specialised form (a producer warp filling a ring of element tiles for
-  // groups of four consumer warps; FP32 or BF16 state, 256 or 1,024 padded
-  // velocities, degree <= 5 or 4)
-  // consumer groups per CTA: 1 or 2 with 256 velocities, 3 with 1,024
+  // groups of consumer warps; FP32 or BF16 state).  groups: 1 and 2 (the form asked
+  // for by number) with 256 padded velocities at degree <= 5, 3 with 1,024 at degree
+  // <= 3, 0 for the wide form, from 512 up at degree 1..5
   size_t (*ws_smem)(int store_kind, int Qp, int groups);  // 0 = no such form
   int (*ws_threads)(int store_kind, int Qp, int groups);
   cudaError_t (*launch_ws)(int store_kind, const void* args, int groups, int grid, size_t smem, cudaStream_t st);

@@ -5,8 +5,8 @@
 // FMA kernel.
 //
 // A CTA has one to three groups of four consumer warps, each thread taking two
-// adjacent velocities of an element (256 velocities in one pass, 1,024 in four), and
-// one producer warp.  The producer keeps a ring of shared-memory stages filled with
+// adjacent velocities of an element (256 velocities in one pass, 1,024 in four; or one
+// group of eight warps with one velocity per thread), and one producer warp.  The producer keeps a ring of shared-memory stages filled with
 // the next elements' state tiles, geometry and neighbour face rows (bulk copies, one
 // "full" mbarrier per stage); the groups take the elements in turn, reduce the node
 // moments and wall numerators from the stage, read their own residual columns
@@ -53,14 +53,27 @@ namespace ws {
 // the CTA), the threads of a group, resident CTAs and registers per thread.  The
 // register file of each of the SM's four sub-partitions holds 16,384 registers
 // and the warps are dealt out over them: four warps each leave 128 registers per
-// thread, five 96, three 168.
+// thread, five 96, three 168, seven 72.
+//
+// The form asked for by number with 256 velocities has eight consumer warps (288
+// threads), whatever the automatic one has.  Two groups of four warps with two velocities
+// per thread hold their registers only up to degree 3 with two CTAs on an SM (degree 1:
+// three, one producer warp being short of that many small elements); above, one group of
+// eight warps takes one velocity per thread.  One step of 31M values, us, at degree 1..5:
+// the former kernel (one velocity per thread, BF16 on tensor cores) FP32 676, 538, 519,
+// 523, 845, BF16 1283, 893, 668, 586, 697; two groups, one CTA per SM 819, 839, 599, 584,
+// 644 and 994, 1034, 709, 611, 672; now 611, 508, 466, 504, 540 and 732, 602, 565, 582, 621.
 template <int QT, int G, int N>
 __host__ __device__ constexpr int ctas() {
+  if (N == 1) return 2;
+  if (G == 2) return P <= 1 ? 3 : 2;
   return QT == 0 || G > 1 ? 1 : P <= 2 ? 4 : P <= 4 ? 3 : 2;
 }
 template <int QT, int G, int N>
 __host__ __device__ constexpr int max_regs() {
-  return QT == 0 ? 168 : G == 3 ? 128 : G == 2 ? 168 : P <= 2 ? 96 : P <= 4 ? 128 : 168;
+  if (N == 1) return 96;
+  if (G == 2) return P <= 1 ? 72 : 96;
+  return QT == 0 ? 168 : G == 3 ? 128 : P <= 2 ? 96 : P <= 4 ? 128 : 168;
 }
 // Consumer threads of a group.  The wide form (QT == 0: the velocity count is taken
 // from the arguments) has one group of at most eleven warps, three warps per
@@ -538,6 +551,7 @@ __global__ void __maxnreg__((max_regs<QT, G, N>())) stage_kernel_ws(const StageA
         L::record(mm, m0, m1);
         L::record(mm + 4, m2, m3);
         L::record(mm + 8, mx, my);
+        // from shared memory again where the registers are short
         const T f = N == 1 && P <= 4 ? fr[n] : lane_value<L, ST>(fcol + n * Q, w, ws);
         const T eu = L::fmat(ey, my, L::mul(ex, mx));
         T feq = L::fmat(ey, m2, L::fmat(ex, m1, m0));
@@ -601,7 +615,10 @@ template <class ST>
 Form form_of(int Qp, int groups) {
   if (Qp == 1024 && groups == 3) return form_as<ST, 1024, 3, 2>(Qp);
   if (Qp == 256 && groups == 1) return form_as<ST, 256, 1, 2>(Qp);
-  if (Qp == 256 && groups == 2) return form_as<ST, 256, 2, 2>(Qp);
+  if (Qp == 256 && groups == 2) {
+    if constexpr (P <= 3) return form_as<ST, 256, 2, 2>(Qp);
+    else return form_as<ST, 256, 1, 1>(Qp);
+  }
   if (Qp >= 512 && groups == 0) return form_as<ST, 0, 1, 2>(Qp);
   return Form();
 }
