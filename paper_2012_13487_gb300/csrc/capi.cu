@@ -289,6 +289,7 @@ struct Group {
 
 struct Batch {
   int device = 0;
+  int nsm = 0, smem_sm = 0;      // SMs of the device and shared memory of one, bytes
   cudaStream_t stream = nullptr;
   cudaStream_t capture = nullptr;
   std::vector<Case> cases;
@@ -386,10 +387,7 @@ int configure_tc(Batch& b, Group& g) {
   const StageEntry e = stage_entry(g.p);
   size_t smem = e.tc_smem(g.store, g.Qp);
   if (g.tc_mode < 0 || smem == 0) return fail(FEDBM_EINVAL, "this form has no tensor-core stage kernel");
-  int nsm = 0;
-  FEDBM_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b.device));
-  int smem_sm = 0;
-  FEDBM_CK(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, b.device));
+  const int nsm = b.nsm, smem_sm = b.smem_sm;
   // small tiles: reserve enough shared memory that no more CTAs fit on an SM
   // than its tensor memory serves
   const int max_ctas = 512 / e.tc_tmem_cols(g.Qp);
@@ -488,8 +486,7 @@ int configure_ws(Batch& b, Group& g, int groups = -1) {
                               "256 padded velocities and degree <= 5");
   if (smem > kMaxSmem) return fail(FEDBM_EINVAL, "warp-specialised ring does not fit in shared memory");
   FEDBM_CK(e.set_smem_ws(g.store, g.Qp, groups, kMaxSmem));
-  int nsm = 0;
-  FEDBM_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b.device));
+  const int nsm = b.nsm;
   const int per_sm = e.occupancy_ws(g.store, g.Qp, groups, smem);
   if (per_sm < 1) return fail(FEDBM_EINVAL, "warp-specialised stage kernel cannot be resident on an SM");
   g.tc = 0;
@@ -598,8 +595,7 @@ int configure_tiles(Batch& b, Group& g, int epc, int tpb, int stages) {
   // groups of one batch sharing this kernel with other tiles keep launching
   const int lanes = stage_lanes(g, e_pc, t_pb);
   FEDBM_CK(e.set_smem(g.store, g.Qp, lanes, kMaxSmem));
-  int nsm = 0;
-  FEDBM_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b.device));
+  const int nsm = b.nsm;
   const int per_sm = e.occupancy(g.store, g.Qp, lanes, t_pb, smem);
   if (per_sm < 1) return fail(FEDBM_EINVAL, "stage tile cannot be resident on an SM");
   const int64_t ntiles = (g.K + e_pc - 1) / e_pc;
@@ -1078,6 +1074,20 @@ void free_batch(Batch* b) {
   delete b;
 }
 
+// What the transfer kernels need to know of case c's slice of its group.
+transfer::Shape layout_of(const Batch& b, const Group& g, const Case& cs) {
+  transfer::Shape t;
+  t.store = g.store;
+  t.K = cs.K;
+  t.Np = g.Np;
+  t.Q = g.Q;
+  t.Qp = g.Qp;
+  t.vel64 = g.vel64;
+  t.iperm = g.iperm;
+  t.nsm = b.nsm;
+  t.smem_sm = b.smem_sm;
+  return t;
+}
 int create_batch(const fedbm_case_desc* cd, int ncases, void* stream, Batch** out) {
   if (!cd || ncases < 1 || !out) return fail(FEDBM_EINVAL, "need at least one case and an output pointer");
   *out = nullptr;
@@ -1136,12 +1146,15 @@ int create_batch(const fedbm_case_desc* cd, int ncases, void* stream, Batch** ou
   int rc = FEDBM_OK;
   if ((rc = [&]() -> int {
          FEDBM_CK(cudaGetDevice(&b->device));
+         FEDBM_CK(cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, b->device));
+         FEDBM_CK(cudaDeviceGetAttribute(&b->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, b->device));
          int r = ensure_ops_uploaded(b->device);
          if (r != FEDBM_OK) return r;
          FEDBM_CK(cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking));
          for (Group& g : b->groups) {
            const int epc = g.epc, tpb = g.tpb, st = g.nstages;
            if ((r = build_group(*b, g)) != FEDBM_OK) return r;
+           FEDBM_CK(transfer::prepare(layout_of(*b, g, b->cases[g.cases[0]])));
            // default: the FMA kernel for every form, as its warp-specialised
            // variant where ws_default says so (with its compile-time operator
            // tables it measured faster than the tensor-core form on FP32 state
@@ -1207,19 +1220,6 @@ int timeout_status(int word) {
               : FEDBM_OK;
 }
 
-// What the transfer kernels need to know of case c's slice of its group.
-transfer::Shape layout_of(const Batch& b, const Group& g, const Case& cs) {
-  transfer::Shape t;
-  t.store = g.store;
-  t.K = cs.K;
-  t.Np = g.Np;
-  t.Q = g.Q;
-  t.Qp = g.Qp;
-  t.vel64 = g.vel64;
-  t.iperm = g.iperm;
-  t.device = b.device;
-  return t;
-}
 const void* state_of(const Group& g, int cur, const Case& cs) {
   return static_cast<const unsigned char*>(g.f[cur]) + size_t(cs.k_off) * g.Np * g.Qp * store_bytes(g.store);
 }

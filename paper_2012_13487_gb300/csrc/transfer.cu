@@ -42,12 +42,9 @@ Split split_for(const Shape& sh, size_t table_bytes, size_t value_bytes) {
   const int groups = s.warp ? kThreads / 32 : 1;
   s.rows = s.warp ? sh.Np : std::max(1, std::min(sh.Np, int(kStageBytes / row)));
   s.smem = s.tables + size_t(groups) * s.rows * row;
-  int nsm = 152, smem_sm = 228 * 1024;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, sh.device);
-  cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, sh.device);
-  const int per_sm = std::max(1, std::min(8, int(size_t(smem_sm) / (s.smem + 1024))));
+  const int per_sm = std::max(1, std::min(8, int(size_t(sh.smem_sm) / (s.smem + 1024))));
   const int64_t tiles = s.warp ? (sh.K + groups - 1) / groups : sh.K;
-  s.grid = int(std::max<int64_t>(1, std::min<int64_t>(tiles, int64_t(nsm) * per_sm)));
+  s.grid = int(std::max<int64_t>(1, std::min<int64_t>(tiles, int64_t(sh.nsm) * per_sm)));
   return s;
 }
 
@@ -449,35 +446,54 @@ __global__ void __launch_bounds__(kThreads) moments_kernel(const void* __restric
   }
 }
 
-template <class F>
-cudaError_t allow_smem(F kernel, size_t smem) {
-  if (smem <= 48 * 1024) return cudaSuccess;
-  if (smem > kSmemCap) return cudaErrorInvalidValue;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemCap));
-}
-
+// Work split and kernel of one transfer.
+template <class Kernel>
+struct Plan {
+  Split split;
+  Kernel kernel;
+  cudaError_t allow_smem() const {
+    if (split.smem <= 48 * 1024 || split.smem > kSmemCap) return cudaSuccess;  // a launch beyond is refused
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemCap));
+  }
+};
 template <class ST, typename TIn>
-cudaError_t encode_as(const Shape& sh, const TIn* in, void* out, float* scale, cudaStream_t st) {
+auto encode_plan(const Shape& sh) {
   // internal indices; deviation forms: six words a velocity, for FP64 input w and 1/w behind them
   const size_t q = size_t(sh.Q);
   const size_t tables = !ST::dev ? 4 * q : sizeof(TIn) == 8 ? up16(24 * q) + 16 * q : 24 * q;
   const Split s = split_for(sh, tables, ST::dev ? 4 : sizeof(typename ST::S));
-  auto kernel = s.warp ? encode_kernel<ST, TIn, true> : encode_kernel<ST, TIn, false>;
-  cudaError_t e = allow_smem(kernel, s.smem);
-  if (e != cudaSuccess) return e;
-  kernel<<<s.grid, kThreads, s.smem, st>>>(in, out, scale, sh.vel64, sh.iperm, sh.K, sh.Np, sh.Q, sh.Qp, s.rows,
+  auto kernel = s.warp ? &encode_kernel<ST, TIn, true> : &encode_kernel<ST, TIn, false>;
+  return Plan<decltype(kernel)>{s, kernel};
+}
+template <class ST>
+auto decode_plan(const Shape& sh) {
+  const size_t tables = (ST::dev ? 8 * size_t(sh.Q) : 0) + 4 * size_t(sh.Qp);
+  const Split s = split_for(sh, tables, ST::dev ? 4 : sizeof(typename ST::S));
+  auto kernel = s.warp ? &decode_kernel<ST, true> : &decode_kernel<ST, false>;
+  return Plan<decltype(kernel)>{s, kernel};
+}
+
+template <class ST>
+cudaError_t prepare_as(const Shape& sh) {
+  cudaError_t e = encode_plan<ST, double>(sh).allow_smem();
+  if (e == cudaSuccess) e = encode_plan<ST, float>(sh).allow_smem();
+  return e == cudaSuccess ? decode_plan<ST>(sh).allow_smem() : e;
+}
+
+template <class ST, typename TIn>
+cudaError_t encode_as(const Shape& sh, const TIn* in, void* out, float* scale, cudaStream_t st) {
+  const auto plan = encode_plan<ST, TIn>(sh);
+  const Split& s = plan.split;
+  plan.kernel<<<s.grid, kThreads, s.smem, st>>>(in, out, scale, sh.vel64, sh.iperm, sh.K, sh.Np, sh.Q, sh.Qp, s.rows,
                                            int(s.tables));
   return cudaGetLastError();
 }
 
 template <class ST>
 cudaError_t decode_as(const Shape& sh, const void* in, const float* scale, double* out, cudaStream_t st) {
-  const size_t tables = (ST::dev ? 8 * size_t(sh.Q) : 0) + 4 * size_t(sh.Qp);
-  const Split s = split_for(sh, tables, ST::dev ? 4 : sizeof(typename ST::S));
-  auto kernel = s.warp ? decode_kernel<ST, true> : decode_kernel<ST, false>;
-  cudaError_t e = allow_smem(kernel, s.smem);
-  if (e != cudaSuccess) return e;
-  kernel<<<s.grid, kThreads, s.smem, st>>>(in, scale, out, sh.vel64, sh.iperm, sh.K, sh.Np, sh.Q, sh.Qp, s.rows,
+  const auto plan = decode_plan<ST>(sh);
+  const Split& s = plan.split;
+  plan.kernel<<<s.grid, kThreads, s.smem, st>>>(in, scale, out, sh.vel64, sh.iperm, sh.K, sh.Np, sh.Q, sh.Qp, s.rows,
                                            int(s.tables));
   return cudaGetLastError();
 }
@@ -489,10 +505,8 @@ cudaError_t moments_as(const Shape& sh, const void* in, const float* scale, cons
   int G = 1;
   while (G < 32 && G < chunks) G *= 2;
   const int64_t nodes = sh.K * sh.Np;
-  int nsm = 152;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, sh.device);
   const int64_t per_block = 4 * (kThreads / G);
-  const int grid = int(std::max<int64_t>(1, std::min<int64_t>((nodes + per_block - 1) / per_block, int64_t(nsm) * 32)));
+  const int grid = int(std::max<int64_t>(1, std::min<int64_t>((nodes + per_block - 1) / per_block, int64_t(sh.nsm) * 32)));
   moments_kernel<ST><<<grid, kThreads, 0, st>>>(in, scale, static_cast<const typename ST::R*>(vel), nodes, sh.Np,
                                                 sh.Qp, G, rho, ux, uy);
   return cudaGetLastError();
@@ -509,6 +523,15 @@ cudaError_t encode_any(const Shape& sh, const TIn* in, void* out, float* scale, 
 }
 
 }  // namespace
+
+cudaError_t prepare(const Shape& sh) {
+  switch (sh.store) {
+    case kStoreF64: return prepare_as<StoreF64>(sh);
+    case kStoreF32: return prepare_as<StoreF32>(sh);
+    case kStoreBF16: return prepare_as<StoreBF16>(sh);
+    default: return prepare_as<StoreF16>(sh);
+  }
+}
 
 cudaError_t encode(const Shape& sh, const double* in, void* out, float* scale, cudaStream_t st) {
   return encode_any(sh, in, out, scale, st);

@@ -14,8 +14,13 @@ struct Shape {
   int Np = 0, Q = 0, Qp = 0;
   const double* vel64 = nullptr;   // [3][Qp] e_x, e_y, w in the internal order
   const int32_t* iperm = nullptr;  // [Q] internal index of canonical velocity c
-  int device = 0;
+  int nsm = 0;                     // SMs of the device and shared memory of one, bytes
+  int smem_sm = 0;
 };
+
+// Once per state type and sizes, before the first of the calls below: lets their kernels
+// take the shared memory that these sizes need.
+cudaError_t prepare(const Shape& sh);
 
 // canonical FP64 or FP32 [K][Np][Q] -> internal storage [K][Np][Qp] (padding
 // velocities zero; deviation forms: the per-element scale too)
