@@ -17,6 +17,7 @@
 #include "implicit_space.h"
 #include "krylov.h"
 #include "stage_dispatch.h"
+#include "tile_rule.h"
 #include "transfer.h"
 
 namespace {
@@ -501,66 +502,7 @@ int configure_ws(Batch& b, Group& g, int groups = -1) {
   return FEDBM_OK;
 }
 
-// The FMA kernel's tile where the caller leaves it open: elements and threads per
-// CTA by velocity count, degree, state and the group's element count K.  FP32
-// arithmetic takes two velocities per thread, FP64 one.
-//
-// Where the elements do not fill the SMs several times over (K below 16 per SM),
-// small tiles spread them (about two CTAs per SM) and get more threads than items,
-// which the moment reduction uses; one tile per SM with idle SMs beside it was the
-// rule before.  Above that, 16 velocities run best in CTAs of one warp (no barrier
-// ever waits for another warp), with two items per thread at low degree once there
-// are enough of them.  Stage times on the GB300, us, this rule against 8 (degree <= 2:
-// 16) elements and one thread per item: FP32, 16 velocities, degree 1, 3, 5: K = 128
-// 5.6, 6.6, 8.2 against 6.3, 8.2, 11.9; K = 2,048 5.8, 7.0, 9.4 against 6.4, 8.2, 11.5;
-// K = 51,200 15.7, 38.5, 80.7 against 18.2, 39.6, 82.6; BF16 degree 1, 2, K = 204,800
-// 58.9, 96.3 against 93.9, 126.0; 36 velocities, degree 2, 4: K = 512 6.6, 8.4 against
-// 7.4, 11.1; K = 18,432 degree 2 23.5 against 27.5; FP64, 16 velocities, degree 3: K =
-// 128, 512, 2,048 20.9, 23.0, 39.0 against 28.7, 28.7, 42.7; D2Q1089 at degree 4, K =
-// 800, 256 threads instead of 128: FP32 88.6 against 102.4, BF16 108.9 against 146.7 (at
-// degree 1, 1,024 velocities, FP16, 20M values: 169 against 123, so not there).
-void auto_tile(const Group& g, int* epc, int* tpb) {
-  const bool f64 = g.store == kStoreF64;
-  const int64_t K = g.K;
-  const bool few = K < 16 * 152;
-  const int spread = int(std::min<int64_t>(4, (K + 303) / 304));  // elements per CTA, two CTAs per SM
-  if (g.Qp == 16 && f64) {
-    *epc = !few ? 8 : K <= 304 ? 1 : 2;
-    *tpb = !few || K <= 608 ? 128 : K <= 1216 ? 64 : 32;
-  } else if (g.Qp == 16) {
-    *epc = few ? spread : K < 32768 ? 4 : g.p <= 3 ? 8 : 4;
-    if (K >= 32768 && g.p == 1 && g.store >= kStoreBF16) *epc = 16;
-    *tpb = few ? 32 * spread : 32;
-  } else if (g.Qp < 128 && !f64) {
-    *epc = std::max(1, 128 / g.Qp);
-    if (few) *epc = std::min(*epc, spread);
-    *tpb = few ? std::min(128, 64 * *epc) : g.p <= 2 && K >= 64 * 152 ? 32 : 64;
-  } else {
-    *epc = std::max(1, 128 / g.Qp);
-    const int items = *epc * g.Qp / (f64 ? 1 : 2);
-    const bool wide = !f64 && items >= 512 && (g.p >= 3 || (g.p == 2 && items > 512));
-    *tpb = wide ? 256 : std::min(128, std::max(32, (items + 31) / 32 * 32));
-  }
-}
-
-// Velocities per thread of the FMA kernel's update (FP32 arithmetic) on a tile of epc
-// elements and tpb threads: two, the faster where the tile has a pair for every thread, as
-// the automatic tiles of enough elements have; one on a tile that a caller gives a thread
-// for every value, or a warp without a pair, and that has neighbours to share its SM with
-// (from 16 elements per SM up, or tiles of one element where they are more than two per
-// SM).  There idle threads would hold registers that keep other CTAs off the SM: one step of
-// 20M values, us, with one kernel of one velocity per thread (before), two, one: 256
-// velocities, 256 threads, FP32 degree 3, 4, 5 468, 450, 460; 532, 491, 769; 406, 377, 362;
-// 16 velocities, 8 elements on 128 threads, BF16 degree 4, 5 793, 753; 681, 822; 506, 526;
-// 36 velocities, 4 elements on 128 threads, degree 3 FP32, FP16 572, 803; 708, 915; 538,
-// 797.  Below those counts two was as fast or faster (36 velocities, 264 elements, 4 on 128
-// threads, degree 5 FP32 88; 53; 59).
-int stage_lanes(const Group& g, int epc, int tpb) {
-  const int values = epc * g.Qp, pairs = values / 2;
-  const bool idle = tpb >= values || tpb > (pairs + 31) / 32 * 32;
-  const bool shared = g.K >= 16 * 152 || (epc == 1 && g.K > 2 * 152);
-  return g.store != kStoreF64 && idle && shared ? 1 : 2;
-}
+TileShape tile_shape(const Batch& b, const Group& g) { return TileShape{g.p, g.store, g.Qp, g.K, b.nsm}; }
 
 // Tile shape, pipeline depth and persistent grid of a group's stage kernel.
 int configure_tiles(Batch& b, Group& g, int epc, int tpb, int stages) {
@@ -576,7 +518,7 @@ int configure_tiles(Batch& b, Group& g, int epc, int tpb, int stages) {
   // the group is changed only once the whole configuration is valid
   int e_pc = epc, t_pb = tpb;
   if (epc <= 0 && tpb <= 0) {
-    auto_tile(g, &e_pc, &t_pb);
+    auto_tile(tile_shape(b, g), &e_pc, &t_pb);
   } else {
     if (epc <= 0) e_pc = g.Qp < 128 ? std::max(1, 128 / g.Qp) : 1;
     if (tpb <= 0) t_pb = std::min(128, std::max(32, (e_pc * g.Qp + 31) / 32 * 32));
@@ -593,7 +535,7 @@ int configure_tiles(Batch& b, Group& g, int epc, int tpb, int stages) {
   const StageEntry e = stage_entry(g.p);
   // the kernel's dynamic shared-memory limit stays at the maximum, so that
   // groups of one batch sharing this kernel with other tiles keep launching
-  const int lanes = stage_lanes(g, e_pc, t_pb);
+  const int lanes = stage_lanes(tile_shape(b, g), e_pc, t_pb);
   FEDBM_CK(e.set_smem(g.store, g.Qp, lanes, kMaxSmem));
   const int nsm = b.nsm;
   const int per_sm = e.occupancy(g.store, g.Qp, lanes, t_pb, smem);
@@ -1169,7 +1111,7 @@ int create_batch(const fedbm_case_desc* cd, int ncases, void* stream, Batch** ou
            // warp-specialised form takes over where it exists (D2Q1089, degree 5, FP32:
            // 700 us against 1103 us for a step of 20M values)
            const bool too_big = stage_smem_bytes(g.p, g.store, std::max(1, epc), g.Qp, 1) > kMaxSmem;
-           const bool wide = epc == 0 && tpb == 0 && st == 0 && g.K >= 2 * 152 && ws_default(g);
+           const bool wide = epc == 0 && tpb == 0 && st == 0 && g.K >= 2 * b->nsm && ws_default(g);
            const int ncl = g.vsplit >= 2 ? g.vsplit
                            : g.vsplit == 0 && too_big && !want_tc && !wide ? auto_cluster(g) : 0;
            if (ncl >= 2) {

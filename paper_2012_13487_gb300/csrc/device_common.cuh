@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "store_kind.h"
+
 namespace fedbm {
 
 // FP32 -> FP64 with integer operations for zeros and normal numbers: the
@@ -18,10 +20,6 @@ __device__ __forceinline__ double widen(float x) {
   return __hiloint2double(int(hi), int(u << 29));
 }
 
-// Storage forms of the distribution state.  Plain forms store f itself; the
-// deviation forms store q with f_i = w_i (1 + s_k q_i), s_k a per-element
-// power-of-two scale, and compute in FP32.
-enum StoreKind { kStoreF64 = 0, kStoreF32 = 1, kStoreBF16 = 2, kStoreF16 = 3 };
 
 struct StoreF64 {
   using S = double;
