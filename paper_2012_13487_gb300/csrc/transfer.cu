@@ -77,18 +77,19 @@ struct Walk {
 // (f - w) / w rounded to FP32, as the FP64 quotient rounds, without FP64 arithmetic per
 // value (its rate is low here): w is held as three FP32 pieces, all its 53 bits, and 1/w
 // as two.  x - w is formed as a sum s + low whose rounding errors are kept (Knuth's
-// two-sum, The Art of Computer Programming vol. 2, 4.2.2, theorem B), its product with
-// 1/w likewise with the product's error from an FMA (Dekker 1971), so that what is
-// rounded in the last addition is off by about 2^-46.  Over 16 to 1,089 velocities and
+// two-sum, The Art of Computer Programming vol. 2, 4.2.2, theorem B), and its product with
+// 1/w ends in an FMA that adds the small terms to the exact leading product, so that what
+// is rounded there is off by about 2^-46.  Over 16 to 1,089 velocities and
 // deviations of 1e-7 to 1e6 the result is off by at most 1.0 units of 2^-24 |d|, as the FP64
 // quotient rounded to FP32 is; one difference and one product in plain FP32 had 3.6.
 // An FP64 x that FP32 holds exactly takes the same path, so that an FP32 value and the
 // same value given in FP64 give the same bits; any other is subtracted and scaled in
-// FP64.  Weights below 2^-96, whose last bits FP32's denormals do not hold, and results
-// out of its range take the FP64 quotient.
+// FP64.  Weights below 2^-96, whose last bits FP32's denormals do not hold (marked by an
+// inverse that is not a number), weights of 0 and results out of FP32's range are told by
+// one comparison of the result and take the FP64 quotient.
 constexpr double kTinyWeight = 1.262177448353619e-29;  // 2^-96
 struct __align__(16) DevRow {
-  float wh, wl, ih, il;  // ih < 0: tiny weight, 0: weight 0
+  float wh, wl, ih, il;  // ih: NaN for a tiny weight or 0
 };
 struct __align__(8) DevIndex {
   float wll;
@@ -111,24 +112,24 @@ __device__ __forceinline__ float two_difference_ordered(float a, float b, float&
   err = -__fadd_rn(b, __fadd_rn(s, -a));
   return s;
 }
-__device__ __noinline__ float deviation64(double x, double w) { return float((x - w) / w); }
+__device__ __noinline__ float deviation64(double x, double w) { return w > 0.0 ? float((x - w) / w) : 0.f; }
 template <typename TIn>
 __device__ __forceinline__ float deviation(TIn x, const DevTable& t, int c, const DevIndex& at) {
-  const DevRow r = t.row[c];
-  if (r.ih <= 0.f) return r.ih == 0.f ? 0.f : deviation64(double(x), t.w64[at.at]);
   const float xf = float(x);
-  if constexpr (sizeof(TIn) == 8) {
-    if (__double_as_longlong(widen(xf)) != __double_as_longlong(x)) {
-      const double2 w = t.wide[c];
-      return float((x - w.x) * w.y);
-    }
+  bool narrow = true;
+  if constexpr (sizeof(TIn) == 8) narrow = __double_as_longlong(widen(xf)) == __double_as_longlong(x);
+  float d;
+  if (narrow) {
+    const DevRow r = t.row[c];
+    float ea, es;
+    // x - wh is 0 or, as a multiple of half a unit in wh's last place, at least |wl|
+    const float s = two_difference_ordered(two_difference(xf, r.wh, ea), r.wl, es);
+    const float low = __fadd_rn(__fadd_rn(ea, es), -at.wll);
+    d = fmaf(s, r.ih, fmaf(s, r.il, __fmul_rn(low, r.ih)));
+  } else {
+    const double2 w = t.wide[c];
+    d = float((x - w.x) * w.y);
   }
-  float ea, es;
-  // x - wh is 0 or, as a multiple of half a unit in wh's last place, at least |wl|
-  const float s = two_difference_ordered(two_difference(xf, r.wh, ea), r.wl, es);
-  const float low = __fadd_rn(__fadd_rn(ea, es), -at.wll);
-  const float p = __fmul_rn(s, r.ih), ep = fmaf(s, r.ih, -p);
-  const float d = __fadd_rn(p, __fadd_rn(ep, fmaf(s, r.il, __fmul_rn(low, r.ih))));
   return fabsf(d) <= 3e38f ? d : deviation64(double(x), t.w64[at.at]);
 }
 
@@ -141,10 +142,10 @@ __device__ __forceinline__ float deviation(TIn x, const DevTable& t, int c, cons
 // with two FP64 divisions per value, scattered 2- and 4-byte stores and an
 // integer division per value (GB300, ncu): BF16 from FP32 input 15.3 ms at 335M
 // values (1,024 velocities), 1.45 ms at 31M (256) and 2.44 ms at 44M (16), FP32
-// from FP32 71 us at 31M; now (events around the call) 1.02 ms, 97 us, 142 us and 49 us.
-// Of these, the quotient with its rounding errors costs the 16-bit forms 15 us at 31M and
-// 17 us at 44M against a difference and a product in plain FP32, whose codes can round the
-// other way near a tie; from FP64 input BF16 takes 3.29 ms, 313 us and 439 us.
+// from FP32 71 us at 31M; now (events around the call) 0.93 ms, 90 us, 132 us and 49 us.
+// Of these, the quotient with its rounding errors costs the 16-bit forms 7 us at 31M and
+// at 44M against a difference and a product in plain FP32, whose codes can round the other
+// way near a tie; from FP64 input BF16 takes 3.27 ms, 310 us and 438 us.
 template <class ST, typename TIn, bool kWarp>
 __global__ void __launch_bounds__(kThreads) encode_kernel(const TIn* __restrict__ in, void* out, float* scale,
                                                           const double* __restrict__ vel64,
@@ -168,10 +169,10 @@ __global__ void __launch_bounds__(kThreads) encode_kernel(const TIn* __restrict_
       const double w = w64[i];
       const float wh = float(w), wl = float(w - double(wh)), wll = float(w - double(wh) - double(wl));
       const double iw = w > 0 ? 1.0 / w : 0.0;
-      const float ih = !(w > 0) ? 0.f : w < kTinyWeight ? -1.f : float(iw);
+      const float ih = w < kTinyWeight ? __int_as_float(0x7fffffff) : float(iw);
       // the rest of 1/w from the FP64 residual of w ih, whose product has at most 77 bits:
       // formed as an FMA
-      rows_w[c] = DevRow{wh, wl, ih, ih > 0.f ? float(fma(-w, double(ih), 1.0) * iw) : 0.f};
+      rows_w[c] = DevRow{wh, wl, ih, float(fma(-w, double(ih), 1.0) * iw)};
       index[c] = DevIndex{wll, i};
       if constexpr (sizeof(TIn) == 8) wide[c] = make_double2(w, iw);
     } else {
