@@ -8,11 +8,9 @@ leaves open: warp & blend nodes with alpha = 0 here).  The FP32 kernels can
 therefore take them as instruction immediates instead of loading them from
 constant memory.  The values are the library's own operators
 (``fedbm_ref_operators``) rounded to FP32 exactly as the runtime upload rounds
-them; a CPU test checks that the committed file still matches.  Degree 6 (784
-entries per derivative matrix) keeps constant memory, and at degree 5 only the
-kernels that the workloads use take the table (the kernel selects them), since
-folding the tables into every unrolled node loop makes those translation units
-take many minutes to compile.  Run as
+them; a CPU test checks that the committed file still matches.  Every kernel of
+degree <= 5 that computes in FP32 takes the even and odd parts; degree 6 (784
+entries per derivative matrix) keeps constant memory.  Run as
 ``python -m paper_2012_13487_gb300.csrc.gen_ops_tables`` after a build.
 """
 import os
@@ -85,7 +83,8 @@ def render():
     lines = ["// Generated by gen_ops_tables.py from the library's operators: FP32 Dr, Ds",
              "// (row-major Np x Np) and LIFT (row-major Np x 3(p+1)) of the FEDBM_P of the",
              "// including translation unit, and Se, So, De, Do, Le, Lo of stage_eo.cuh, in the",
-             "// order of the runtime upload.  Do not edit."]
+             "// order of the runtime upload.  The kernels take the second table; the first is the",
+             "// one a test holds against the library's operators.  Do not edit."]
     for p in range(MAX_P + 1):
         lines.append("#%s FEDBM_P == %d" % ("if" if p == 0 else "elif", p))
         lines += macro("FEDBM_OPS32_TABLE", table(p)) + macro("FEDBM_EO32_TABLE", eo_table(p))

@@ -61,8 +61,6 @@ __host__ __device__ constexpr EoPairs eo_pairs() {
 
 static __constant__ double c_eo64[EO_N];
 static __constant__ float c_eo32[EO_N];
-// every FP32 coefficient twice, as the broadcast operand of a packed FMA
-static __constant__ unsigned long long c_eo32x2[EO_N];
 
 // Coefficient idx in the compute precision.  kImm: this degree's FP32 table as
 // compile-time constants (the operators depend only on the degree, and with the
@@ -111,7 +109,6 @@ struct EoPacked {
     return r;
   }
   static __device__ __forceinline__ T fmat(T x, T y, T z) { return f2fma(x, y, z); }
-  static __device__ __forceinline__ T fmac(int idx, T x, T z) { return f2fma(c_eo32x2[idx], x, z); }
 };
 
 // Two velocities per thread with the operators as immediates: additions and

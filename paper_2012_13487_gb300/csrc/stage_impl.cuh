@@ -29,7 +29,6 @@
 #include "device_common.cuh"
 #include "stage_dispatch.h"
 
-#include <cstring>
 #include <type_traits>
 
 
@@ -86,16 +85,6 @@ __device__ __forceinline__ unsigned long long f2mul(unsigned long long a, unsign
 }
 
 #include "stage_eo.cuh"
-
-// Which FMA kernels take the operators as immediates: every FP32-arithmetic
-// kernel up to degree 4; at degree 5 only the compile-time velocity counts of
-// the FP32 and BF16 states, which keeps that translation unit's compile time
-// within a few minutes.
-template <class ST, int QT>
-__host__ __device__ constexpr bool ops_immediate() {
-  return kHaveOpsTable && sizeof(typename ST::R) == 4 &&
-         (P <= 4 || (QT > 0 && (ST::kind == kStoreF32 || ST::kind == kStoreBF16)));
-}
 
 // ---- moment accumulators ----------------------------------------------------
 struct AccD {
@@ -1242,24 +1231,16 @@ cudaError_t set_smem(int store_kind, int Qp, int lanes, size_t smem) {
 cudaError_t upload(const double* Dr, const double* Ds, const double* LIFT) {
   double h64[OPS_N], eo64[EO_N] = {};
   float eo32[EO_N];
-  unsigned long long eo32x2[EO_N];
   for (int j = 0; j < NP * NP; ++j) {
     h64[OFF_DR + j] = Dr[j];
     h64[OFF_DS + j] = Ds[j];
   }
   for (int j = 0; j < NP * NF; ++j) h64[OFF_LIFT + j] = LIFT[j];
   eo_coefficients(Dr, Ds, LIFT, eo64);
-  for (int j = 0; j < EO_N; ++j) {
-    eo32[j] = float(eo64[j]);
-    uint32_t bits;
-    std::memcpy(&bits, &eo32[j], 4);
-    eo32x2[j] = (static_cast<unsigned long long>(bits) << 32) | bits;
-  }
+  for (int j = 0; j < EO_N; ++j) eo32[j] = float(eo64[j]);
   cudaError_t e = cudaMemcpyToSymbol(c_ops64, h64, sizeof(h64));
   if (e != cudaSuccess) return e;
   e = cudaMemcpyToSymbol(c_eo64, eo64, sizeof(eo64));
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpyToSymbol(c_eo32x2, eo32x2, sizeof(eo32x2));
   if (e != cudaSuccess) return e;
   return cudaMemcpyToSymbol(c_eo32, eo32, sizeof(eo32));
 }
