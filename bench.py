@@ -772,7 +772,8 @@ def run_ours(args, w, name):
             "mass_after": mass,
             "forms": forms,
         }
-        print(json.dumps(line), flush=True)
+        print("bench detail: " + json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(contract_line(line)), flush=True)
     if dist is not None:
         dist.destroy_process_group()
 
@@ -804,6 +805,28 @@ FORM_PROFILES = {
     "cavity_kn8_128x128x2_p3_nc32_bf16_red_comp": "cavity_kn8_128x128x2_p3_nc32x32_bf16",
     "cavity_kn8_32x32x2_p5_d2q1089_fp32_split": "cavity_kn8_32x32x2_p5_nc33x33_sqrt2_fp32",
 }
+
+
+def contract_line(line):
+    """The line that goes to standard output: every key of the contract, short enough to be
+    kept whole by a reader of the last few kilobytes; what explains it (the other forms, the
+    paths and samples in words) goes to standard error with the full line.  Of the other
+    forms the values stay."""
+    out = {k: v for k, v in line.items() if k != "forms"}
+
+    def drop(key, *names):
+        if isinstance(out.get(key), dict):
+            out[key] = {k: v for k, v in out[key].items() if k not in names}
+
+    drop("error", "copy")
+    drop("cpu_baseline", "all_cores")
+    drop("roofline", "algorithmic_bytes_per_launch")
+    drop("e2e", "serial", "path")
+    drop("repeats", "ms_per_step_min", "ms_per_step_max", "ms_per_step_median")
+    if isinstance(line.get("forms"), dict):
+        out["forms"] = {k: float("%.4g" % v["value"]) for k, v in line["forms"].items()
+                        if isinstance(v, dict) and isinstance(v.get("value"), (int, float))}
+    return out
 
 
 def measure_forms(args, w, st, value, roof, error):
