@@ -277,6 +277,7 @@ struct Group {
   void* vel = nullptr;          // [kVelRows][Qp]
   double* vel64 = nullptr;      // [3][Qp]
   int32_t* iperm = nullptr;     // [Q] internal index of canonical velocity c
+  void* weights = nullptr;      // deviation forms: tables of the load (transfer.h), [Q] each
   void* wall_feq = nullptr;     // [4 * ncases][Qp]
   void* wall_den_inv = nullptr; // [4 * ncases]
   double* Jk = nullptr;         // [K]
@@ -967,6 +968,17 @@ int build_group(Batch& b, Group& g) {
   if ((rc = upload_vec(nbr, reinterpret_cast<void**>(&g.nbr))) != FEDBM_OK) return rc;
   if ((rc = upload_vec(v64, reinterpret_cast<void**>(&g.vel64))) != FEDBM_OK) return rc;
   if ((rc = upload_vec(iperm, reinterpret_cast<void**>(&g.iperm))) != FEDBM_OK) return rc;
+  if (g.store >= kStoreBF16) {
+    std::vector<transfer::DevRow> row(Q);
+    std::vector<transfer::DevIndex> index(Q);
+    std::vector<double> wide(size_t(2) * Q);
+    transfer::weight_tables(&v64[size_t(2) * Qp], iperm.data(), Q, row.data(), index.data(), wide.data());
+    std::vector<unsigned char> all(size_t(40) * Q);
+    std::memcpy(all.data(), row.data(), size_t(16) * Q);
+    std::memcpy(all.data() + size_t(16) * Q, wide.data(), size_t(16) * Q);
+    std::memcpy(all.data() + size_t(32) * Q, index.data(), size_t(8) * Q);
+    if ((rc = upload_vec(all, &g.weights)) != FEDBM_OK) return rc;
+  }
   if ((rc = upload_vec(Jk, reinterpret_cast<void**>(&g.Jk))) != FEDBM_OK) return rc;
   if ((rc = upload_vec(mw, reinterpret_cast<void**>(&g.mw))) != FEDBM_OK) return rc;
   if (g.store == kStoreF64) {
@@ -1004,7 +1016,7 @@ void free_batch(Batch* b) {
       cudaFree(g.f[c]);
       cudaFree(g.scale[c]);
     }
-    void* bufs[] = {g.res, g.nbr, g.geo, g.vel, g.vel64, g.iperm, g.wall_feq, g.wall_den_inv, g.Jk, g.mw, g.partial,
+    void* bufs[] = {g.res, g.nbr, g.geo, g.vel, g.vel64, g.iperm, g.weights, g.wall_feq, g.wall_den_inv, g.Jk, g.mw, g.partial,
                     g.flag, g.sr_step};
     for (void* p : bufs) cudaFree(p);
     if (g.branch) cudaStreamDestroy(g.branch);
@@ -1026,6 +1038,13 @@ transfer::Shape layout_of(const Batch& b, const Group& g, const Case& cs) {
   t.Qp = g.Qp;
   t.vel64 = g.vel64;
   t.iperm = g.iperm;
+  if (g.weights) {  // rows, then w and 1/w, then indices: 40 bytes a velocity
+    const size_t q = size_t(g.Q);
+    unsigned char* base = static_cast<unsigned char*>(g.weights);
+    t.weights.row = reinterpret_cast<const transfer::DevRow*>(base);
+    t.weights.wide = reinterpret_cast<const double*>(base + 16 * q);
+    t.weights.index = reinterpret_cast<const transfer::DevIndex*>(base + 32 * q);
+  }
   t.nsm = b.nsm;
   t.smem_sm = b.smem_sm;
   return t;

@@ -2,6 +2,7 @@
 #include "transfer.h"
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "device_common.cuh"
@@ -34,9 +35,9 @@ struct Split {
 
 inline size_t up16(size_t b) { return (b + 15) / 16 * 16; }
 
-Split split_for(const Shape& sh, size_t table_bytes, size_t value_bytes) {
+Split split_for(const Shape& sh, size_t table_bytes, size_t value_bytes, bool by_warp) {
   Split s;
-  s.warp = sh.Np * sh.Qp <= kWarpValues;
+  s.warp = by_warp;
   s.tables = up16(table_bytes);
   const size_t row = size_t(sh.Qp) * value_bytes;
   const int groups = s.warp ? kThreads / 32 : 1;
@@ -88,13 +89,8 @@ struct Walk {
 // inverse that is not a number), weights of 0 and results out of FP32's range are told by
 // one comparison of the result and take the FP64 quotient.
 constexpr double kTinyWeight = 1.262177448353619e-29;  // 2^-96
-struct __align__(16) DevRow {
-  float wh, wl, ih, il;  // ih: NaN for a tiny weight or 0
-};
-struct __align__(8) DevIndex {
-  float wll;
-  int at;  // internal index
-};
+// ih: NaN for a tiny weight or 0.  (Laid out by weight_tables once per solver; in every CTA
+// instead, the FP64 quotients were half of the time of a small load.)
 struct DevTable {  // canonical order
   const DevRow* row;
   const DevIndex* index;
@@ -149,34 +145,28 @@ __device__ __forceinline__ float deviation(TIn x, const DevTable& t, int c, cons
 template <class ST, typename TIn, bool kWarp>
 __global__ void __launch_bounds__(kThreads) encode_kernel(const TIn* __restrict__ in, void* out, float* scale,
                                                           const double* __restrict__ vel64,
-                                                          const int32_t* __restrict__ iperm, int64_t K, int Np,
-                                                          int Q, int Qp, int rows, int table_bytes) {
+                                                          const int32_t* __restrict__ iperm, Weights weights,
+                                                          int64_t K, int Np, int Q, int Qp, int rows,
+                                                          int table_bytes) {
   using S = typename ST::S;
   using T = std::conditional_t<ST::dev, float, S>;  // staged values
   constexpr int V = 16 / int(sizeof(S));
   extern __shared__ __align__(16) unsigned char smem[];
   const double* w64 = vel64 + 2 * Qp;
   // tables in canonical order: the internal index, and for the deviation forms the weight's
-  // pieces (sized in encode_as)
+  // pieces (sized in encode_plan)
   DevRow* rows_w = reinterpret_cast<DevRow*>(smem);
   DevIndex* index = reinterpret_cast<DevIndex*>(rows_w + Q);
   double2* wide = reinterpret_cast<double2*>(smem + (size_t(24) * Q + 15) / 16 * 16);
   int* perm = reinterpret_cast<int*>(smem);
   const DevTable dt{rows_w, index, wide, w64};
   for (int c = threadIdx.x; c < Q; c += kThreads) {
-    const int i = iperm[c];
     if constexpr (ST::dev) {
-      const double w = w64[i];
-      const float wh = float(w), wl = float(w - double(wh)), wll = float(w - double(wh) - double(wl));
-      const double iw = w > 0 ? 1.0 / w : 0.0;
-      const float ih = w < kTinyWeight ? __int_as_float(0x7fffffff) : float(iw);
-      // the rest of 1/w from the FP64 residual of w ih, whose product has at most 77 bits:
-      // formed as an FMA
-      rows_w[c] = DevRow{wh, wl, ih, float(fma(-w, double(ih), 1.0) * iw)};
-      index[c] = DevIndex{wll, i};
-      if constexpr (sizeof(TIn) == 8) wide[c] = make_double2(w, iw);
+      rows_w[c] = weights.row[c];
+      index[c] = weights.index[c];
+      if constexpr (sizeof(TIn) == 8) wide[c] = reinterpret_cast<const double2*>(weights.wide)[c];
     } else {
-      perm[c] = i;
+      perm[c] = iperm[c];
     }
   }
   const int G = kWarp ? 32 : kThreads;
@@ -276,44 +266,31 @@ __global__ void __launch_bounds__(kThreads) encode_kernel(const TIn* __restrict_
   }
 }
 
-// Decode: the mirror image.  The internal row is read as 16-byte vectors and
-// scattered into shared memory by the canonical order; the caller's rows are
-// written along the canonical order.  Deviation forms stage s q (exact in
-// FP32: s is a power of two) and form w + w (s q) with one FP64 FMA per value.
-// Before (gathered 2- and 4-byte loads, three FP64-rate operations and two
-// integer divisions per value): 2.44 ms at 335M BF16 values, 90 us at 31M FP32
-// values; now 1.34 ms and 73 us (56 us for the latter's bytes).
+// Read-out of plain state through shared memory: the mirror image.  The internal row is
+// read as 16-byte vectors and scattered into shared memory by the canonical order; the
+// caller's rows are written along the canonical order.  31M FP32 values 73 us, 56 us the bytes
+// at the measured rate; gathered 4-byte loads, a thread per value, 90 us.
 template <class ST, bool kWarp>
-__global__ void __launch_bounds__(kThreads) decode_kernel(const void* __restrict__ in,
-                                                          const float* __restrict__ scale, double* __restrict__ out,
-                                                          const double* __restrict__ vel64,
+__global__ void __launch_bounds__(kThreads) decode_kernel(const void* __restrict__ in, double* __restrict__ out,
                                                           const int32_t* __restrict__ iperm, int64_t K, int Np,
                                                           int Q, int Qp, int rows, int table_bytes) {
   using S = typename ST::S;
-  using T = std::conditional_t<ST::dev, float, S>;
   constexpr int V = 16 / int(sizeof(S));
   extern __shared__ __align__(16) unsigned char smem[];
-  double* wc = reinterpret_cast<double*>(smem);  // deviation forms: w in canonical order
-  int* inv = reinterpret_cast<int*>(smem + (ST::dev ? size_t(Q) * 8 : 0));  // canonical index, -1 for padding
-  const double* w64 = vel64 + 2 * Qp;
+  int* inv = reinterpret_cast<int*>(smem);  // canonical index, -1 for padding
   for (int i = threadIdx.x; i < Qp; i += kThreads) inv[i] = -1;
   __syncthreads();
-  for (int c = threadIdx.x; c < Q; c += kThreads) {
-    const int i = iperm[c];
-    inv[i] = c;
-    if constexpr (ST::dev) wc[c] = w64[i];
-  }
+  for (int c = threadIdx.x; c < Q; c += kThreads) inv[iperm[c]] = c;
   const int G = kWarp ? 32 : kThreads;
   const int grp = kWarp ? threadIdx.x / 32 : 0, lane = kWarp ? threadIdx.x % 32 : threadIdx.x;
   const int ngroups = kWarp ? kThreads / 32 : 1;
-  T* buf = reinterpret_cast<T*>(smem + table_bytes) + size_t(grp) * rows * Qp;
+  S* buf = reinterpret_cast<S*>(smem + table_bytes) + size_t(grp) * rows * Qp;
   __syncthreads();
 
   const int vrow = Qp / V;  // vectors per row
   for (int64_t k = blockIdx.x * int64_t(ngroups) + grp; k < K; k += int64_t(gridDim.x) * ngroups) {
     const S* src = static_cast<const S*>(in) + k * Np * Qp;
     double* dst = out + k * Np * Q;
-    const float s = ST::dev ? scale[k] : 0.f;
     for (int r0 = 0; r0 < Np; r0 += rows) {
       const int nr = min(rows, Np - r0);
       const uint4* s0 = reinterpret_cast<const uint4*>(src + size_t(r0) * Qp);
@@ -329,14 +306,11 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const void* __restrict
         for (int u = 0; u < U; ++u) {
           if (v + u * G >= nvec) break;
           const S* q = reinterpret_cast<const S*>(&x[u]);
-          T* row = buf + size_t(w.row) * Q;
+          S* row = buf + size_t(w.row) * Q;
 #pragma unroll
           for (int j = 0; j < V; ++j) {
             const int c = inv[w.c * V + j];
-            if (c >= 0) {
-              if constexpr (ST::dev) row[c] = s * ST::to_r(q[j]);
-              else row[c] = q[j];
-            }
+            if (c >= 0) row[c] = q[j];
           }
           w.next();
         }
@@ -345,14 +319,46 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const void* __restrict
       group_sync<kWarp>();
       double* d0 = dst + size_t(r0) * Q;
       const int n = nr * Q;
-      if constexpr (ST::dev) {
-        Walk c(lane, G, Q);
-        for (int j = lane; j < n; j += G, c.next()) d0[j] = fma(wc[c.c], widen(buf[j]), wc[c.c]);
-      } else {
-        for (int j = lane; j < n; j += G) d0[j] = widen(buf[j]);
-      }
+      for (int j = lane; j < n; j += G) d0[j] = widen(buf[j]);
       group_sync<kWarp>();
     }
+  }
+}
+
+// Loads of plain state and read-outs without the staging: a thread per value, scattered
+// and gathered by the velocity order.  Deviation forms are always read out so, as w + w (s q)
+// with one FP64 FMA per value; the product s q is exact in FP32 (s is a power of two).
+template <class ST, typename TIn>
+__global__ void __launch_bounds__(kThreads) encode_direct_kernel(const TIn* __restrict__ in, void* out,
+                                                                 const int32_t* __restrict__ iperm, int64_t K, int Np,
+                                                                 int Q, int Qp) {
+  using S = typename ST::S;
+  const int64_t k = blockIdx.x;
+  const TIn* src = in + k * Np * Q;
+  S* dst = static_cast<S*>(out) + k * Np * Qp;
+  const int pad = Qp - Q;
+  for (int j = threadIdx.x; j < Np * Q; j += blockDim.x) {
+    const int n = j / Q;
+    dst[n * Qp + iperm[j - n * Q]] = S(src[j]);
+  }
+  for (int j = threadIdx.x; j < Np * pad; j += blockDim.x) dst[(j / pad) * Qp + Q + j % pad] = S(0);
+}
+template <class ST>
+__global__ void __launch_bounds__(kThreads) decode_direct_kernel(const void* __restrict__ in,
+                                                                 const float* __restrict__ scale,
+                                                                 double* __restrict__ out,
+                                                                 const double* __restrict__ vel64,
+                                                                 const int32_t* __restrict__ iperm, int64_t rows,
+                                                                 int Np, int Q, int Qp) {
+  using S = typename ST::S;
+  const double* w64 = vel64 + 2 * Qp;
+  const int64_t n = rows * Q;
+  for (int64_t j = blockIdx.x * int64_t(kThreads) + threadIdx.x; j < n; j += int64_t(gridDim.x) * kThreads) {
+    const int64_t r = j / Q;
+    const int i = iperm[int(j - r * Q)];
+    const S q = static_cast<const S*>(in)[r * Qp + i];
+    if constexpr (ST::dev) out[j] = fma(w64[i], widen(scale[r / Np] * ST::to_r(q)), w64[i]);
+    else out[j] = widen(q);
   }
 }
 
@@ -366,7 +372,7 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const void* __restrict
 // values at 16 velocities (4 of 32 lanes busy; 26 us for the bytes) and 851 us
 // for 335M BF16 values at 1,024 velocities (96 bytes of table per 16 of state);
 // now 51 us and 192 us.
-template <class ST>
+template <class ST, int kNodes>
 __global__ void __launch_bounds__(kThreads) moments_kernel(const void* __restrict__ in,
                                                            const float* __restrict__ scale,
                                                            const typename ST::R* __restrict__ vel, int64_t nodes,
@@ -375,7 +381,6 @@ __global__ void __launch_bounds__(kThreads) moments_kernel(const void* __restric
   using R = typename ST::R;
   using S = typename ST::S;
   constexpr int V = 16 / int(sizeof(S));
-  constexpr int kNodes = 4;
   const int lane = threadIdx.x % G;
   const int64_t ngroups = int64_t(gridDim.x) * (kThreads / G);
   const R *ex = vel + kVelEx * Qp, *ey = vel + kVelEy * Qp, *wv = vel + kVelW * Qp;
@@ -447,6 +452,41 @@ __global__ void __launch_bounds__(kThreads) moments_kernel(const void* __restric
   }
 }
 
+// Where the direct kernels are taken: small calls, whose time is the staging's two trips
+// through shared memory and its tables, and shapes that the staged split serves badly (tiny
+// elements, of which a warp takes one at a time; elements of 768 to 1,536 values, whose eight
+// buffers leave an SM few CTAs; elements of several passes).  Staged against direct on the
+// GB300, us: loads of FP64 state, 1e4 values of 16 and 36
+// velocities 6.2 and 4.2, 1e6 and 2e7 values of 256 velocities at degree 2 10.3 and 7.6, 72.5
+// and 63.4, but 16 velocities at degree 2, 1e6 and 2e7 8.2 and 10.3, 65 and 109.  Read-outs:
+// 16 velocities at degree 0, 2e7 FP32 values 274 and 62; 256 at degree 0 and 4 50 and 63, 47
+// and 64, 1,089 at degree 5 67 and 61; BF16, 256 velocities, degree 4, 1e5, 4e6 and 2e7 values
+// 7.6 and 4.1, 22.6 and 19.5, 89 and 82.  Of the deviation forms' 65 shapes the staged read-out was
+// faster in one (8.3 and 10.3 us), so there is none any more.
+bool warp_split(const Shape& sh) { return sh.Np * sh.Qp <= kWarpValues; }
+bool direct_load(const Shape& sh, size_t value_bytes) {
+  if (!warp_split(sh)) return false;
+  const int64_t values = sh.K * sh.Np * sh.Q;
+  const int element = sh.Np * sh.Qp;
+  if (element > 1024) return value_bytes == 8 || values <= int64_t(8) << 20;
+  if (element > 768 && values <= int64_t(value_bytes == 8 ? 8 : 2) << 20) return true;
+  return sh.K <= 16 * sh.nsm && values <= 200000;
+}
+bool direct_read(const Shape& sh, size_t value_bytes) {
+  const int64_t values = sh.K * sh.Np * sh.Q;
+  const int element = sh.Np * sh.Qp;
+  const bool f64 = value_bytes == 8, large = values >= int64_t(8) << 20;
+  if (!warp_split(sh)) return element > 12000 || sh.K < (f64 ? 1 : 8) * sh.nsm;
+  return values < 800000 || element * int(value_bytes) < 1024 || (element > 1024 && (f64 || !large));
+}
+// Moments: one node per group of lanes instead of four where the nodes do not fill the SMs
+// (about 2.5 CTAs each), and for long FP64 rows.  Four against one, us: FP64, 672 nodes of 16
+// velocities 9.2 and 6.2, 360 nodes of 256 16.4 and 8.2, 840 and 19,840 of 1,024 35 and 14, 160 and
+// 151; BF16, 672 nodes of 16 5.1 and 4.1; FP32, 1.2M nodes of 16 29 and 44.
+bool few_nodes(const Shape& sh, int64_t nodes, int G, size_t r_bytes) {
+  return nodes * G <= int64_t(640) * sh.nsm || (r_bytes == 8 && sh.Qp >= 512);
+}
+
 // Work split and kernel of one transfer.
 template <class Kernel>
 struct Plan {
@@ -458,44 +498,73 @@ struct Plan {
   }
 };
 template <class ST, typename TIn>
-auto encode_plan(const Shape& sh) {
+auto encode_plan(const Shape& sh, bool by_warp) {
   // internal indices; deviation forms: six words a velocity, for FP64 input w and 1/w behind them
   const size_t q = size_t(sh.Q);
   const size_t tables = !ST::dev ? 4 * q : sizeof(TIn) == 8 ? up16(24 * q) + 16 * q : 24 * q;
-  const Split s = split_for(sh, tables, ST::dev ? 4 : sizeof(typename ST::S));
+  const Split s = split_for(sh, tables, ST::dev ? 4 : sizeof(typename ST::S), by_warp);
   auto kernel = s.warp ? &encode_kernel<ST, TIn, true> : &encode_kernel<ST, TIn, false>;
   return Plan<decltype(kernel)>{s, kernel};
 }
 template <class ST>
 auto decode_plan(const Shape& sh) {
-  const size_t tables = (ST::dev ? 8 * size_t(sh.Q) : 0) + 4 * size_t(sh.Qp);
-  const Split s = split_for(sh, tables, ST::dev ? 4 : sizeof(typename ST::S));
+  const Split s = split_for(sh, 4 * size_t(sh.Qp), sizeof(typename ST::S), warp_split(sh));
   auto kernel = s.warp ? &decode_kernel<ST, true> : &decode_kernel<ST, false>;
   return Plan<decltype(kernel)>{s, kernel};
 }
 
+// Elements by warps or by CTAs; few elements of the deviation forms by a CTA each, where a
+// warp would walk one alone (336 values, 24 elements, FP64 input: 10.3 us by warps, 8.2 with the
+// former CTA per element).
+template <class ST>
+bool load_by_warp(const Shape& sh) {
+  return warp_split(sh) && (!ST::dev || sh.Np * sh.Qp <= 128 || sh.K >= 8 * sh.nsm);
+}
+
+// For every element count: a batch has cases of the same sizes and different counts.
 template <class ST>
 cudaError_t prepare_as(const Shape& sh) {
-  cudaError_t e = encode_plan<ST, double>(sh).allow_smem();
-  if (e == cudaSuccess) e = encode_plan<ST, float>(sh).allow_smem();
-  return e == cudaSuccess ? decode_plan<ST>(sh).allow_smem() : e;
+  cudaError_t e = cudaSuccess;
+  for (bool by_warp : {false, true}) {
+    if (by_warp && !warp_split(sh)) continue;
+    if (e == cudaSuccess) e = encode_plan<ST, double>(sh, by_warp).allow_smem();
+    if (e == cudaSuccess) e = encode_plan<ST, float>(sh, by_warp).allow_smem();
+  }
+  if constexpr (!ST::dev)
+    if (e == cudaSuccess) e = decode_plan<ST>(sh).allow_smem();
+  return e;
 }
 
 template <class ST, typename TIn>
 cudaError_t encode_as(const Shape& sh, const TIn* in, void* out, float* scale, cudaStream_t st) {
-  const auto plan = encode_plan<ST, TIn>(sh);
+  if constexpr (!ST::dev) {
+    if (direct_load(sh, sizeof(typename ST::S))) {
+      const int block = std::min(kThreads, (sh.Np * sh.Q + 31) / 32 * 32);
+      encode_direct_kernel<ST, TIn><<<int(sh.K), block, 0, st>>>(in, out, sh.iperm, sh.K, sh.Np, sh.Q, sh.Qp);
+      return cudaGetLastError();
+    }
+  }
+  const auto plan = encode_plan<ST, TIn>(sh, load_by_warp<ST>(sh));
   const Split& s = plan.split;
-  plan.kernel<<<s.grid, kThreads, s.smem, st>>>(in, out, scale, sh.vel64, sh.iperm, sh.K, sh.Np, sh.Q, sh.Qp, s.rows,
-                                           int(s.tables));
+  plan.kernel<<<s.grid, kThreads, s.smem, st>>>(in, out, scale, sh.vel64, sh.iperm, sh.weights, sh.K, sh.Np, sh.Q,
+                                                sh.Qp, s.rows, int(s.tables));
   return cudaGetLastError();
 }
 
 template <class ST>
 cudaError_t decode_as(const Shape& sh, const void* in, const float* scale, double* out, cudaStream_t st) {
-  const auto plan = decode_plan<ST>(sh);
-  const Split& s = plan.split;
-  plan.kernel<<<s.grid, kThreads, s.smem, st>>>(in, scale, out, sh.vel64, sh.iperm, sh.K, sh.Np, sh.Q, sh.Qp, s.rows,
-                                           int(s.tables));
+  if (ST::dev || direct_read(sh, sizeof(typename ST::S))) {
+    const int64_t rows = sh.K * sh.Np;
+    const int64_t blocks = (rows * sh.Q + kThreads - 1) / kThreads;
+    const int grid = int(std::max<int64_t>(1, std::min<int64_t>(blocks, int64_t(sh.nsm) * 32)));
+    decode_direct_kernel<ST><<<grid, kThreads, 0, st>>>(in, scale, out, sh.vel64, sh.iperm, rows, sh.Np, sh.Q, sh.Qp);
+    return cudaGetLastError();
+  }
+  if constexpr (!ST::dev) {
+    const auto plan = decode_plan<ST>(sh);
+    const Split& s = plan.split;
+    plan.kernel<<<s.grid, kThreads, s.smem, st>>>(in, out, sh.iperm, sh.K, sh.Np, sh.Q, sh.Qp, s.rows, int(s.tables));
+  }
   return cudaGetLastError();
 }
 
@@ -506,10 +575,12 @@ cudaError_t moments_as(const Shape& sh, const void* in, const float* scale, cons
   int G = 1;
   while (G < 32 && G < chunks) G *= 2;
   const int64_t nodes = sh.K * sh.Np;
-  const int64_t per_block = 4 * (kThreads / G);
+  const bool few = few_nodes(sh, nodes, G, sizeof(typename ST::R));
+  const int64_t per_block = (few ? 1 : 4) * (kThreads / G);
   const int grid = int(std::max<int64_t>(1, std::min<int64_t>((nodes + per_block - 1) / per_block, int64_t(sh.nsm) * 32)));
-  moments_kernel<ST><<<grid, kThreads, 0, st>>>(in, scale, static_cast<const typename ST::R*>(vel), nodes, sh.Np,
-                                                sh.Qp, G, rho, ux, uy);
+  auto kernel = few ? &moments_kernel<ST, 1> : &moments_kernel<ST, 4>;
+  kernel<<<grid, kThreads, 0, st>>>(in, scale, static_cast<const typename ST::R*>(vel), nodes, sh.Np, sh.Qp, G, rho, ux,
+                                    uy);
   return cudaGetLastError();
 }
 
@@ -524,6 +595,19 @@ cudaError_t encode_any(const Shape& sh, const TIn* in, void* out, float* scale, 
 }
 
 }  // namespace
+
+void weight_tables(const double* w, const int32_t* iperm, int Q, DevRow* row, DevIndex* index, double* wide) {
+  for (int c = 0; c < Q; ++c) {
+    const double v = w[iperm[c]], iw = v > 0 ? 1.0 / v : 0.0;
+    const float wh = float(v), wl = float(v - double(wh)), wll = float(v - double(wh) - double(wl));
+    const float ih = v < kTinyWeight ? std::nanf("") : float(iw);
+    // the rest of 1/w from the residual 1 - w ih, formed exactly by an FMA
+    row[c] = DevRow{wh, wl, ih, float(std::fma(-v, double(ih), 1.0) * iw)};
+    index[c] = DevIndex{wll, iperm[c]};
+    wide[2 * c] = v;
+    wide[2 * c + 1] = iw;
+  }
+}
 
 cudaError_t prepare(const Shape& sh) {
   switch (sh.store) {

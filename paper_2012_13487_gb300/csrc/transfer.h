@@ -7,6 +7,23 @@
 namespace fedbm {
 namespace transfer {
 
+// A weight in three FP32 pieces wh + wl + wll and its inverse in two, ih + il, in canonical
+// order, with the velocity's internal index (see encode in transfer.cu).
+struct alignas(16) DevRow {
+  float wh, wl, ih, il;
+};
+struct alignas(8) DevIndex {
+  float wll;
+  int32_t at;
+};
+struct Weights {
+  const DevRow* row = nullptr;      // [Q], device memory
+  const DevIndex* index = nullptr;  // [Q]
+  const double* wide = nullptr;     // [Q][2] w, 1/w
+};
+// The tables of Q canonical velocities from the weights in the internal order (host).
+void weight_tables(const double* w, const int32_t* iperm, int Q, DevRow* row, DevIndex* index, double* wide);
+
 // One case's slice of its group.
 struct Shape {
   int store = 0;              // StoreKind
@@ -14,6 +31,7 @@ struct Shape {
   int Np = 0, Q = 0, Qp = 0;
   const double* vel64 = nullptr;   // [3][Qp] e_x, e_y, w in the internal order
   const int32_t* iperm = nullptr;  // [Q] internal index of canonical velocity c
+  Weights weights;                 // deviation forms
   int nsm = 0;                     // SMs of the device and shared memory of one, bytes
   int smem_sm = 0;
 };
